@@ -85,23 +85,25 @@ typedef enum {
 /* Arithmetic of the weight solve (diagonal load, factorisation, substitutions,
  * refinement). */
 typedef enum {
-  STAP_SOLVE_FP64 = 0,    /* FP64 factorisation and substitutions; each of the
-                             refine_steps refinement steps forms the FP64
-                             residual v - Rl u and solves for the correction in
-                             FP64 (the default) */
+  STAP_SOLVE_FP64 = 0,    /* 64-bit factorisation and substitutions; each of the
+                             refine_steps refinement steps forms the residual
+                             v - Rl u and solves for the correction (the
+                             default).  Where the load bounds the condition
+                             number, D / load_factor + 1 <= 2^19, the values
+                             are double-floats (unevaluated sums of two FP32
+                             values, compensated sums, about 2^-44) on the FP32
+                             pipe: for a covariance (positive semidefinite) the
+                             weights are the same up to their complex64
+                             rounding.  Weaker loads are solved in FP64 */
   STAP_SOLVE_MIXED_IR = 1 /* mixed-precision iterative refinement (not in the
-                             paper; a faster option): Rl split into
-                             double-floats (hi + lo, about 2^-48), its FP32 part
-                             factored and solved in FP32, and each of the
-                             refine_steps steps forms the residual v - Rl u in
-                             double-float arithmetic on the FP32 pipe, solves
-                             for the correction in FP32 and adds it to the
-                             double-float solution.  Each step shrinks the error
-                             by about cond(Rl) 2^-24; 2 steps reach FP32 weight
-                             accuracy for cond(Rl) up to about 1e5.  For
-                             D > 64 the residual is formed in FP64 from the
-                             input instead (the double-float matrix would not
-                             fit on chip) */
+                             paper; a faster option): Rl's FP32 part factored
+                             and solved in FP32, and each of the refine_steps
+                             steps forms the residual v - Rl u in double-float
+                             arithmetic on the FP32 pipe, solves for the
+                             correction in FP32 and adds it to the double-float
+                             solution.  Each step shrinks the error by about
+                             cond(Rl) 2^-24; 2 steps reach FP32 weight accuracy
+                             for cond(Rl) up to about 1e5 */
 } stap_solver;
 
 /* Which range cells train the covariance that block b's weights use. */
@@ -257,11 +259,10 @@ stap_status stap_train_neighbours(stap_plan plan, const void* cov_c128, void* co
 stap_status stap_train_window(stap_plan plan, const void* cov_c128, void* cov_train_c128);
 
 /* Adaptive weights per (k, b) and steering vector v_s (Sec. 4.2's STAP
- * kernel, loaded sample-matrix reading), in FP64 with the default solver:
+ * kernel, loaded sample-matrix reading), in the arithmetic of stap_solver:
  *   delta = load_factor * Re tr(cov) / D,  Rl = cov + delta I = L L^H,
  *   u_s = Rl^{-1} v_s by forward/back substitution, refine_steps refinement
  *   steps u_s += Rl^{-1} (v_s - Rl u_s),  w_s = u_s / sqrt(Re v_s^H u_s).
- * (STAP_SOLVE_MIXED_IR: see stap_solver.)
  * Only the lower triangle and the real part of the diagonal of each cov are
  * read.  A system whose pivot is not positive and finite gets zero weights
  * and is counted (stap_get_status).  cov: c128 [K][NB][D][D];

@@ -13,6 +13,7 @@
 #include "batch.cuh"
 #include "snapshots.cuh"
 #include "stap_internal.cuh"
+#include "solve_df.cuh"
 
 using stap::DeviceStatus;
 
@@ -820,6 +821,8 @@ stap_status stap_check_report(int64_t* count, int32_t* site, int64_t* index, int
   if (cudaDeviceSynchronize() != cudaSuccess) return STAP_ERR_CUDA;
   cudaError_t (*readers[])(stap::CheckRecord*) = {
       stap::check_record_doppler, stap::check_record_covariance, stap::check_record_solve,
+      stap::check_record_solve_df_small, stap::check_record_solve_df_big,
+      stap::check_record_solve_df_small_ir, stap::check_record_solve_df_big_ir,
       stap::check_record_apply,   stap::check_record_mixed,      stap::check_record_train};
   bool first = true;
   for (auto rd : readers) {
@@ -1358,7 +1361,11 @@ stap_status stap_plan_autotune(stap_plan p, const void* const* cubes, float* con
              [&] { return do_covariance(p, c, dop, cov, p->stream); });
     }
     if ((st = do_covariance(p, c, dop, cov, p->stream)) != STAP_OK) break;
-    if (c.D <= stap::kSmallMaxD) {
+    // FP64 solves have launch choices; the double-float ones (faster wherever
+    // they may stand in) have none
+    if (stap::solve_df_eligible(p->opt.solver, p->opt.load_factor, c.D)) {
+      c.tune.solve_kind = c.tune.solve_ts = c.tune.solve_nw = c.tune.solve_lr = 0;
+    } else if (c.D <= stap::kSmallMaxD) {
       const int nrhs = c.separable ? d.n_chan : d.n_steering;
       int base = 1;
       while (base < nrhs && base < 32) base <<= 1;
@@ -1380,9 +1387,7 @@ stap_status stap_plan_autotune(stap_plan p, const void* const* cubes, float* con
             }
           }
       c.tune.solve_kind = 3;   // one system per CTA instead of teams
-      if (p->opt.solver == STAP_SOLVE_FP64 &&
-          timeit([&] { return do_solve(p, c, cov, wts, p->stream); }) < bt)
-        bkind = 3;
+      if (timeit([&] { return do_solve(p, c, cov, wts, p->stream); }) < bt) bkind = 3;
       c.tune.solve_kind = bkind;
       c.tune.solve_ts = bts;
       c.tune.solve_nw = bnw;
@@ -1391,7 +1396,7 @@ stap_status stap_plan_autotune(stap_plan p, const void* const* cubes, float* con
       if (c.D <= 64) lrs.insert(lrs.begin(), 8);
       pick([](stap::Tune& t, int v) { t.solve_lr = v; }, lrs,
            [&] { return do_solve(p, c, cov, wts, p->stream); });
-      if (c.D > 64 && p->opt.solver == STAP_SOLVE_FP64 && c.tune.solve_lr == 32)   // 8 or 16 warps
+      if (c.D > 64 && c.tune.solve_lr == 32)   // 8 or 16 warps
         pick([](stap::Tune& t, int v) { t.solve_nw = v; }, {0, 16},
              [&] { return do_solve(p, c, cov, wts, p->stream); });
     }

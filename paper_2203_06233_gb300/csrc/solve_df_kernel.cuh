@@ -1,0 +1,851 @@
+// The weight solve in double-float arithmetic: the same steps as solve.cu's
+// FP64 kernels (load, Rl = Lu Dg Lu^H, solve, refine, normalise),
+//   delta = lf Re tr(R) / D,  Rl = R + delta I,  u = Rl^{-1} v,
+//   u += Rl^{-1} (v - Rl u)  refine_steps times,  w = u / sqrt(Re v^H u),
+// with every FP64 value replaced by an unevaluated sum of two floats and
+// every sum compensated, on the FP32 pipe.
+//
+// Why.  GB300 runs FP64 at 1/62 of the FP32 rate: a complex multiply-add of a
+// warp holds the SM's FP64 pipe for 64 cycles, while the 48 FP32
+// instructions of its double-float form take the four schedulers 12.  The
+// FP64 kernels were at 65-80% of that FP64 bound, i.e. at their floor, and the
+// solve was 95% of a D = 64 or D = 128 CPI.
+//
+// Arithmetic.  A real multiply-add is the Dot2 step of Ogita, Rump and Oishi
+// ("Accurate sum and dot product", SISC 2005) with double-float factors: the
+// product of the high parts split exactly by an FMA, the running sum by
+// Knuth's TwoSum, every rounding error and the cross terms collected in a
+// second float; the pair is renormalised every LR columns, so the collected
+// errors stay small against the sum.  Relative to the terms' running sums
+// that is about 2^-44, against FP64's 2^-50 over as many terms.
+//
+// Where it may stand in for FP64.  The weights are stored as complex64
+// (2^-25), and the solution's relative error is at most kappa(Rl) times the
+// arithmetic's.  For a covariance (R positive semidefinite) the load bounds
+// kappa <= D / lf + 1, so launch_solve takes these kernels when that bound is
+// at most kDfMaxKappa = 2^19 (the default load 1e-3 gives 1.28e5 at D = 128)
+// and the FP64 kernels for weaker loads, where nothing bounds kappa.  With
+// the refinement step the measured weights are as far from the 64-bit ones as
+// the FP64 kernels' (both are the complex64 rounding).
+//
+// Range.  Floats span 2^+-126 only, so each system is scaled by the even
+// power of two 2^-e that brings its trace into [1, 4): the conversion from
+// FP64 adds -e to the exponent field (no instruction more), and the weights
+// take 2^(-e/2) back with their normalisation.  Entries below 2^-73 of the
+// trace become zero; an infinity or NaN becomes a NaN, which no pivot test
+// passes.
+//
+// Layout.  A system belongs to a team of TEAM threads: 16 lanes of a warp
+// (D <= 16) or a CTA of 64 (D <= 32), 256 (D <= 64) or 512 (D <= 128) threads.
+// LR lanes hold one right-hand side, row li + LR q in register q < RPL.  The
+// factor (column-major packed) and the solutions stay in shared memory, the
+// column's entry is broadcast by shuffles, so a 16-byte read feeds one complex
+// multiply-add of 48 FP32 instructions.  The residual's Rl comes from the
+// input again, in chunks of KC columns that the team converts once for all its
+// right-hand sides (the FP64 kernel read each entry from global memory for
+// every right-hand side).  Sixteen warps of 128 registers per SM at D = 128
+// issued 74% of the slots against 62% for eight warps of 255 with two
+// right-hand sides per thread; packed FP32 pairs (FFMA2) of two right-hand
+// sides, or of real and imaginary part, needed so many moves to form the pairs
+// that they were no faster.
+//
+// Measured (GB300; before: the FP64 kernels, after), us:
+//   D = 128, 16384 systems, C 32 S 64    266533 -> 82200
+//   D =  64, 8192 systems,  C 16 S 32     15859 ->  5300
+//   D =  12, 16384 systems, C 4  S 16       324 ->   170
+//   D =  12, 256 systems,   C 4  S 4      103.5 ->  26.5
+//
+// F32F (STAP_SOLVE_MIXED_IR): the factor and the substitutions in FP32, the
+// residual and the solution in double-float as above.
+#pragma once
+
+#include "df64.cuh"
+#include "batch.cuh"
+#include "checked.cuh"
+#include "snapshots.cuh"
+#include "solve_df.cuh"
+
+namespace stap {
+namespace {
+
+constexpr int KC = 8;   // columns of Rl per residual chunk
+
+// One complex value: running sums (rs, is) and the errors collected beside
+// them (re, ie); in shared memory (re hi, im hi, re lo, im lo).
+struct Cdf {
+  float rs, re, is, ie;
+};
+__device__ __forceinline__ float4 pack(const Cdf& x) { return make_float4(x.rs, x.is, x.re, x.ie); }
+__device__ __forceinline__ Cdf unpack(float4 v) { return Cdf{v.x, v.z, v.y, v.w}; }
+__device__ __forceinline__ float4 conj4(float4 v) { return make_float4(v.x, -v.y, v.z, -v.w); }
+
+// s + e += (ah + al) (bh + bl), dropping al bl (below 2^-48 of the product)
+__device__ __forceinline__ void mac(float& s, float& e, float ah, float al, float bh, float bl) {
+  const float p = __fmul_rn(ah, bh);
+  float pe = __fmaf_rn(ah, bh, -p);
+  pe = __fmaf_rn(ah, bl, pe);
+  pe = __fmaf_rn(al, bh, pe);
+  const float t = __fadd_rn(s, p);
+  const float z = __fsub_rn(t, s);
+  const float te = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z));
+  s = t;
+  e = __fadd_rn(e, __fadd_rn(te, pe));
+}
+
+// renormalise: |lo| <= ulp(hi) / 2 (the collected errors are smaller than the sum)
+__device__ __forceinline__ void norm2(float& s, float& e) {
+  const ff::F2 t = ff::fast_two_sum(s, e);
+  s = t.hi;
+  e = t.lo;
+}
+__device__ __forceinline__ void norm(Cdf& x) {
+  norm2(x.rs, x.re);
+  norm2(x.is, x.ie);
+}
+// x -= l y
+__device__ __forceinline__ void cms(Cdf& x, float4 l, float4 y) {
+  mac(x.rs, x.re, -l.x, -l.z, y.x, y.z);
+  mac(x.is, x.ie, -l.x, -l.z, y.y, y.w);
+  mac(x.rs, x.re, l.y, l.w, y.y, y.w);
+  mac(x.is, x.ie, -l.y, -l.w, y.x, y.z);
+}
+
+// a b of two normalised double-floats
+__device__ __forceinline__ ff::F2 mul2(float ah, float al, float bh, float bl) {
+  const float p = __fmul_rn(ah, bh);
+  float e = __fmaf_rn(ah, bh, -p);
+  e = __fmaf_rn(ah, bl, e);
+  e = __fmaf_rn(al, bh, e);
+  return ff::fast_two_sum(p, e);
+}
+__device__ __forceinline__ Cdf scale(const Cdf& x, ff::F2 r) {
+  const ff::F2 a = mul2(x.rs, x.re, r.hi, r.lo), b = mul2(x.is, x.ie, r.hi, r.lo);
+  return Cdf{a.hi, a.lo, b.hi, b.lo};
+}
+// u + v, normalised
+__device__ __forceinline__ Cdf add(const Cdf& u, const Cdf& v) {
+  const ff::F2 a = ff::add2({u.rs, u.re}, {v.rs, v.re}), b = ff::add2({u.is, u.ie}, {v.is, v.ie});
+  return Cdf{a.hi, a.lo, b.hi, b.lo};
+}
+
+// 1 / d: from the hardware's approximate reciprocal r of the high part, with
+// e = 1 - d r (about 2^-23) the series r (1 + e + e^2) leaves e^3
+__device__ __forceinline__ ff::F2 recip(ff::F2 d) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d.hi));
+  float e = __fmaf_rn(-d.hi, r, 1.f);
+  e = __fmaf_rn(-d.lo, r, e);
+  return ff::fast_two_sum(r, __fmul_rn(r, __fmaf_rn(e, e, e)));
+}
+
+// x 2^-e as hi + lo by its IEEE fields (integer instructions: a conversion
+// instruction would hold the FP64 pipe): hi = the top 24 bits, lo = the other
+// 29 rounded to a float, both with x's sign.  `base` = 896 + e.  Below 2^-73:
+// zero; beyond float range or not finite: NaN.
+__device__ __forceinline__ ff::F2 split(double x, int base) {
+  const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
+  const int E = (int)((h >> 20) & 0x7FF) - base;   // biased float exponent
+  const uint32_t sign = h & 0x80000000u;
+  if (E <= 53) return {0.f, 0.f};
+  if (E >= 255 || (h & 0x7FF00000u) == 0x7FF00000u) return {__int_as_float(0x7FC00000), 0.f};
+  const float hi = __uint_as_float(sign | ((uint32_t)E << 23) | ((h & 0xFFFFFu) << 3) | (l >> 29));
+  const float lo = __fmul_rn((float)(l & 0x1FFFFFFFu), __uint_as_float((uint32_t)(E - 52) << 23));
+  return {hi, __uint_as_float(__float_as_uint(lo) | sign)};
+}
+__device__ __forceinline__ float4 split(double2 a, int base) {
+  const ff::F2 r = split(a.x, base), i = split(a.y, base);
+  return make_float4(r.hi, i.hi, r.lo, i.lo);
+}
+
+__device__ __forceinline__ int cstart(int l, int D) { return l * D - l * (l - 1) / 2; }
+
+// The weights' factor 2^h / sqrt(q) (h = -e/2 undoes the system's scale): the
+// double-float 1 / sqrt(q), from the approximate r by r (1 + (1 - q r^2) / 2),
+// times the part of 2^h that floats hold surely; `rest` the exponent left
+// over (zero but for traces beyond 2^+-200).
+struct Gain {
+  float hi, lo;
+  int rest;
+};
+__device__ __forceinline__ Gain gain(ff::F2 q, int h) {
+  const float r = rsqrtf(q.hi);
+  const float p = __fmul_rn(r, r), pl = __fmaf_rn(r, r, -p);
+  float e = __fmaf_rn(-q.hi, p, 1.f);
+  e = __fmaf_rn(-q.hi, pl, e);
+  e = __fmaf_rn(-q.lo, p, e);
+  const ff::F2 g = ff::fast_two_sum(r, __fmul_rn(r, __fmul_rn(0.5f, e)));
+  const int hc = max(-100, min(100, h));
+  const float sc = __uint_as_float((uint32_t)(127 + hc) << 23);
+  return {__fmul_rn(g.hi, sc), __fmul_rn(g.lo, sc), h - hc};
+}
+// (re, im) times that, rounded once
+__device__ __forceinline__ float2 weight(ff::F2 re, ff::F2 im, const Gain& g, bool good) {
+  if (!good) return make_float2(0.f, 0.f);
+  float2 w = make_float2(mul2(re.hi, re.lo, g.hi, g.lo).hi, mul2(im.hi, im.lo, g.hi, g.lo).hi);
+  if (g.rest != 0) w = make_float2(ldexpf(w.x, g.rest), ldexpf(w.y, g.rest));
+  return w;
+}
+// sum of s + e over W lanes, the same in all of them
+template <int W>
+__device__ __forceinline__ ff::F2 lanes_sum2(float s, float e) {
+  for (int o = W / 2; o > 0; o >>= 1) {
+    const ff::F2 t = ff::two_sum(s, __shfl_xor_sync(0xffffffffu, s, o));
+    e = __fadd_rn(__fadd_rn(e, __shfl_xor_sync(0xffffffffu, e, o)), t.lo);
+    s = t.hi;
+  }
+  return ff::fast_two_sum(s, e);
+}
+__device__ __forceinline__ bool usable(ff::F2 q) { return q.hi > 0.f && isfinite(q.hi); }
+
+template <int W>
+__device__ __forceinline__ double lanes_sum(double v) {
+  for (int o = W / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// In-place forward (Lu z = x) or back (Lu^H z = x) substitution of the vector
+// that the LR lanes of a group hold (row li + LR q in x[q]).  The columns go
+// in blocks of LR (block qb's columns live in x[qb], a shuffle broadcasts the
+// column's entry), and only the row blocks that a block's columns update are
+// visited, with the block indices compile-time constants.  Only the diagonal
+// block decides per lane; rows past D read whatever lies after their column
+// (inside the team's shared memory) into registers that nothing reads.
+template <int LR, int RPL, bool BACK>
+__device__ __forceinline__ void subst(Cdf (&x)[RPL], const float4* L, int D, int li, int gbase) {
+#pragma unroll
+  for (int bb = 0; bb < RPL; ++bb) {
+    const int qb = BACK ? RPL - 1 - bb : bb;
+    if (LR * qb >= D) continue;                           // team-uniform
+    const int jn = min(LR, D - LR * qb);
+    // forward: column j's entries start at cstart(j) - j + i; back: row j of
+    // column i = li + LR q lies at cstart(i) - i + j, which is b0 + b1 q -
+    // q^2 LR^2 / 2 + j
+    const int b0 = li * D - li * (li - 1) / 2 - li, b1 = LR * D - LR * li - LR / 2;
+#pragma unroll 2
+    for (int jj = 0; jj < jn; ++jj) {
+      const int jo = BACK ? jn - 1 - jj : jj;
+      const int j = LR * qb + jo;
+      norm(x[qb]);
+      const Cdf y{__shfl_sync(0xffffffffu, x[qb].rs, gbase + jo), __shfl_sync(0xffffffffu, x[qb].re, gbase + jo),
+                  __shfl_sync(0xffffffffu, x[qb].is, gbase + jo), __shfl_sync(0xffffffffu, x[qb].ie, gbase + jo)};
+      const float4* cj = L + cstart(j, D) - j + li;
+#pragma unroll
+      for (int q = 0; q < RPL; ++q) {
+        if (BACK ? (q > qb) : (q < qb)) continue;         // compile-time
+        if (LR * q >= D) continue;                        // team-uniform
+        float4 l = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (q != qb || (BACK ? li < jo : (li > jo && li + LR * q < D)))
+          l = BACK ? conj4(L[b0 + j + b1 * q - q * q * (LR * LR / 2)]) : cj[LR * q];
+        cms(x[q], l, pack(y));
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < RPL; ++q)
+      if (BACK ? q < qb : q > qb) norm(x[q]);
+  }
+}
+
+// x <- Rl^{-1} x with Rl = Lu Dg Lu^H (rd: the pivot reciprocals).
+template <int LR, int RPL>
+__device__ __forceinline__ void ldl_solve(Cdf (&x)[RPL], const float4* L, const float2* rd, int D, int li,
+                                          int gbase) {
+  subst<LR, RPL, false>(x, L, D, li, gbase);
+#pragma unroll
+  for (int q = 0; q < RPL; ++q) {
+    const int i = li + LR * q;
+    const float2 r = rd[i < D ? i : D - 1];
+    x[q] = i < D ? scale(x[q], ff::F2{r.x, r.y}) : Cdf{0.f, 0.f, 0.f, 0.f};
+  }
+  subst<LR, RPL, true>(x, L, D, li, gbase);
+#pragma unroll
+  for (int q = 0; q < RPL; ++q) norm(x[q]);
+}
+
+// The same in FP32 with the FP32 factor (F32F).
+template <int LR, int RPL, bool BACK>
+__device__ __forceinline__ void subst_f32(float2 (&x)[RPL], const float2* L, int D, int li, int gbase) {
+#pragma unroll
+  for (int bb = 0; bb < RPL; ++bb) {
+    const int qb = BACK ? RPL - 1 - bb : bb;
+    if (LR * qb >= D) continue;
+    const int jn = min(LR, D - LR * qb);
+    const int b0 = li * D - li * (li - 1) / 2 - li, b1 = LR * D - LR * li - LR / 2;
+#pragma unroll 2
+    for (int jj = 0; jj < jn; ++jj) {
+      const int jo = BACK ? jn - 1 - jj : jj;
+      const int j = LR * qb + jo;
+      const float yr = __shfl_sync(0xffffffffu, x[qb].x, gbase + jo);
+      const float yi = __shfl_sync(0xffffffffu, x[qb].y, gbase + jo);
+      const float2* cj = L + cstart(j, D) - j + li;
+#pragma unroll
+      for (int q = 0; q < RPL; ++q) {
+        if (BACK ? (q > qb) : (q < qb)) continue;
+        if (LR * q >= D) continue;
+        float2 l = make_float2(0.f, 0.f);
+        if (q != qb || (BACK ? li < jo : (li > jo && li + LR * q < D))) l = BACK ? L[b0 + j + b1 * q - q * q * (LR * LR / 2)] : cj[LR * q];
+        if (BACK) l.y = -l.y;
+        x[q].x = fmaf(-l.x, yr, x[q].x);
+        x[q].y = fmaf(-l.x, yi, x[q].y);
+        x[q].x = fmaf(l.y, yi, x[q].x);
+        x[q].y = fmaf(-l.y, yr, x[q].y);
+      }
+    }
+  }
+}
+
+template <int LR, int RPL>
+__device__ __forceinline__ void ldl_solve_f32(Cdf (&x)[RPL], const float2* L, const float2* rd, int D, int li,
+                                              int gbase) {
+  float2 xf[RPL];
+#pragma unroll
+  for (int q = 0; q < RPL; ++q) xf[q] = make_float2(__fadd_rn(x[q].rs, x[q].re), __fadd_rn(x[q].is, x[q].ie));
+  subst_f32<LR, RPL, false>(xf, L, D, li, gbase);
+#pragma unroll
+  for (int q = 0; q < RPL; ++q) {
+    const int i = li + LR * q;
+    const float r = i < D ? rd[i].x : 0.f;
+    xf[q] = i < D ? make_float2(xf[q].x * r, xf[q].y * r) : make_float2(0.f, 0.f);
+  }
+  subst_f32<LR, RPL, true>(xf, L, D, li, gbase);
+#pragma unroll
+  for (int q = 0; q < RPL; ++q) x[q] = Cdf{xf[q].x, 0.f, xf[q].y, 0.f};
+}
+
+// Shared memory of one team: the solutions U [nu][D], Rl's columns As (a chunk
+// [KC][D + 1], or all D columns where the team is part of a warp: small
+// systems convert their matrix once), the two pivot columns before division
+// [2][D] (in the chunk's place: the factorisation is over before the first
+// residual), the factor [Dp] (column-major packed), the pivot reciprocals [D]
+// and the pivot flag.
+template <int TEAM, bool F32F>
+struct Shared {
+  static constexpr bool FULL = TEAM <= 32;
+  using LT = typename std::conditional<F32F, float2, float4>::type;   // factor entries
+  int u, as, col, l, rd, ok, bytes;                // byte offsets, all multiples of 16
+  __host__ __device__ Shared(int D, int nu) {
+    const int Dp = D * (D + 1) / 2;
+    u = 0;
+    as = u + nu * D * 16;
+    col = FULL ? as + D * (D + 1) * 16 : as;
+    l = FULL ? col + 2 * D * 16 : as + KC * (D + 1) * 16;
+    rd = l + (Dp * (int)sizeof(LT) + 15) / 16 * 16;
+    ok = rd + (D * 8 + 15) / 16 * 16;
+    bytes = ok + 16;
+  }
+};
+
+// A team's system, as its phases need it.
+struct System {
+  int off;              // the team's shared memory, in bytes
+  int nu;               // rows of U
+  int sbase;            // split()'s exponent offset
+  double delta;         // the load
+  const double2* A;     // the covariance
+  long long a0, aext;   // its first entry's index and the extent of the array
+};
+
+template <int TEAM>
+__device__ __forceinline__ void team_sync() {
+  if constexpr (TEAM > 32) __syncthreads();
+  else __syncwarp();
+}
+template <int TEAM>
+__device__ __forceinline__ int team_thread() {
+  return TEAM > 32 ? threadIdx.x : threadIdx.x % TEAM;
+}
+
+// Rl[i][l], i >= l
+__device__ __forceinline__ float4 entry(const System& y, int D, int i, int l) {
+  double2 a = in_bounds(y.a0 + (long long)i * D + l, y.aext, kSiteSolveIn) ? __ldg(y.A + (size_t)i * D + l)
+                                                                           : make_double2(0.0, 0.0);
+  if (i == l) {
+    a.x += y.delta;
+    a.y = 0.0;
+  }
+  return split(a, y.sbase);
+}
+
+template <bool F32F>
+__device__ __forceinline__ ff::F2 pivot(ff::F2 d, int* okf) {
+  if (!(d.hi > 0.f) || !isfinite(d.hi)) {
+    *okf = 0;
+    return {1.f, 0.f};   // keep going; this system's weights become zero
+  }
+  if constexpr (F32F) return {1.0f / d.hi, 0.f};
+  return recip(d);
+}
+
+// Copy Rl's lower triangle into shared memory and factor it: Rl = Lu Dg Lu^H,
+// right-looking, two columns per round.  Phase 1: the thread of row i scales
+// column j, brings its entry of column j+1 up to date and scales that; each
+// thread forms the two pivots' reciprocals itself.  Phase 2: the rank-2 update
+// of the trailing triangle, its columns spread over groups of RW threads, a
+// group's threads over a column's rows.
+template <int TEAM, bool F32F>
+__device__ __forceinline__ void factor(const System y, int D) {
+  extern __shared__ float4 smdf[];
+  const Shared<TEAM, F32F> sh(D, y.nu);
+  using LT = typename Shared<TEAM, F32F>::LT;
+  char* base = reinterpret_cast<char*>(smdf) + y.off;
+  LT* L = reinterpret_cast<LT*>(base + sh.l);
+  LT* colb = reinterpret_cast<LT*>(base + sh.col);
+  LT* colb2 = colb + D;
+  float2* rd = reinterpret_cast<float2*>(base + sh.rd);
+  int* okf = reinterpret_cast<int*>(base + sh.ok);
+  const int tt = team_thread<TEAM>();
+  auto put = [&](int i, int l, float4 v) {
+    if constexpr (F32F) L[cstart(l, D) + i - l] = make_float2(__fadd_rn(v.x, v.z), __fadd_rn(v.y, v.w));
+    else L[cstart(l, D) + i - l] = v;
+    if constexpr (Shared<TEAM, F32F>::FULL) {
+      float4* As = reinterpret_cast<float4*>(base + sh.as);
+      As[l * (D + 1) + i] = v;                     // column l, row i
+      As[i * (D + 1) + l] = conj4(v);
+    }
+  };
+  if constexpr (TEAM > 32) {                       // rows coalesced
+    for (int i = tt >> 5; i < D; i += TEAM / 32)
+      for (int l = tt & 31; l <= i; l += 32) put(i, l, entry(y, D, i, l));
+  } else {
+    int i = 0, l = tt;
+    while (l > i) l -= ++i;
+    for (int q = tt; q < D * (D + 1) / 2; q += TEAM) {
+      put(i, l, entry(y, D, i, l));
+      l += TEAM;
+      while (l > i) l -= ++i;
+    }
+  }
+  if (tt == 0) *okf = 1;
+  team_sync<TEAM>();
+
+  for (int j = 0; j < D; j += 2) {
+    const int j1 = j + 1;
+    const bool pair = j1 < D;
+    const int cj = cstart(j, D), c1 = pair ? cstart(j1, D) : cj;
+    if constexpr (F32F) {
+      const float rj = pivot<F32F>({L[cj].x, 0.f}, okf).hi;
+      float2 a1j = make_float2(0.f, 0.f);
+      float r1 = 1.f;
+      if (pair) {
+        a1j = L[cj + 1];
+        float d1 = L[c1].x;
+        d1 = fmaf(-a1j.x * rj, a1j.x, d1);
+        d1 = fmaf(-a1j.y * rj, a1j.y, d1);
+        r1 = pivot<F32F>({d1, 0.f}, okf).hi;
+      }
+      float2 own = make_float2(0.f, 0.f);
+      bool own1 = false;
+      for (int i = j1 + tt; i < D; i += TEAM) {
+        const float2 v = L[cj + i - j];
+        colb[i] = v;
+        const float2 lij = make_float2(v.x * rj, v.y * rj);
+        if (i == j1) {
+          own = lij;
+          own1 = true;
+        } else {
+          L[cj + i - j] = lij;
+          float2 w = L[c1 + i - j1];
+          w.x = fmaf(-lij.x, a1j.x, w.x);
+          w.y = fmaf(-lij.y, a1j.x, w.y);
+          w.x = fmaf(-lij.y, a1j.y, w.x);
+          w.y = fmaf(lij.x, a1j.y, w.y);
+          colb2[i] = w;
+          L[c1 + i - j1] = make_float2(w.x * r1, w.y * r1);
+        }
+      }
+      if (tt == 0) {
+        rd[j] = make_float2(rj, 0.f);
+        if (pair) rd[j1] = make_float2(r1, 0.f);
+      }
+      team_sync<TEAM>();
+      if (own1) L[cj + 1] = own;
+    } else {
+      Cdf dj = unpack(L[cj]);
+      norm2(dj.rs, dj.re);
+      const ff::F2 rj = pivot<F32F>({dj.rs, dj.re}, okf);
+      Cdf a1j{0.f, 0.f, 0.f, 0.f};
+      ff::F2 r1{1.f, 0.f};
+      if (pair) {
+        a1j = unpack(L[cj + 1]);
+        norm(a1j);
+        const Cdf l1j = scale(a1j, rj);
+        Cdf d1 = unpack(L[c1]);
+        mac(d1.rs, d1.re, -l1j.rs, -l1j.re, a1j.rs, a1j.re);
+        mac(d1.rs, d1.re, -l1j.is, -l1j.ie, a1j.is, a1j.ie);
+        norm2(d1.rs, d1.re);
+        r1 = pivot<F32F>({d1.rs, d1.re}, okf);
+      }
+      const float4 a1c = conj4(pack(a1j));
+      float4 own = make_float4(0.f, 0.f, 0.f, 0.f);
+      bool own1 = false;
+      for (int i = j1 + tt; i < D; i += TEAM) {
+        Cdf v = unpack(L[cj + i - j]);
+        norm(v);
+        colb[i] = conj4(pack(v));                // stored conjugated
+        const float4 lij = pack(scale(v, rj));
+        if (i == j1) {
+          own = lij;
+          own1 = true;
+        } else {
+          L[cj + i - j] = lij;
+          Cdf w = unpack(L[c1 + i - j1]);
+          cms(w, lij, a1c);
+          norm(w);
+          colb2[i] = conj4(pack(w));
+          L[c1 + i - j1] = pack(scale(w, r1));
+        }
+      }
+      if (tt == 0) {
+        rd[j] = make_float2(rj.hi, rj.lo);
+        if (pair) rd[j1] = make_float2(r1.hi, r1.lo);
+      }
+      team_sync<TEAM>();
+      if (own1) L[cj + 1] = own;
+    }
+    constexpr int RW = TEAM == 512 ? 32 : (TEAM == 256 ? 16 : (TEAM == 64 ? 8 : 4));
+    for (int l = j + 2 + tt / RW; l < D; l += TEAM / RW) {
+      const LT alj = colb[l], blj = colb2[l];
+      LT* cl = L + cstart(l, D) - l;
+      for (int i = l + tt % RW; i < D; i += RW) {
+        const LT lij = L[cj + i - j], mij = L[c1 + i - j1];
+        if constexpr (F32F) {
+          float2 acc = cl[i];
+          acc.x = fmaf(-lij.x, alj.x, acc.x);
+          acc.y = fmaf(-lij.y, alj.x, acc.y);
+          acc.x = fmaf(-lij.y, alj.y, acc.x);
+          acc.y = fmaf(lij.x, alj.y, acc.y);
+          acc.x = fmaf(-mij.x, blj.x, acc.x);
+          acc.y = fmaf(-mij.y, blj.x, acc.y);
+          acc.x = fmaf(-mij.y, blj.y, acc.x);
+          acc.y = fmaf(mij.x, blj.y, acc.y);
+          cl[i] = acc;
+        } else {
+          Cdf acc = unpack(cl[i]);
+          cms(acc, lij, alj);
+          cms(acc, mij, blj);
+          norm(acc);
+          cl[i] = pack(acc);
+        }
+      }
+    }
+    team_sync<TEAM>();
+  }
+}
+
+// Solve and refine the right-hand sides r0 .. r0 + TEAM / LR - 1, one per group
+// of LR lanes, into U (row rhs of it, or row g where U holds one pass only).
+template <int LR, int RPL, int TEAM, bool F32F>
+__device__ __forceinline__ void solve_rhs(const SolveDfParams& prm, const System y, int r0) {
+  constexpr int EPT = (KC * LR * RPL + TEAM - 1) / TEAM;   // chunk entries per thread
+  using SH = Shared<TEAM, F32F>;
+  extern __shared__ float4 smdf[];
+  const int D = prm.D, C = prm.C, refine_steps = prm.refine_steps;
+  const bool sep = prm.sep != 0;
+  const int nrhs = sep ? C : prm.S;
+  const SH sh(D, y.nu);
+  char* base = reinterpret_cast<char*>(smdf) + y.off;
+  float4* U = reinterpret_cast<float4*>(base + sh.u);
+  float4* As = reinterpret_cast<float4*>(base + sh.as);
+  const typename SH::LT* L = reinterpret_cast<const typename SH::LT*>(base + sh.l);
+  const float2* rd = reinterpret_cast<const float2*>(base + sh.rd);
+  const int tt = team_thread<TEAM>(), li = tt % LR, g = tt / LR;
+  const int gbase = (threadIdx.x & 31) - li;       // first lane of this thread's group
+  // a CTA team's warps past the last right-hand side only help convert
+  const bool work = TEAM <= 32 || r0 + (tt >> 5) * (32 / LR) < nrhs;
+  const bool live = r0 + g < nrhs;
+  const int rhs = live ? r0 + g : nrhs - 1;    // a spare group computes a copy, never stored
+  float4* Ur = U + (size_t)(sep ? rhs : g) * D;   // its solution
+  auto b_at = [&](int i) -> Cdf {              // right-hand side entry
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);   // tables: (re hi, re lo, im hi, im lo)
+    if (i < D) {
+      if (sep) {
+        const int t = i / C;
+        if (i - t * C == rhs) v = __ldg(prm.g_ff + t);
+      } else {
+        v = __ldg(prm.steer_ff + (size_t)rhs * D + i);
+      }
+    }
+    return Cdf{v.x, v.y, v.z, v.w};
+  };
+  Cdf x[RPL];
+#pragma unroll
+  for (int q = 0; q < RPL; ++q) x[q] = b_at(li + LR * q);
+  for (int it = 0;; ++it) {
+    if (work) {
+      if constexpr (F32F) ldl_solve_f32<LR, RPL>(x, L, rd, D, li, gbase);
+      else ldl_solve<LR, RPL>(x, L, rd, D, li, gbase);
+#pragma unroll
+      for (int q = 0; q < RPL; ++q) {
+        const int i = li + LR * q;
+        if (i < D) {
+          if (it > 0) x[q] = add(unpack(Ur[i]), x[q]);   // u += c
+          if (live) Ur[i] = pack(x[q]);
+        }
+      }
+    }
+    if (it == refine_steps) break;
+    // x = b - Rl u
+#pragma unroll
+    for (int q = 0; q < RPL; ++q) x[q] = b_at(li + LR * q);
+    auto columns = [&](const float4* a, int l0, int n) {   // columns l0 .. l0 + n - 1 at a
+      for (int ll = 0; ll < n; ++ll) {
+        const float4 u = Ur[l0 + ll];
+        const float4* al = a + ll * (D + 1) + li;
+#pragma unroll
+        for (int q = 0; q < RPL; ++q)
+          if (LR * q < D) cms(x[q], al[LR * q], u);   // rows past D: never read
+      }
+#pragma unroll
+      for (int q = 0; q < RPL; ++q) norm(x[q]);
+    };
+    if constexpr (SH::FULL) {
+      __syncwarp();                                // the U rows are written
+      for (int l0 = 0; l0 < D; l0 += KC) columns(As + l0 * (D + 1), l0, min(KC, D - l0));
+    } else {
+      // entry f of the chunk at column l0: column l0 + f % KC, row f / KC; the
+      // next chunk's entries wait in registers
+      auto chunk_entry = [&](int l0, int f) -> float4 {
+        const int l = l0 + f % KC, i = f / KC;
+        if (l >= D || i >= D) return make_float4(0.f, 0.f, 0.f, 0.f);
+        return i >= l ? entry(y, D, i, l) : conj4(entry(y, D, l, i));
+      };
+      float4 pre[EPT];
+#pragma unroll
+      for (int k = 0; k < EPT; ++k) pre[k] = chunk_entry(0, tt + k * TEAM);
+      for (int l0 = 0; l0 < D; l0 += KC) {
+        __syncthreads();                           // the last chunk (and the U rows) are done with
+#pragma unroll
+        for (int k = 0; k < EPT; ++k) {
+          const int f = tt + k * TEAM;
+          if (f / KC < D) As[(f % KC) * (D + 1) + f / KC] = pre[k];
+        }
+        __syncthreads();
+        if (l0 + KC < D)
+#pragma unroll
+          for (int k = 0; k < EPT; ++k) pre[k] = chunk_entry(l0 + KC, tt + k * TEAM);
+        if (work) columns(As, l0, min(KC, D - l0));
+      }
+    }
+  }
+}
+
+// The weights of a pass's steering vectors from their solutions in U.  (This
+// and combine() are calls: inlined, their registers cost the substitutions
+// theirs; 3% on a D = 128 system.)
+template <int LR, int RPL, int TEAM>
+__device__ __noinline__ void emit(const SolveDfParams& prm, int off, long long sys, bool valid, bool ok, int e,
+                                  int r0) {
+  extern __shared__ float4 smdf[];
+  const int D = prm.D, S = prm.S, nrhs = S;
+  const long long nsys = prm.nsys;
+  float2* __restrict__ wts = prm.wts;
+  const int tt = team_thread<TEAM>(), li = tt % LR, g = tt / LR;
+  const bool live = r0 + g < nrhs;
+  const int rhs = live ? r0 + g : nrhs - 1;
+  const float4* Ur = smdf + off / 16 + (size_t)g * D;
+  float qs = 0.f, qe = 0.f;
+#pragma unroll
+  for (int q = 0; q < RPL; ++q) {
+    const int i = li + LR * q;
+    if (i < D) {
+      const float4 v = __ldg(prm.steer_ff + (size_t)rhs * D + i), u = Ur[i];
+      mac(qs, qe, v.x, v.y, u.x, u.z);
+      mac(qs, qe, v.z, v.w, u.y, u.w);
+    }
+  }
+  const ff::F2 qd = lanes_sum2<LR>(qs, qe);
+  const bool good = ok && usable(qd);
+  const Gain sf = gain(qd, -e / 2);
+  if (valid && live) {
+    const long long w0 = (sys * S + rhs) * D;
+#pragma unroll
+    for (int q = 0; q < RPL; ++q) {
+      const int i = li + LR * q;
+      if (i < D && in_bounds(w0 + i, nsys * S * D, kSiteSolveOut)) {
+        const float4 u = Ur[i];
+        wts[w0 + i] = weight({u.x, u.z}, {u.y, u.w}, sf, good);
+      }
+    }
+  }
+}
+
+// Separable steering: u_s = sum_c a_s[c] U_c from the team's basis solutions U
+// (at byte `off` of shared memory) and the normalised weights. 
+template <int LR, int RPL, int TEAM>
+__device__ __noinline__ void combine(const SolveDfParams& prm, int off, long long sys, bool valid, bool ok, int e) {
+  constexpr int NG = TEAM / LR;
+  extern __shared__ float4 smdf[];
+  const float4* U = smdf + off / 16;
+  const int D = prm.D, S = prm.S, C = prm.C;
+  const long long nsys = prm.nsys;
+  float2* __restrict__ wts = prm.wts;
+  const int tt = team_thread<TEAM>(), li = tt % LR, g = tt / LR;
+  // u_s = sum_c a_s[c] U_c: a group takes a steering vector s1 -- with
+  // conjugate-symmetric factors (a_{S-1-s} = conj(a_s)) the pair s1,
+  // S-1-s1 from the four real sums P = sum ar Ur, Q = sum ai Ui,
+  // R = sum ar Ui, T = sum ai Ur: u_s1 = (P - Q) + j (R + T),
+  // u_s2 = (P + Q) + j (R - T)
+  const bool sym = prm.sym != 0;
+  const int n1 = sym ? (S + 1) / 2 : S;
+  for (int p0 = 0; p0 < n1; p0 += NG) {
+    const int s1 = min(p0 + g, n1 - 1), s2 = S - 1 - s1;
+    const bool st1 = valid && p0 + g < n1, st2 = st1 && sym && s2 != s1;
+    const float4* as = prm.sep_a_ff + (size_t)s1 * C;
+    const float4* v1 = prm.steer_ff + (size_t)s1 * D;
+    const float4* v2 = prm.steer_ff + (size_t)s2 * D;
+    ff::F2 w1r[RPL], w1i[RPL], w2r[RPL], w2i[RPL];
+    float q1s = 0.f, q1e = 0.f, q2s = 0.f, q2e = 0.f;
+    constexpr int QB = RPL % 4 == 0 ? 4 : (RPL % 3 == 0 ? 3 : 2);   // rows per pass over the basis
+#pragma unroll
+    for (int q0 = 0; q0 < RPL; q0 += QB) {
+    if (LR * q0 >= D) continue;
+    Cdf PR[QB], TQ[QB];                        // (P, R) and (T, Q) of each row
+#pragma unroll
+    for (int q = 0; q < QB; ++q) PR[q] = TQ[q] = Cdf{0.f, 0.f, 0.f, 0.f};
+    for (int c = 0; c < C; ++c) {
+      const float4 a = __ldg(as + c);
+#pragma unroll
+      for (int q = 0; q < QB; ++q) {
+        const int i = li + LR * (q0 + q);
+        const float4 u = U[(size_t)c * D + (i < D ? i : D - 1)];
+        mac(PR[q].rs, PR[q].re, a.x, a.y, u.x, u.z);
+        mac(TQ[q].is, TQ[q].ie, a.z, a.w, u.y, u.w);
+        mac(PR[q].is, PR[q].ie, a.x, a.y, u.y, u.w);
+        mac(TQ[q].rs, TQ[q].re, a.z, a.w, u.x, u.z);
+      }
+    }
+#pragma unroll
+    for (int q = q0; q < q0 + QB; ++q) {
+      const int i = li + LR * q;
+      norm(PR[q - q0]);
+      norm(TQ[q - q0]);
+      const ff::F2 P{PR[q - q0].rs, PR[q - q0].re}, R{PR[q - q0].is, PR[q - q0].ie};
+      const ff::F2 T{TQ[q - q0].rs, TQ[q - q0].re}, Q{TQ[q - q0].is, TQ[q - q0].ie};
+      const ff::F2 ur1 = ff::sub2(P, Q), ui1 = ff::add2(R, T);
+      const ff::F2 ur2 = ff::add2(P, Q), ui2 = ff::sub2(R, T);
+      if (i < D) {
+        const float4 b1 = __ldg(v1 + i), b2 = __ldg(v2 + i);
+        mac(q1s, q1e, b1.x, b1.y, ur1.hi, ur1.lo);
+        mac(q1s, q1e, b1.z, b1.w, ui1.hi, ui1.lo);
+        mac(q2s, q2e, b2.x, b2.y, ur2.hi, ur2.lo);
+        mac(q2s, q2e, b2.z, b2.w, ui2.hi, ui2.lo);
+      }
+      w1r[q] = ur1;
+      w1i[q] = ui1;
+      w2r[q] = ur2;
+      w2i[q] = ui2;
+    }
+    }
+    const ff::F2 d1 = lanes_sum2<LR>(q1s, q1e), d2 = lanes_sum2<LR>(q2s, q2e);
+    const bool good1 = ok && usable(d1), good2 = ok && usable(d2);
+    const Gain f1 = gain(d1, -e / 2), f2 = gain(d2, -e / 2);
+#pragma unroll
+    for (int q = 0; q < RPL; ++q) {
+      const int i = li + LR * q;
+      if (i < D) {
+        const long long o1 = (sys * S + s1) * D + i, o2 = (sys * S + s2) * D + i, ext = nsys * S * D;
+        if (st1 && in_bounds(o1, ext, kSiteSolveOut))
+          wts[o1] = weight(w1r[q], w1i[q], f1, good1);
+        if (st2 && in_bounds(o2, ext, kSiteSolveOut))
+          wts[o2] = weight(w2r[q], w2i[q], f2, good2);
+      }
+    }
+  }
+}
+
+template <int LR, int RPL, int TEAM, bool F32F>
+__device__ __forceinline__ void solve_df_body(const SolveDfParams& prm, long long bx, long long gx) {
+  constexpr int PASS = TEAM / LR;                  // right-hand sides per pass, one per group
+  const long long nsys = prm.nsys;
+  const int D = prm.D;
+  const bool sep = prm.sep != 0;
+  extern __shared__ float4 smdf[];
+  const int team = TEAM > 32 ? 0 : threadIdx.x / TEAM;   // team in CTA
+  const int teams = TEAM > 32 ? 1 : blockDim.x / TEAM;
+  const int tt = team_thread<TEAM>();
+  System y;
+  y.nu = sep ? prm.C : PASS;
+  const Shared<TEAM, F32F> sh(D, y.nu);
+  y.off = team * sh.bytes;
+  y.aext = nsys * (long long)D * D;
+  const int* okf = reinterpret_cast<const int*>(reinterpret_cast<char*>(smdf) + y.off + sh.ok);
+
+  for (long long base_sys = bx * teams; base_sys < nsys; base_sys += gx * teams) {
+    const long long sys = base_sys + team;
+    const bool valid = sys < nsys;                 // the last CTA's spare teams repeat the last system
+    y.a0 = (valid ? sys : nsys - 1) * (long long)D * D;
+    y.A = prm.cov + y.a0;
+    // trace: lanes over the diagonal (every warp of a CTA team its own sum)
+    constexpr int TW = TEAM > 32 ? 32 : TEAM;
+    double tr = 0.0;
+    for (int j = threadIdx.x % TW; j < D; j += TW)
+      if (in_bounds(y.a0 + (long long)j * D + j, y.aext, kSiteSolveIn)) tr += __ldg(&y.A[(size_t)j * D + j].x);
+    tr = lanes_sum<TW>(tr);
+    y.delta = prm.load_factor * tr * (1.0 / D);
+    // scale 2^-e, e even, trace 2^-e in [1, 4)
+    const int et = (int)(((uint32_t)__double2hiint(tr) >> 20) & 0x7FF);
+    const int e = et == 0 || et == 0x7FF ? 0 : (et - 1023) & ~1;
+    y.sbase = 896 + e;
+    factor<TEAM, F32F>(y, D);
+    const bool ok = *okf != 0;
+    const int nrhs = sep ? prm.C : prm.S;
+    for (int r0 = 0; r0 < nrhs; r0 += PASS) {
+      solve_rhs<LR, RPL, TEAM, F32F>(prm, y, r0);
+      if (!sep) emit<LR, RPL, TEAM>(prm, y.off, sys, valid, ok, e, r0);
+      team_sync<TEAM>();   // the next pass reuses U's rows, the combination reads them all
+    }
+    if (sep) combine<LR, RPL, TEAM>(prm, y.off, sys, valid, ok, e);
+    if (valid && !ok && tt == 0) atomicAdd(&prm.status->n_failed, 1ULL);
+    team_sync<TEAM>();     // the next system reuses the team's shared memory
+  }
+}
+
+constexpr int cta_threads(int team) { return team > 32 ? team : 128; }
+// CTAs per SM that the registers must allow (shared memory allows about as many)
+constexpr int min_ctas(int team) { return team == 512 ? 1 : (team == 256 ? 3 : (team == 64 ? 12 : 6)); }
+
+template <int LR, int RPL, int TEAM, bool F32F>
+__global__ void __launch_bounds__(cta_threads(TEAM), min_ctas(TEAM))
+solve_df_kernel(SolveDfParams p) {
+  solve_df_body<LR, RPL, TEAM, F32F>(p, blockIdx.x, gridDim.x);
+}
+
+// the same solves as a persistent launch over the CPIs of a batch
+template <int LR, int RPL, int TEAM, bool F32F>
+__global__ void __launch_bounds__(cta_threads(TEAM), min_ctas(TEAM))
+solve_df_batched(BatchCtl ctl) {
+  batched_loop<SolveDfParams>(ctl, [&](const SolveDfParams& p, int bx, int, int gx) {
+    solve_df_body<LR, RPL, TEAM, F32F>(p, bx, gx);
+  });
+}
+
+template <int LR, int RPL, int TEAM, bool F32F>
+cudaError_t launch_df(SolveDfParams p, cudaStream_t s) {
+  constexpr int PASS = TEAM / LR;
+  constexpr size_t kMaxSmem = 227 * 1024;
+  // the basis form keeps all C solutions in shared memory
+  if (p.sep && Shared<TEAM, F32F>(p.D, p.C).bytes > (int)kMaxSmem) p.sep = p.sym = 0;
+  const size_t tb = Shared<TEAM, F32F>(p.D, p.sep ? p.C : PASS).bytes;
+  int threads = TEAM;
+  if (TEAM <= 32) {
+    // several teams per CTA; with few systems one warp per CTA, so that they
+    // spread over the SMs
+    threads = p.nsys * TEAM <= 152LL * 4 * 32 ? 32 : 128;
+    while (threads > 32 && tb * (threads / TEAM) > 64 * 1024) threads >>= 1;
+  }
+  const int teams = TEAM > 32 ? 1 : threads / TEAM;
+  const size_t smem = tb * teams;
+  if (smem > kMaxSmem) return cudaErrorInvalidValue;
+  static int set_bytes[64] = {0}, set_bytes_b[64] = {0};
+  cudaError_t err = ensure_smem(solve_df_kernel<LR, RPL, TEAM, F32F>, smem, set_bytes);
+  if (err == cudaSuccess) err = ensure_smem(solve_df_batched<LR, RPL, TEAM, F32F>, smem, set_bytes_b);
+  if (err != cudaSuccess) return err;
+  const long long units = (p.nsys + teams - 1) / teams;
+  const long long blocks = units < (1LL << 30) ? units : (1LL << 30);
+  p.gx = (int)blocks;
+  return launch_params(reinterpret_cast<const void*>(solve_df_kernel<LR, RPL, TEAM, F32F>),
+                       reinterpret_cast<const void*>(solve_df_batched<LR, RPL, TEAM, F32F>),
+                       dim3((unsigned)blocks), threads, smem, s, p, blocks);
+}
+
+}  // namespace
+}  // namespace stap

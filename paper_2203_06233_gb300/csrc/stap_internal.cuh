@@ -35,7 +35,7 @@ struct Tune {
   int apply_kind = 0;  // apply: 1 FP32 register-resident, 2 FP32 general, 3 tensor cores
   int slabs = 0;       // single-CPI run: range slabs pipelined on prioritised streams, 1..8
   int solve_kind = 0;  // D <= 32 solve: 1 register-resident (D = 8, 12, 16), 2 shared-memory
-                       // teams, 3 one system per CTA
+                       // teams, 3 one system per CTA (all FP64; 0: by the load, solve_df.cuh)
   int cov_kind = 0;    // covariance: 1 FP32 error-free, 2 tensor cores (mixed-precision plans)
 };
 
@@ -118,7 +118,8 @@ cudaError_t launch_apply_tc(const float2* dop, const float2* wts, float* out, in
                             int ldr, int T, int B, int S, int precision, DeviceStatus* status,
                             cudaStream_t s, int wait_polls = kDefaultWaitPolls);
 
-// FP64 loading, Cholesky, solves, refinement and scaling for nsys systems.
+// Loading, factorisation, solves, refinement and scaling for nsys systems, by
+// the double-float kernels (solve_df.cuh) or the FP64 ones.
 // cov [nsys][D][D] c128 -> wts [nsys][S][D] c64; steer [S][D] c128.  If
 // sep_g [T] and sep_a [S][C] are given, steer[s] = sep_g (x) sep_a[s] and the
 // solve runs on the C basis vectors instead of the S steering vectors.
