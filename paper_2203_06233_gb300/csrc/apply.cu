@@ -3,14 +3,9 @@
 // the last step of the STAP kernel of arXiv 2203.06233 Sec. 4.2 (the adaptive
 // filter output |w^H x|^2).
 //
-// Mapping: a CTA owns NBB consecutive training blocks of one Doppler bin (up
-// to 256 range cells).  Their weights go to shared memory as [block][d][s]
-// and their D x cells snapshot tile is staged by the same gather as the
-// covariance kernel.  A thread owns one range cell and walks the steering
-// vectors in chunks of SC, keeping SC complex accumulators in registers: per
-// snapshot entry it reads x once and the chunk's weights as broadcast 16-byte
-// loads, i.e. 1 + SC/2 shared loads for 4*SC FMAs.  Each output row
-// out[s][k][cells] is written coalesced along range.
+// Two kernels: a tiled one for any shape, and a register-resident one for
+// small even D.  Both sum over the snapshot entries in increasing order with
+// the same FMAs, so their results are the same bit for bit.
 #include "batch.cuh"
 #include "checked.cuh"
 #include "snapshots.cuh"
@@ -18,98 +13,191 @@
 namespace stap {
 namespace {
 
-constexpr int SC = 8;       // steering vectors per register chunk
-constexpr int kThreads = 256;
-
 // Parameters of one apply launch (one CPI); gx = the launch's grid.x.
 struct ApplyParams {
   const float2* dop;
   const float2* wts;
   float* out;
-  int C, K, R, ldr, T, B, S, NBB, CC;
+  int C, K, R, ldr, T, B, S;
+  int nct, nst;   // tiled kernel: cell tiles per training block, steering tiles
   int gx;
 };
 
-__device__ __forceinline__ void apply_body(const ApplyParams& prm, int bx, int by) {
+// Tiled form: a CTA owns one training block's tile of up to 32 CELLS range
+// cells of one Doppler bin and up to 64 steering vectors, a GEMM of [S][D]
+// weights by [D][cells] snapshots.  Warp w owns 8 steering vectors, a lane
+// CELLS cells: 8 CELLS complex accumulators in registers, fed per snapshot
+// entry by CELLS / 2 16-byte reads of its cells and four broadcast 16-byte
+// reads of the warp's weights for 32 CELLS FMAs, so that the FP32 pipe and not
+// shared memory bounds it.  Both operands come in chunks of DC snapshot
+// entries, two buffers filled by cp.async (8 bytes each: any alignment of the
+// range axis, and the weights land transposed), the next chunk in flight
+// under this chunk's FMAs.  CELLS = 4, 2 or 1 by the block size, so that a
+// tile is not mostly empty lanes.
+//
+// Before: one cell and 8 steering vectors per thread, the whole [D][256]
+// tile staged, then computed, by the one CTA that fits an SM.  C16 K256 R4096
+// T4 B128 S32 (D = 64): 1326 -> 417 us (41 TFLOP/s); C32 K512 R2048 T4 B256 S64
+// (D = 128): 4201 -> 1492 us (46 TFLOP/s).
+constexpr int DC = 16;         // snapshot entries per chunk
+constexpr int kTileS = 64;     // steering vectors per CTA at most
+
+__device__ __forceinline__ void cp_async8(void* dst, const void* src, bool valid) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  const int n = valid ? 8 : 0;   // 0: the eight bytes are zeroed, nothing is read
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+}
+
+template <int CELLS>
+__device__ __forceinline__ void apply_tile_body(const ApplyParams& prm, int bx, int by) {
   const float2* __restrict__ dop = prm.dop;
   const float2* __restrict__ wts = prm.wts;
   float* __restrict__ out = prm.out;
-  const int C = prm.C, K = prm.K, R = prm.R, ldr = prm.ldr, T = prm.T, B = prm.B, S = prm.S,
-            NBB = prm.NBB, CC = prm.CC;
+  const int C = prm.C, K = prm.K, R = prm.R, ldr = prm.ldr, T = prm.T, B = prm.B, S = prm.S;
+  constexpr int RT = 32 * CELLS;
   extern __shared__ float4 sm4[];
-  float2* sm = reinterpret_cast<float2*>(sm4);
-  const int D = C * T;
-  const int NB = R / B;
+  __shared__ long long rowbase[128];               // dop offset of snapshot row d
+  const int nw = blockDim.x >> 5, SP = 8 * nw + 2;
+  float2* xs = reinterpret_cast<float2*>(sm4);     // [2][DC][RT]
+  float2* ws = xs + 2 * DC * RT;                   // [2][DC][SP]
+  const int D = C * T, NB = R / B;
   const int k = by;
-  const int b0 = bx * NBB;
-  const int nbb = min(NBB, NB - b0);
-  const int Sp = (S + SC - 1) / SC * SC;        // padded steering count (zero weights beyond S)
-  float2* ws = sm;                              // [nbb][D][Sp]
-  float2* xs = sm + (size_t)NBB * D * Sp;       // [D][CC + 1]
-  const int ld = CC + 1;
-
-  {  // weights of the nbb blocks, [j][d][s] in shared memory (zero for s >= S)
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int row = warp; row < nbb * Sp; row += nw) {   // row = (block j, steering s)
-      const int j = row / Sp, s = row - j * Sp;
-      const float2* src = wts + (((size_t)k * NB + b0 + j) * S + s) * D;
-      for (int d = lane; d < D; d += 32)
-        ws[((size_t)j * D + d) * Sp + s] =
-            (s < S && in_bounds((((long long)k * NB + b0 + j) * S + s) * D + d, (long long)K * NB * S * D,
-                                kSiteApplyIn))
-                ? __ldg(src + d) : make_float2(0.f, 0.f);
-    }
+  const int st = bx % prm.nst, bt = bx / prm.nst;
+  const int b = bt / prm.nct, ct = bt - b * prm.nct;
+  const int tc = (B + prm.nct - 1) / prm.nct;      // cells of a tile
+  const int c0 = ct * tc, nc = min(tc, B - c0);    // the tile's first cell in the block, its cells
+  const int r0 = b * B + c0;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int d = tid; d < D; d += blockDim.x) {
+    const int t = d / C, c = d - t * C;
+    rowbase[d] = ((long long)c * K + wrap_bin(k + t - T / 2, K)) * ldr + r0;
   }
-  const int cells = nbb * B;
-  for (int c0 = 0; c0 < cells; c0 += CC) {
-    const int cc = min(CC, cells - c0);
-    __syncthreads();
-    stage_snapshots(xs, ld, dop, C, K, ldr, T, k, b0 * B + c0, cc);
-    __syncthreads();
-    for (int rr = threadIdx.x; rr < cc; rr += blockDim.x) {
-      const int j = (c0 + rr) / B;
-      const float2* wj = ws + (size_t)j * D * Sp;
-      const size_t r = (size_t)b0 * B + c0 + rr;
-      for (int s0 = 0; s0 < S; s0 += SC) {
-        float2 acc[SC];
+  __syncthreads();
+  const long long w0 = (((long long)k * NB + b) * S + st * kTileS) * D;
+  const int ns = min(kTileS, S - st * kTileS);     // this CTA's steering vectors
+  auto fill = [&](int d0, int buf) {
+    const int dn = min(DC, D - d0);
+    for (int e = tid; e < dn * RT; e += blockDim.x) {
+      const int d = e / RT, c = e % RT;
+      const long long o = rowbase[d0 + d] + c;
+      const bool ok = c < nc && in_bounds(o, ((long long)C * K - 1) * ldr + R, kSiteApplyIn);
+      cp_async8(xs + (buf * DC + d) * RT + c, dop + (ok ? o : 0), ok);
+    }
+    for (int e = tid; e < 8 * nw * DC; e += blockDim.x) {
+      const int s = e / DC, d = e % DC;
+      const long long o = w0 + (long long)s * D + d0 + d;
+      const bool ok = s < ns && d < dn && in_bounds(o, (long long)K * NB * S * D, kSiteApplyIn);
+      cp_async8(ws + (buf * DC + d) * SP + s, wts + (ok ? o : 0), ok);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float2 acc[8][CELLS];
 #pragma unroll
-        for (int q = 0; q < SC; ++q) acc[q] = make_float2(0.f, 0.f);
-        for (int d = 0; d < D; ++d) {
-          const float2 x = xs[d * ld + rr];
-          const float4* w4 = reinterpret_cast<const float4*>(wj + (size_t)d * Sp + s0);
+  for (int s = 0; s < 8; ++s)
 #pragma unroll
-          for (int q = 0; q < SC / 2; ++q) {
-            const float4 w = w4[q];      // weights s0+2q and s0+2q+1
-            // acc += conj(w) * x
-            acc[2 * q].x = fmaf(w.x, x.x, acc[2 * q].x);
-            acc[2 * q].x = fmaf(w.y, x.y, acc[2 * q].x);
-            acc[2 * q].y = fmaf(w.x, x.y, acc[2 * q].y);
-            acc[2 * q].y = fmaf(-w.y, x.x, acc[2 * q].y);
-            acc[2 * q + 1].x = fmaf(w.z, x.x, acc[2 * q + 1].x);
-            acc[2 * q + 1].x = fmaf(w.w, x.y, acc[2 * q + 1].x);
-            acc[2 * q + 1].y = fmaf(w.z, x.y, acc[2 * q + 1].y);
-            acc[2 * q + 1].y = fmaf(-w.w, x.x, acc[2 * q + 1].y);
-          }
+    for (int c = 0; c < CELLS; ++c) acc[s][c] = make_float2(0.f, 0.f);
+  fill(0, 0);
+  const int nch = (D + DC - 1) / DC;
+  for (int ch = 0; ch < nch; ++ch) {
+    const int buf = ch & 1;
+    if (ch + 1 < nch) {
+      fill((ch + 1) * DC, buf ^ 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+    const int dn = min(DC, D - ch * DC);
+    const float2* xb = xs + buf * DC * RT;
+    const float2* wb = ws + buf * DC * SP + 8 * warp;
+#pragma unroll 2
+    for (int d = 0; d < dn; ++d) {
+      float2 x[CELLS];
+      if constexpr (CELLS == 1) {
+        x[0] = xb[d * RT + lane];
+      } else {
+#pragma unroll
+        for (int c = 0; c < CELLS; c += 2) {       // cells 32 c + 2 lane and the next
+          const float4 v = *reinterpret_cast<const float4*>(xb + d * RT + 32 * c + 2 * lane);
+          x[c] = make_float2(v.x, v.y);
+          x[c + 1] = make_float2(v.z, v.w);
         }
+      }
 #pragma unroll
-        for (int q = 0; q < SC; ++q)
-          if (s0 + q < S && in_bounds(((long long)(s0 + q) * K + k) * ldr + (long long)r,
-                                      ((long long)S * K - 1) * ldr + R, kSiteApplyOut))
-            out[((size_t)(s0 + q) * K + k) * ldr + r] = fmaf(acc[q].x, acc[q].x, acc[q].y * acc[q].y);
+      for (int s = 0; s < 8; s += 2) {
+        const float4 w = *reinterpret_cast<const float4*>(wb + d * SP + s);
+#pragma unroll
+        for (int c = 0; c < CELLS; ++c) {          // acc += conj(w) x
+          acc[s][c].x = fmaf(w.x, x[c].x, acc[s][c].x);
+          acc[s][c].x = fmaf(w.y, x[c].y, acc[s][c].x);
+          acc[s][c].y = fmaf(w.x, x[c].y, acc[s][c].y);
+          acc[s][c].y = fmaf(-w.y, x[c].x, acc[s][c].y);
+          acc[s + 1][c].x = fmaf(w.z, x[c].x, acc[s + 1][c].x);
+          acc[s + 1][c].x = fmaf(w.w, x[c].y, acc[s + 1][c].x);
+          acc[s + 1][c].y = fmaf(w.z, x[c].y, acc[s + 1][c].y);
+          acc[s + 1][c].y = fmaf(-w.w, x[c].x, acc[s + 1][c].y);
+        }
+      }
+    }
+    __syncthreads();                               // the buffer is refilled next
+  }
+  const long long ext = ((long long)S * K - 1) * ldr + R;
+  const bool even = ((r0 | ldr) & 1) == 0 && (reinterpret_cast<uintptr_t>(out) & 7) == 0;
+#pragma unroll
+  for (int s = 0; s < 8; ++s) {
+    if (8 * warp + s >= ns) break;
+    const long long o = ((long long)(st * kTileS + 8 * warp + s) * K + k) * ldr + r0;
+    float p[CELLS];
+#pragma unroll
+    for (int c = 0; c < CELLS; ++c) p[c] = fmaf(acc[s][c].x, acc[s][c].x, acc[s][c].y * acc[s][c].y);
+    if constexpr (CELLS == 1) {
+      if (lane < nc && in_bounds(o + lane, ext, kSiteApplyOut)) out[o + lane] = p[0];
+    } else {
+#pragma unroll
+      for (int c = 0; c < CELLS; c += 2) {
+        const int cell = 32 * c + 2 * lane;
+        if (even && cell + 1 < nc) {
+          if (in_bounds(o + cell + 1, ext, kSiteApplyOut))
+            *reinterpret_cast<float2*>(out + o + cell) = make_float2(p[c], p[c + 1]);
+        } else {
+          if (cell < nc && in_bounds(o + cell, ext, kSiteApplyOut)) out[o + cell] = p[c];
+          if (cell + 1 < nc && in_bounds(o + cell + 1, ext, kSiteApplyOut)) out[o + cell + 1] = p[c + 1];
+        }
       }
     }
   }
 }
 
-__global__ void __launch_bounds__(kThreads)
-apply_kernel(ApplyParams p) {
-  apply_body(p, blockIdx.x, blockIdx.y);
+template <int CELLS>
+__global__ void __launch_bounds__(256, CELLS == 4 ? 2 : (CELLS == 2 ? 3 : 4))
+apply_tile_kernel(ApplyParams p) {
+  apply_tile_body<CELLS>(p, blockIdx.x, blockIdx.y);
 }
 
 // the same apply as a persistent launch over the CPIs of a batch
-__global__ void __launch_bounds__(kThreads)
-apply_batched(BatchCtl ctl) {
-  batched_loop<ApplyParams>(ctl, [&](const ApplyParams& p, int bx, int by, int) { apply_body(p, bx, by); });
+template <int CELLS>
+__global__ void __launch_bounds__(256, CELLS == 4 ? 2 : (CELLS == 2 ? 3 : 4))
+apply_tile_batched(BatchCtl ctl) {
+  batched_loop<ApplyParams>(ctl, [&](const ApplyParams& p, int bx, int by, int) {
+    apply_tile_body<CELLS>(p, bx, by);
+  });
+}
+
+template <int CELLS>
+cudaError_t launch_apply_tile(const float2* dop, const float2* wts, float* out, int C, int K, int R, int ldr,
+                              int T, int B, int S, cudaStream_t s) {
+  constexpr int RT = 32 * CELLS;
+  const int nct = (B + RT - 1) / RT, nst = (S + kTileS - 1) / kTileS;
+  const int nw = (min(S, kTileS) + 7) / 8;
+  const size_t smem = 2 * (size_t)DC * (RT + 8 * nw + 2) * sizeof(float2);
+  static int set_bytes[64] = {0}, set_bytes_b[64] = {0};
+  cudaError_t e = ensure_smem(apply_tile_kernel<CELLS>, smem, set_bytes);
+  if (e == cudaSuccess) e = ensure_smem(apply_tile_batched<CELLS>, smem, set_bytes_b);
+  if (e != cudaSuccess) return e;
+  dim3 grid((unsigned)(R / B) * nct * nst, K);
+  const ApplyParams p{dop, wts, out, C, K, R, ldr, T, B, S, nct, nst, (int)grid.x};
+  return launch_params(reinterpret_cast<const void*>(apply_tile_kernel<CELLS>),
+                       reinterpret_cast<const void*>(apply_tile_batched<CELLS>), grid, 32 * nw, smem, s, p);
 }
 
 // Register-resident form for small even D (the common shapes).  A thread owns
@@ -210,7 +298,7 @@ cudaError_t launch_apply_reg(const float2* dop, const float2* wts, float* out, i
   if (e == cudaSuccess) e = ensure_smem(apply_reg_batched<D>, smem, set_bytes_b);
   if (e != cudaSuccess) return e;
   dim3 grid((R + kRegCells - 1) / kRegCells, K);
-  const ApplyParams p{dop, wts, out, C, K, R, ldr, T, B, S, 0, 0, (int)grid.x};
+  const ApplyParams p{dop, wts, out, C, K, R, ldr, T, B, S, 1, 1, (int)grid.x};
   return launch_params(reinterpret_cast<const void*>(apply_reg_kernel<D>),
                        reinterpret_cast<const void*>(apply_reg_batched<D>), grid, kRegThreads, smem, s, p);
 }
@@ -245,25 +333,15 @@ cudaError_t launch_apply(const float2* dop, const float2* wts, float* out, int C
       default: break;
     }
   }
-  constexpr size_t kBudget = 160 * 1024;
-  const int Sp = (S + SC - 1) / SC * SC;
-  int NBB = B >= kThreads ? 1 : kThreads / B;   // up to 256 cells per CTA
-  if (NBB > NB) NBB = NB;
-  auto wbytes = [&](int nbb) { return (size_t)nbb * D * Sp * sizeof(float2); };
-  while (NBB > 1 && wbytes(NBB) > kBudget / 2) --NBB;
-  if (wbytes(NBB) + (size_t)D * 2 * sizeof(float2) > kBudget) return cudaErrorInvalidValue;
-  int CC = NBB * B;                              // cells staged per pass
-  if (wbytes(NBB) + (size_t)D * (CC + 1) * sizeof(float2) > kBudget)
-    CC = (int)((kBudget - wbytes(NBB)) / ((size_t)D * sizeof(float2))) - 1;
-  const size_t smem = wbytes(NBB) + (size_t)D * (CC + 1) * sizeof(float2);
-  static int set_bytes[64] = {0}, set_bytes_b[64] = {0};
-  cudaError_t e = ensure_smem(apply_kernel, smem, set_bytes);
-  if (e == cudaSuccess) e = ensure_smem(apply_batched, smem, set_bytes_b);
-  if (e != cudaSuccess) return e;
-  dim3 grid((NB + NBB - 1) / NBB, K);
-  const ApplyParams p{dop, wts, out, C, K, R, ldr, T, B, S, NBB, CC, (int)grid.x};
-  return launch_params(reinterpret_cast<const void*>(apply_kernel), reinterpret_cast<const void*>(apply_batched),
-                       grid, kThreads, smem, s, p);
+  // cells per lane: the tile size (128, 64 or 32 cells) that pads the block
+  // least, and where a tile is one or two chunks deep, i.e. nothing hides its
+  // loads but other CTAs, the smaller tiles of which more fit an SM
+  // (D = 15, K128 R3000 B100 S11: 38.7 us with 64-cell tiles, 41.9 with 128)
+  auto padded = [&](int cells) { return (B + 32 * cells - 1) / (32 * cells) * cells; };
+  if (D > 2 * DC && padded(4) <= padded(2) && padded(4) <= padded(1))
+    return launch_apply_tile<4>(dop, wts, out, C, K, R, ldr, T, B, S, s);
+  if (padded(2) <= padded(1)) return launch_apply_tile<2>(dop, wts, out, C, K, R, ldr, T, B, S, s);
+  return launch_apply_tile<1>(dop, wts, out, C, K, R, ldr, T, B, S, s);
 }
 
 }  // namespace stap
