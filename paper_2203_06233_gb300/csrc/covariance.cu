@@ -19,6 +19,9 @@
 // D x B snapshot tiles in shared memory (chunks of BC cells if B is large) and
 // gives each thread whole entries (i >= l) of the lower triangle; the upper
 // triangle is written as the conjugate mirror.
+#include <algorithm>
+#include <cmath>
+
 #include "df64.cuh"
 #include "batch.cuh"
 #include "checked.cuh"
@@ -109,30 +112,45 @@ covariance_ff_kernel(const float2* __restrict__ dop, double2* __restrict__ cov, 
 //
 // Accumulation on a fixed grid (error-free transformation in the manner of
 // Rump, Ogita & Oishi, "Accurate floating-point summation part I", SISC 2008,
-// ExtractScalar): for an entry whose row maxima are m1, m2 pick the power of
-// two sig >= 4 B m1 m2.  For each product, s = fma(a, b, sig) rounds a*b onto
-// the grid of sig, q = s - sig is exact, and the running sum of the q stays
-// exact because every q lies on that grid and |sum| <= sig/2.  The remainder
-// fma(a, b, -q) (|.| <= ulp(sig)/2) goes to a second FP32 accumulator.  Five
-// FP32 instructions per real product; the pair is combined in FP64 at the end.
-constexpr int kPairMaxThreads = 1024;   // one thread per Q entry, up to this
+// ExtractScalar).  An entry's partial sums, and the products in them, are at
+// most n1 n2 in magnitude, the product of its two rows' 2-norms over the cells
+// (Cauchy and Schwarz, for any subset of the terms), so with a power of two
+// sig >= 2 n1 n2 a running sum that starts at 1.5 sig stays inside [sig, 2 sig),
+// where floats are the multiples of ulp(sig).  Each product is added by
+// t = fma(a, b, s), which rounds the product onto that grid; q = t - s is
+// exact, and what the grid left out, fma(a, b, -q) (|.| <= ulp(sig) / 2), goes
+// to a second FP32 accumulator: four FP32 instructions per real product.  At
+// the end s - 1.5 sig is exact, and the pair is combined in FP64.  (Bounding
+// the sums by 4 B m1 m2 with the rows' maxima, as before, takes a fifth
+// instruction -- the sums then start at zero beside the grid constant -- on a
+// grid about eight times coarser for noise-like rows.)
+//
+// A thread computes one entry, two cells per pair of 16-byte reads of shared
+// memory for 32 FP32 instructions.  The row pitch is an odd number of 16-byte
+// units, so eight lanes reading eight consecutive rows touch all the banks
+// once.  (Two by two entries per thread halve the reads but leave a quarter
+// of the warps: slower but for D = 64, 5% there.)
+// Measured, before and after: C16 K256 R4096 T4 B128 (D = 64) 1387 -> 1036 us;
+// C8 K256 R8192 T3 B64 (D = 24) 577 -> 433; C4 K256 R4096 T3 B64 (D = 12) 79.1 ->
+// 69; error against 64 bits at D = 64 5.6e-12 -> 7.6e-13.
+constexpr int kPairMaxThreads = 1024;   // one thread per entry, up to this
 
-__device__ __forceinline__ float pow2_ceil(float x) {  // smallest power of two >= x
+__device__ __forceinline__ float pow2_ceil(float x) {  // smallest power of two >= x, at most 2^126
   if (!(x > 0.f)) return 1.0f;
   unsigned u = __float_as_uint(x);
   unsigned e = u >> 23;
   if (u & 0x7fffffu) e += 1;
   if (e < 1) e = 1;
-  if (e > 254) e = 254;
+  if (e > 253) e = 253;
   return __uint_as_float(e << 23);
 }
 
-__device__ __forceinline__ void grid_add(float& hi, float& lo, float a, float b, float sig) {
-  const float s = __fmaf_rn(a, b, sig);
-  const float q = __fsub_rn(s, sig);
-  const float r = __fmaf_rn(a, b, -q);
-  hi = __fadd_rn(hi, q);
-  lo = __fadd_rn(lo, r);
+// s += a b on the grid, the remainder to lo
+__device__ __forceinline__ void grid_add(float& s, float& lo, float a, float b) {
+  const float t = __fmaf_rn(a, b, s);
+  const float q = __fsub_rn(t, s);
+  lo = __fadd_rn(lo, __fmaf_rn(a, b, -q));
+  s = t;
 }
 
 // Parameters of one bin-pair launch (one CPI): grid gx = NB blocks by K / KT
@@ -141,9 +159,13 @@ struct CovPairsParams {
   const float2* dop;
   double2* cov;
   int C, K, ldr, T, B, NB, KT, CB;
+  int lower;       // write only the lower triangle
   double invB;
   int gx;
 };
+
+// row pitch in cells: at least cb, and an odd number of 16-byte units
+__host__ __device__ constexpr int pair_ld(int cb) { return (cb + 1) / 4 * 4 + 2; }
 
 __device__ __forceinline__ void covariance_pairs_body(const CovPairsParams& prm, int bx, int by) {
   const float2* __restrict__ dop = prm.dop;
@@ -157,41 +179,62 @@ __device__ __forceinline__ void covariance_pairs_body(const CovPairsParams& prm,
   const int h = T / 2;
   const int NBIN = KT + T - 1;                    // staged bins k0-h .. k0+KT-1+(T-1-h)
   const int nrows = NBIN * C;
-  const int ld = CB + 1;
+  const int ld = pair_ld(CB);
   const int Ediag = C * (C + 1) / 2, Eoff = C * C;
-  // items: d-major; d = 0 has NBIN * Ediag items, d > 0 has (NBIN - d) * Eoff
+  // entries: d-major; d = 0 has NBIN * Ediag, d > 0 has (NBIN - d) * Eoff
   const int nitems = NBIN * Ediag + (T - 1) * (2 * NBIN - T) / 2 * Eoff;
   double2* Q = smd;                                             // [nitems]
-  float* m = reinterpret_cast<float*>(Q + nitems);              // [nrows] row maxima
+  float* m = reinterpret_cast<float*>(Q + nitems);              // [nrows] row norms
   float2* X = reinterpret_cast<float2*>(m + ((nrows + 3) & ~3));  // [nrows][ld]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   const bool pow2B = (B & (B - 1)) == 0;
   const float invBf = 1.0f / (float)B;
-
   // the B cells in chunks of CB: each chunk is summed error-free on its own
   // grid and added to Q in FP64
   for (int c0 = 0; c0 < B; c0 += CB) {
     const int cc = min(CB, B - c0);
+    const int ce = (cc + 1) & ~1;                  // cells come in pairs: a zero follows an odd last one
     __syncthreads();
     for (int row = warp; row < nrows; row += nwarps) {   // rows (bin j, channel c)
       const int j = row / C, c = row - j * C;
       const int kk = wrap_bin(k0 - h + j, K);
       const float2* src = dop + ((size_t)c * K + kk) * ldr + (size_t)b * B + c0;
       float2* dst = X + row * ld;
-      float mx = 0.f;
-      for (int cell = lane; cell < cc; cell += 32) {
-        const bool ok = in_bounds(((long long)c * K + kk) * ldr + (long long)b * B + c0 + cell,
-                                  ((long long)C * K - 1) * ldr + (long long)NB * B, kSiteCovIn);
+      float ss = 0.f;
+      for (int cell = lane; cell < ce; cell += 32) {
+        const bool ok = cell < cc && in_bounds(((long long)c * K + kk) * ldr + (long long)b * B + c0 + cell,
+                                               ((long long)C * K - 1) * ldr + (long long)NB * B, kSiteCovIn);
         const float2 x = ok ? __ldg(src + cell) : make_float2(0.f, 0.f);
         dst[cell] = x;
-        mx = fmaxf(mx, fmaxf(fabsf(x.x), fabsf(x.y)));
+        ss = fmaf(x.x, x.x, ss);
+        ss = fmaf(x.y, x.y, ss);
       }
-      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      if (lane == 0) m[row] = mx;
+      for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+      float n = sqrtf(ss);
+      if (!(ss > 1e-24f && ss < 1e36f)) {          // warp-uniform: squares may have over- or underflowed
+        // again from values scaled by the power of two next to the largest; a
+        // row with an infinity or NaN keeps its largest value, its entries are
+        // not finite either
+        float mx = 0.f;
+        for (int cell = lane; cell < cc; cell += 32) mx = fmaxf(mx, fmaxf(fabsf(dst[cell].x), fabsf(dst[cell].y)));
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        n = mx;
+        if (mx > 0.f && mx < __int_as_float(0x7f800000)) {
+          const float up = pow2_ceil(mx), dn = 1.0f / up;
+          ss = 0.f;
+          for (int cell = lane; cell < cc; cell += 32) {
+            const float2 x = dst[cell];
+            ss = fmaf(x.x * dn, x.x * dn, ss);
+            ss = fmaf(x.y * dn, x.y * dn, ss);
+          }
+          for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+          n = up * sqrtf(ss);
+        }
+      }
+      if (lane == 0) m[row] = n;
     }
     __syncthreads();
 
-    const float fourB = 4.0f * (float)cc;
     for (int it = threadIdx.x; it < nitems; it += blockDim.x) {
       int d = 0, rem = it;
       if (rem >= NBIN * Ediag) {
@@ -213,18 +256,23 @@ __device__ __forceinline__ void covariance_pairs_body(const CovPairsParams& prm,
         c2 = e - c1 * C;
       }
       const int ra = j1 * C + c1, rb = (j1 + d) * C + c2;
-      const float2* xa = X + ra * ld;
-      const float2* xb = X + rb * ld;
-      const float sig = pow2_ceil(fourB * m[ra] * m[rb]);
-      float hr = 0.f, lr = 0.f, hi = 0.f, li = 0.f;
+      const float4* xa = reinterpret_cast<const float4*>(X + ra * ld);   // two cells each
+      const float4* xb = reinterpret_cast<const float4*>(X + rb * ld);
+      const float s0 = 1.5f * pow2_ceil(2.01f * m[ra] * m[rb]);
+      float sr = s0, si = s0, lr = 0.f, li = 0.f;
 #pragma unroll 4
-      for (int cell = 0; cell < cc; ++cell) {
-        const float2 a = xa[cell], bb = xb[cell];
-        grid_add(hr, lr, a.x, bb.x, sig);
-        grid_add(hr, lr, a.y, bb.y, sig);
-        grid_add(hi, li, a.y, bb.x, sig);
-        grid_add(hi, li, -a.x, bb.y, sig);
+      for (int p = 0; p < ce / 2; ++p) {
+        const float4 a = xa[p], bb = xb[p];
+        grid_add(sr, lr, a.x, bb.x);
+        grid_add(si, li, a.y, bb.x);
+        grid_add(sr, lr, a.y, bb.y);
+        grid_add(si, li, -a.x, bb.y);
+        grid_add(sr, lr, a.z, bb.z);
+        grid_add(si, li, a.w, bb.z);
+        grid_add(sr, lr, a.w, bb.w);
+        grid_add(si, li, -a.z, bb.w);
       }
+      const float hr = __fsub_rn(sr, s0), hi = __fsub_rn(si, s0);   // exact
       double2 v;
       if (pow2B) {  // 1/B is a power of two: scaling the pair in FP32 is exact
         v = make_double2(ff::f2d_exact(hr * invBf) + ff::f2d_exact(lr * invBf),
@@ -258,6 +306,7 @@ __device__ __forceinline__ void covariance_pairs_body(const CovPairsParams& prm,
     const int kl = idx / (D * D);
     const int e = idx - kl * D * D;
     const int i = e / D, l = e - i * D;
+    if (prm.lower && l > i) continue;
     const int t1 = i / C, c1 = i - t1 * C, t2 = l / C, c2 = l - t2 * C;
     double2 v;
     if (t1 <= t2) {
@@ -285,10 +334,22 @@ covariance_pairs_batched(BatchCtl ctl) {
   });
 }
 
+// Entries of KT bins, and the threads that take them: whole warps, at most
+// kPairMaxThreads with the rounds balanced above that.
+int pair_items(int C, int T, int KT) {
+  const int nbin = KT + T - 1;
+  return nbin * (C * (C + 1) / 2) + (T - 1) * (2 * nbin - T) / 2 * C * C;
+}
+int pair_threads(int items) {
+  const int rounds = (items + kPairMaxThreads - 1) / kPairMaxThreads;
+  const int threads = ((items + rounds - 1) / rounds + 31) / 32 * 32;
+  return threads < 64 ? 64 : threads;
+}
+
 }  // namespace
 
 cudaError_t launch_covariance_fp32(const float2* dop, double2* cov, int C, int K, int R, int ldr,
-                                   int T, int B, cudaStream_t s, const Tune& tn) {
+                                   int T, int B, cudaStream_t s, const Tune& tn, bool lower_only) {
   const int D = C * T;
   const int E = D * (D + 1) / 2;
   const int NB = R / B;
@@ -298,15 +359,33 @@ cudaError_t launch_covariance_fp32(const float2* dop, double2* cov, int C, int K
   {
     constexpr size_t kPairBudget = 200 * 1024;
     auto pair_smem = [&](int kt, int cb) {
-      const int nbin = kt + T - 1;
-      const size_t nitems = (size_t)nbin * (C * (C + 1) / 2) +
-                            (size_t)(T - 1) * (2 * nbin - T) / 2 * C * C;
-      const size_t nrows = (size_t)nbin * C;
-      return nitems * sizeof(double2) + ((nrows + 3) & ~(size_t)3) * sizeof(float) +
-             nrows * (cb + 1) * sizeof(float2);
+      const size_t nrows = (size_t)(kt + T - 1) * C;
+      return (size_t)pair_items(C, T, kt) * sizeof(double2) + ((nrows + 3) & ~(size_t)3) * sizeof(float) +
+             nrows * pair_ld(cb) * sizeof(float2);
     };
-    int KT = K < 16 ? K : 16;  // K is a power of two, so KT divides it
-    while (KT > 1 && pair_smem(KT, B) > kPairBudget) KT >>= 1;
+    // Bins per CTA, the least time by a model of the rounds of CTAs over the
+    // SMs: more bins share more products, but fewer CTAs fit an SM beside one
+    // another, and w resident warps reach about w / (w + 12) of the issue rate
+    // (fitted to the measured times of KT = 1 .. 16 at ten shapes of D = 4 to
+    // 80; within 9% of the fastest KT on each).
+    int KT = 1;
+    double best = 1e300;
+    for (int kt = 1; kt <= 16 && kt <= K; kt *= 2) {   // K is a power of two, so kt divides it
+      const size_t sm = pair_smem(kt, B);
+      if (sm > kPairBudget) break;
+      const int items = pair_items(C, T, kt), threads = pair_threads(items);
+      const int slots = (items + threads - 1) / threads * threads;   // whole rounds of the CTA
+      const double ctas = (double)NB * (K / kt), warps = threads / 32;
+      double per = (double)((228 * 1024) / (sm + 1024));             // CTAs per SM: shared memory,
+      per = std::min({per, std::floor(51.0 / warps), std::ceil(ctas / 152.0)});   // 40 registers, the grid
+      if (per < 1.0) per = 1.0;
+      const double w = per * warps;
+      const double t = std::max(ctas / (152.0 * per), 1.0) * per * slots * (w + 12.0) / w;
+      if (t < best) {
+        best = t;
+        KT = kt;
+      }
+    }
     if (tn.cov_kt > 0 && tn.cov_kt <= K && K % tn.cov_kt == 0 && pair_smem(tn.cov_kt, B) <= kPairBudget)
       KT = tn.cov_kt;
     int CB = B;
@@ -318,23 +397,10 @@ cudaError_t launch_covariance_fp32(const float2* dop, double2* cov, int C, int K
       if (e == cudaSuccess) e = ensure_smem(covariance_pairs_batched, smem, set_bytes_b);
       if (e != cudaSuccess) return e;
       dim3 grid(NB, K / KT);
-      // Many Q entries (large C): one thread per entry, rounded up to whole
-      // warps (at most 32 warps, rounds balanced above that), so that they
-      // are not spread unevenly over a last, partly idle round of threads.
-      // Few entries: 256 threads, which share the SMs better with the solve
-      // kernels of other range slabs.
-      const int nbin = KT + T - 1;
-      const int nitems = nbin * (C * (C + 1) / 2) + (T - 1) * (2 * nbin - T) / 2 * C * C;
-      int threads = 256;
-      if (nitems > 512) {
-        const int rounds = (nitems + kPairMaxThreads - 1) / kPairMaxThreads;
-        threads = ((nitems + rounds - 1) / rounds + 31) / 32 * 32;
-        if (threads > kPairMaxThreads) threads = kPairMaxThreads;
-      }
-      const CovPairsParams p{dop, cov, C, K, ldr, T, B, NB, KT, CB, 1.0 / (double)B, (int)grid.x};
+      const CovPairsParams p{dop, cov, C, K, ldr, T, B, NB, KT, CB, lower_only ? 1 : 0, 1.0 / (double)B, (int)grid.x};
       return launch_params(reinterpret_cast<const void*>(covariance_pairs_kernel),
-                           reinterpret_cast<const void*>(covariance_pairs_batched), grid, threads, smem,
-                           s, p);
+                           reinterpret_cast<const void*>(covariance_pairs_batched), grid,
+                           pair_threads(pair_items(C, T, KT)), smem, s, p);
     }
   }
   // general form: one tile per system, cells in chunks

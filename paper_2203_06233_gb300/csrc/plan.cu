@@ -300,7 +300,7 @@ stap_status do_doppler(stap_plan p, const Cpi& c, const void* cube, void* dop, c
 }
 
 // lower: the chain's own buffer, of which the solve reads only the lower
-// triangle (the tensor-core kernels then skip the upper one)
+// triangle (the kernels then skip the upper one)
 stap_status do_covariance(stap_plan p, const Cpi& c, const void* dop, void* cov, cudaStream_t st,
                           int nr = -1, bool lower = false) {
   NvtxRange range("stap_covariance");
@@ -317,7 +317,7 @@ stap_status do_covariance(stap_plan p, const Cpi& c, const void* dop, void* cov,
   return check_launch(stap::launch_covariance_fp32(static_cast<const float2*>(dop),
                                                    static_cast<double2*>(cov), c.Cd, d.n_dop,
                                                    R, d.n_range, c.Td, d.training_block, st,
-                                                   c.tune));
+                                                   c.tune, lower));
 }
 
 stap_status do_solve(stap_plan p, const Cpi& c, const void* cov, void* wts, cudaStream_t st,

@@ -93,9 +93,11 @@ cudaError_t launch_doppler(const float2* cube, float2* dop, const float* win, co
                            const Tune& t = Tune());
 
 // Covariance per (k, block) from the Doppler cube, accumulated error-free in
-// FP32 pairs; written as FP64 complex [K][NB][D][D] (full Hermitian).
+// FP32 pairs; written as FP64 complex [K][NB][D][D] (full Hermitian, or with
+// lower_only at least the lower triangle).
 cudaError_t launch_covariance_fp32(const float2* dop, double2* cov, int C, int K, int R, int ldr,
-                                   int T, int B, cudaStream_t s, const Tune& t = Tune());
+                                   int T, int B, cudaStream_t s, const Tune& t = Tune(),
+                                   bool lower_only = false);
 
 // True for the precisions whose covariance and apply run on the tensor cores.
 bool tc_precision(int precision);
