@@ -354,17 +354,18 @@ stap_status do_apply(stap_plan p, const Cpi& c, const void* dop, const void* wts
                                          c.tune));
 }
 
+// the training matrices inside a run: the lower triangles, all the solve reads
 stap_status do_train(stap_plan p, const Cpi& c, const void* cov, void* ctr, cudaStream_t st) {
   if (p->opt.training == STAP_TRAIN_WINDOW) {
     NvtxRange range("stap_train_window");
     return check_launch(stap::launch_train_window(static_cast<const double2*>(cov),
                                                   static_cast<double2*>(ctr), c.d.n_dop, c.NB, c.D,
-                                                  p->opt.train_guard, p->opt.train_half, st));
+                                                  p->opt.train_guard, p->opt.train_half, st, true));
   }
   NvtxRange range("stap_train_neighbours");
   return check_launch(stap::launch_train_neighbours(static_cast<const double2*>(cov),
                                                     static_cast<double2*>(ctr), c.d.n_dop, c.NB,
-                                                    c.D, st));
+                                                    c.D, st, true));
 }
 
 // ctr: the training matrices' buffer when the plan trains on neighbour blocks

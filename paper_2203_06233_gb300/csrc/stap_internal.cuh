@@ -44,15 +44,16 @@ struct Tune {
 cudaError_t launch_pivot_reciprocal(const double* in, double* out, long long n, cudaStream_t s);
 
 // Training with guard cells: out[k][b] = mean of in[k][b-1] and in[k][b+1]
-// (the one that exists at either end); NB >= 2.
+// (the one that exists at either end); NB >= 2.  lower_only: the lower
+// triangles only (the rest of out is left as it is).
 cudaError_t launch_train_neighbours(const double2* in, double2* out, int K, int NB, int D,
-                                    cudaStream_t s);
+                                    cudaStream_t s, bool lower_only = false);
 
 // Sliding training window: out[k][j] = mean of in[k][i] over the groups
 // i = j-guard-half .. j-guard-1 and j+guard+1 .. j+guard+half in 0 .. NB-1;
 // needs guard >= 0, half >= 1, NB >= 2 guard + 2.
 cudaError_t launch_train_window(const double2* in, double2* out, int K, int NB, int D, int guard,
-                                int half, cudaStream_t s);
+                                int half, cudaStream_t s, bool lower_only = false);
 
 // First out-of-range index found by the checked build in one source file
 // (checked.cuh): how many accesses were skipped, and the first one's site
