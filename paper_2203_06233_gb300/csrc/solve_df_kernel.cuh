@@ -35,8 +35,8 @@
 // trace become zero; an infinity or NaN becomes a NaN, which no pivot test
 // passes.
 //
-// Layout.  A system belongs to a team of TEAM threads: 16 lanes of a warp
-// (D <= 16) or a CTA of 64 (D <= 32), 256 (D <= 64) or 512 (D <= 128) threads.
+// Layout.  A system belongs to a team of TEAM threads: half a warp or a warp
+// (D <= 16) or a CTA of 64, 128 (D <= 32), 256 (D <= 64) or 512 (D <= 128) threads.
 // LR lanes hold one right-hand side, row li + LR q in register q < RPL.  The
 // factor (column-major packed) and the solutions stay in shared memory, the
 // column's entry is broadcast by shuffles, so a 16-byte read feeds one complex
@@ -221,7 +221,7 @@ __device__ __forceinline__ void subst(Cdf (&x)[RPL], const float4* L, int D, int
     // column i = li + LR q lies at cstart(i) - i + j, which is b0 + b1 q -
     // q^2 LR^2 / 2 + j
     const int b0 = li * D - li * (li - 1) / 2 - li, b1 = LR * D - LR * li - LR / 2;
-#pragma unroll 2
+#pragma unroll (LR >= 16 ? 2 : 1)
     for (int jj = 0; jj < jn; ++jj) {
       const int jo = BACK ? jn - 1 - jj : jj;
       const int j = LR * qb + jo;
@@ -311,13 +311,18 @@ __device__ __forceinline__ void ldl_solve_f32(Cdf (&x)[RPL], const float2* L, co
   for (int q = 0; q < RPL; ++q) x[q] = Cdf{xf[q].x, 0.f, xf[q].y, 0.f};
 }
 
-// Shared memory of one team: the solutions U [nu][D], Rl's columns As (a chunk
-// [KC][D + 1], or all D columns where the team is part of a warp: small
-// systems convert their matrix once), the two pivot columns before division
+// Shared memory of one team: the solutions U [nu][D], Rl in As (a chunk of
+// columns [KC][D + 1], or where the team is part of a warp the whole matrix:
+// small systems convert it once -- as columns [D][D + 1] (SQUARE), or for more
+// than 12 rows, where that would cost a third of the resident warps (D = 15:
+// 197 -> 160 us per 3840 systems), as the lower triangle packed like the factor), the two pivot columns before division
 // [2][D] (in the chunk's place: the factorisation is over before the first
 // residual), the factor [Dp] (column-major packed), the pivot reciprocals [D]
 // and the pivot flag.
-template <int TEAM, bool F32F>
+template <int LR, int RPL>
+__host__ __device__ constexpr bool square() { return LR * RPL <= 12; }
+
+template <int TEAM, bool F32F, bool SQUARE>
 struct Shared {
   static constexpr bool FULL = TEAM <= 32;
   using LT = typename std::conditional<F32F, float2, float4>::type;   // factor entries
@@ -326,7 +331,7 @@ struct Shared {
     const int Dp = D * (D + 1) / 2;
     u = 0;
     as = u + nu * D * 16;
-    col = FULL ? as + D * (D + 1) * 16 : as;
+    col = FULL ? as + (SQUARE ? D * (D + 1) : Dp) * 16 : as;
     l = FULL ? col + 2 * D * 16 : as + KC * (D + 1) * 16;
     rd = l + (Dp * (int)sizeof(LT) + 15) / 16 * 16;
     ok = rd + (D * 8 + 15) / 16 * 16;
@@ -381,11 +386,12 @@ __device__ __forceinline__ ff::F2 pivot(ff::F2 d, int* okf) {
 // thread forms the two pivots' reciprocals itself.  Phase 2: the rank-2 update
 // of the trailing triangle, its columns spread over groups of RW threads, a
 // group's threads over a column's rows.
-template <int TEAM, bool F32F>
+template <int TEAM, bool F32F, bool SQUARE>
 __device__ __forceinline__ void factor(const System y, int D) {
   extern __shared__ float4 smdf[];
-  const Shared<TEAM, F32F> sh(D, y.nu);
-  using LT = typename Shared<TEAM, F32F>::LT;
+  using SH = Shared<TEAM, F32F, SQUARE>;
+  const SH sh(D, y.nu);
+  using LT = typename SH::LT;
   char* base = reinterpret_cast<char*>(smdf) + y.off;
   LT* L = reinterpret_cast<LT*>(base + sh.l);
   LT* colb = reinterpret_cast<LT*>(base + sh.col);
@@ -396,10 +402,14 @@ __device__ __forceinline__ void factor(const System y, int D) {
   auto put = [&](int i, int l, float4 v) {
     if constexpr (F32F) L[cstart(l, D) + i - l] = make_float2(__fadd_rn(v.x, v.z), __fadd_rn(v.y, v.w));
     else L[cstart(l, D) + i - l] = v;
-    if constexpr (Shared<TEAM, F32F>::FULL) {
+    if constexpr (SH::FULL) {
       float4* As = reinterpret_cast<float4*>(base + sh.as);
-      As[l * (D + 1) + i] = v;                     // column l, row i
-      As[i * (D + 1) + l] = conj4(v);
+      if constexpr (!SQUARE) {
+        As[cstart(l, D) + i - l] = v;
+      } else {
+        As[l * (D + 1) + i] = v;                   // column l, row i
+        As[i * (D + 1) + l] = conj4(v);
+      }
     }
   };
   if constexpr (TEAM > 32) {                       // rows coalesced
@@ -501,7 +511,7 @@ __device__ __forceinline__ void factor(const System y, int D) {
       team_sync<TEAM>();
       if (own1) L[cj + 1] = own;
     }
-    constexpr int RW = TEAM == 512 ? 32 : (TEAM == 256 ? 16 : (TEAM == 64 ? 8 : 4));
+    constexpr int RW = TEAM == 512 ? 32 : (TEAM >= 128 ? 16 : (TEAM >= 32 ? 8 : 4));
     for (int l = j + 2 + tt / RW; l < D; l += TEAM / RW) {
       const LT alj = colb[l], blj = colb2[l];
       LT* cl = L + cstart(l, D) - l;
@@ -536,7 +546,7 @@ __device__ __forceinline__ void factor(const System y, int D) {
 template <int LR, int RPL, int TEAM, bool F32F>
 __device__ __forceinline__ void solve_rhs(const SolveDfParams& prm, const System y, int r0) {
   constexpr int EPT = (KC * LR * RPL + TEAM - 1) / TEAM;   // chunk entries per thread
-  using SH = Shared<TEAM, F32F>;
+  using SH = Shared<TEAM, F32F, square<LR, RPL>()>;
   extern __shared__ float4 smdf[];
   const int D = prm.D, C = prm.C, refine_steps = prm.refine_steps;
   const bool sep = prm.sep != 0;
@@ -586,20 +596,39 @@ __device__ __forceinline__ void solve_rhs(const SolveDfParams& prm, const System
     // x = b - Rl u
 #pragma unroll
     for (int q = 0; q < RPL; ++q) x[q] = b_at(li + LR * q);
-    auto columns = [&](const float4* a, int l0, int n) {   // columns l0 .. l0 + n - 1 at a
+    // columns l0 .. l0 + n - 1 at a, pitch D + 1; rows past D: never read
+    auto columns = [&](const float4* a, int l0, int n) {
       for (int ll = 0; ll < n; ++ll) {
         const float4 u = Ur[l0 + ll];
         const float4* al = a + ll * (D + 1) + li;
 #pragma unroll
         for (int q = 0; q < RPL; ++q)
-          if (LR * q < D) cms(x[q], al[LR * q], u);   // rows past D: never read
+          if (LR * q < D) cms(x[q], al[LR * q], u);
       }
 #pragma unroll
       for (int q = 0; q < RPL; ++q) norm(x[q]);
     };
-    if constexpr (SH::FULL) {
+    if constexpr (SH::FULL && square<LR, RPL>()) {
       __syncwarp();                                // the U rows are written
       for (int l0 = 0; l0 < D; l0 += KC) columns(As + l0 * (D + 1), l0, min(KC, D - l0));
+    } else if constexpr (SH::FULL) {
+      __syncwarp();
+      // column l: rows i >= l lie at cstart(l) - l + i, above the diagonal the
+      // conjugates of row l at cstart(i) - i + l
+      for (int l = 0; l < D; ++l) {
+        const float4 u = Ur[l];
+        const int below = cstart(l, D) - l;
+#pragma unroll
+        for (int q = 0; q < RPL; ++q) {
+          const int i = min(li + LR * q, D - 1);
+          const bool low = i >= l;
+          const float4 a = As[low ? below + i : cstart(i, D) - i + l];
+          cms(x[q], low ? a : conj4(a), u);
+        }
+        if (l % KC == KC - 1 || l == D - 1)
+#pragma unroll
+          for (int q = 0; q < RPL; ++q) norm(x[q]);
+      }
     } else {
       // entry f of the chunk at column l0: column l0 + f % KC, row f / KC; the
       // next chunk's entries wait in registers
@@ -764,7 +793,7 @@ __device__ __forceinline__ void solve_df_body(const SolveDfParams& prm, long lon
   const int tt = team_thread<TEAM>();
   System y;
   y.nu = sep ? prm.C : PASS;
-  const Shared<TEAM, F32F> sh(D, y.nu);
+  const Shared<TEAM, F32F, square<LR, RPL>()> sh(D, y.nu);
   y.off = team * sh.bytes;
   y.aext = nsys * (long long)D * D;
   const int* okf = reinterpret_cast<const int*>(reinterpret_cast<char*>(smdf) + y.off + sh.ok);
@@ -785,7 +814,7 @@ __device__ __forceinline__ void solve_df_body(const SolveDfParams& prm, long lon
     const int et = (int)(((uint32_t)__double2hiint(tr) >> 20) & 0x7FF);
     const int e = et == 0 || et == 0x7FF ? 0 : (et - 1023) & ~1;
     y.sbase = 896 + e;
-    factor<TEAM, F32F>(y, D);
+    factor<TEAM, F32F, square<LR, RPL>()>(y, D);
     const bool ok = *okf != 0;
     const int nrhs = sep ? prm.C : prm.S;
     for (int r0 = 0; r0 < nrhs; r0 += PASS) {
@@ -801,7 +830,7 @@ __device__ __forceinline__ void solve_df_body(const SolveDfParams& prm, long lon
 
 constexpr int cta_threads(int team) { return team > 32 ? team : 128; }
 // CTAs per SM that the registers must allow (shared memory allows about as many)
-constexpr int min_ctas(int team) { return team == 512 ? 1 : (team == 256 ? 3 : (team == 64 ? 12 : 6)); }
+constexpr int min_ctas(int team) { return team == 512 ? 1 : (team == 256 ? 3 : (team == 128 ? 6 : (team == 64 ? 12 : 6))); }
 
 template <int LR, int RPL, int TEAM, bool F32F>
 __global__ void __launch_bounds__(cta_threads(TEAM), min_ctas(TEAM))
@@ -823,8 +852,8 @@ cudaError_t launch_df(SolveDfParams p, cudaStream_t s) {
   constexpr int PASS = TEAM / LR;
   constexpr size_t kMaxSmem = 227 * 1024;
   // the basis form keeps all C solutions in shared memory
-  if (p.sep && Shared<TEAM, F32F>(p.D, p.C).bytes > (int)kMaxSmem) p.sep = p.sym = 0;
-  const size_t tb = Shared<TEAM, F32F>(p.D, p.sep ? p.C : PASS).bytes;
+  if (p.sep && Shared<TEAM, F32F, square<LR, RPL>()>(p.D, p.C).bytes > (int)kMaxSmem) p.sep = p.sym = 0;
+  const size_t tb = Shared<TEAM, F32F, square<LR, RPL>()>(p.D, p.sep ? p.C : PASS).bytes;
   int threads = TEAM;
   if (TEAM <= 32) {
     // several teams per CTA; with few systems one warp per CTA, so that they

@@ -89,6 +89,16 @@ def test_weights_match_64_bit_solutions(C, T, S, solver, refine):
         _check(w, ref if steer is None else _reference(R, steer, 1e-3))
 
 
+@pytest.mark.parametrize("C,T", [(4, 2), (3, 3), (5, 2), (4, 3)])
+def test_many_small_systems_take_half_a_warp_each(C, T):
+    """From 2048 systems of up to 12 rows on, an odd number of teams included."""
+    R = _covariances(8 * 257, C * T, seed=C)
+    for S in (3, 16):
+        w, status = _solve(R, C, T, S)
+        assert status == (stap.STAP_OK, 0)
+        _check(w, _reference(R, _default_steering(C, T, S), 1e-3))
+
+
 @pytest.mark.parametrize("scale", [2.0 ** -600, 1e-40, 3e-20, 1e30, 2.0 ** 600])
 def test_any_power_of_the_input_scale_gives_the_same_weights(scale):
     """Floats span 2^+-126: the system's scale is taken out of the matrix and
