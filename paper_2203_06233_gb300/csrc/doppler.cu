@@ -38,8 +38,41 @@ __host__ __device__ constexpr int bitrev(int x, int bits) {
   return r;
 }
 
+// a b, with the FMAs as the compiler contracts the plain product in the
+// 32-point transform: the split second pass then gives its bits (the
+// tensor-core covariance of the mixed precisions amplifies any other rounding
+// of the transform far above it)
+struct SplitMul {
+  __device__ __forceinline__ float2 operator()(float2 a, float2 b) const {
+    return make_float2(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x)));
+  }
+};
+struct PlainMul {
+  __device__ __forceinline__ float2 operator()(float2 a, float2 b) const { return cmulf(a, b); }
+};
+
+// The butterfly stages of an in-register radix-2 FFT of length N on
+// bit-reversed input.  tw[m] = W_K^m; W_N^j = tw[j * (K / N)].
+template <int N, int K, class Mul = PlainMul>
+__device__ __forceinline__ void fft_stages(float2 (&v)[N], const float2* __restrict__ tw) {
+#pragma unroll
+  for (int len = 2; len <= N; len <<= 1) {
+    const int half = len >> 1;
+#pragma unroll
+    for (int j = 0; j < half; ++j) {
+      const float2 w = tw[j * (K / len)];
+#pragma unroll
+      for (int st = 0; st < N; st += len) {
+        const float2 a = v[st + j];
+        const float2 b = (j == 0) ? v[st + j + half] : Mul()(v[st + j + half], w);
+        v[st + j] = make_float2(a.x + b.x, a.y + b.y);
+        v[st + j + half] = make_float2(a.x - b.x, a.y - b.y);
+      }
+    }
+  }
+}
+
 // In-register radix-2 FFT of length N (forward, natural order in and out).
-// tw[m] = W_K^m; W_N^j = tw[j * (K / N)].
 template <int N, int K>
 __device__ __forceinline__ void fft_reg(float2 (&v)[N], const float2* __restrict__ tw) {
   constexpr int LOGN = ilog2c(N);
@@ -52,23 +85,24 @@ __device__ __forceinline__ void fft_reg(float2 (&v)[N], const float2* __restrict
       v[j] = t;
     }
   }
-#pragma unroll
-  for (int len = 2; len <= N; len <<= 1) {
-    const int half = len >> 1;
-#pragma unroll
-    for (int j = 0; j < half; ++j) {
-#pragma unroll
-      for (int st = 0; st < N; st += len) {
-        const float2 a = v[st + j];
-        float2 b = v[st + j + half];
-        if (4 * j == len) b = make_float2(b.y, -b.x);          // W_4 = -i
-        else if (j != 0) b = cmulf(b, tw[j * (K / len)]);
-        v[st + j] = make_float2(a.x + b.x, a.y + b.y);
-        v[st + j + half] = make_float2(a.x - b.x, a.y - b.y);
-      }
-    }
-  }
+  fft_stages<N, K>(v, tw);
 }
+
+// Shared-memory layout of the transpose: row n1 (N2 + PAD) + k2 of TR columns.
+// With 8 columns (64 bytes) a warp of pass A writes four rows N2 apart, on
+// the same half of the banks without the pad row.
+template <int LOGK, int TR>
+struct Rows {
+  static constexpr int N1 = 1 << ((LOGK + 1) / 2), N2 = 1 << (LOGK / 2);
+  static constexpr int PITCH = N2 + (TR == 8 && N2 > 1 ? 1 : 0);
+  // The second pass in two steps (K = 512: 32 points, which in registers leave
+  // room for two CTAs per SM, half of whose threads have no second pass; C32
+  // P512 R4096: 315 -> 231 us, 4.6 TB/s of the cube and the result.  A three-pass
+  // 8 x 8 x 8 form took 245)
+  static constexpr bool SPLIT = N1 == 32 && N2 == 16;
+  // CTAs per SM that the registers must allow
+  static constexpr int MINB = SPLIT && TR == 8 ? 4 : 0;   // (0: no say)
+};
 
 // Parameters of one launch (one CPI): grid gx = ceil(R / TR) range tiles by
 // C * TW rows.
@@ -93,7 +127,8 @@ __device__ __forceinline__ void doppler_body(const DopplerParams& prm, int bx, i
   constexpr int N2 = 1 << (LOGK / 2);
   extern __shared__ float2 smem[];
   float2* tw = smem;        // [K]
-  float2* Y = smem + K;     // [N1][N2][TR]
+  constexpr int PITCH = Rows<LOGK, TR>::PITCH;
+  float2* Y = smem + K;     // [N1][PITCH][TR]
 
   const int tid = threadIdx.x;
   const int c = by / TW, t = by - c * TW;   // channel, sub-window
@@ -126,18 +161,62 @@ __device__ __forceinline__ void doppler_body(const DopplerParams& prm, int bx, i
 #pragma unroll
     for (int k2 = 0; k2 < N2; ++k2) {
       const float2 y = (k2 == 0) ? v[k2] : cmulf(v[k2], tw[n1 * k2]);
-      Y[(n1 * N2 + k2) * TR + col] = y;
+      Y[(n1 * PITCH + k2) * TR + col] = y;
     }
   }
   __syncthreads();
 
+  if constexpr (Rows<LOGK, TR>::SPLIT) {
+    // ---- pass B in two steps, the same butterflies on the same values as the
+    // 32-point transform in registers (so the same bits): of the bit-reversed
+    // input, positions 8 q .. 8 q + 7 are the rows n1 = 4 rev3(i) + rev2(q); their
+    // three stages first, in place (position i in row 4 i + rev2(q)), then for
+    // each position j the last two stages over q.
+    constexpr int GT = N1;                           // groups of TR threads
+    const int col = tid % TR, r = r0 + col;
+    for (int g = tid / TR; g < 4 * N2; g += GT) {
+      const int k2 = g % N2, q = g / N2, rq = ((q & 1) << 1) | (q >> 1);
+      float2 v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = Y[((4 * bitrev(i, 3) + rq) * PITCH + k2) * TR + col];
+      fft_stages<8, K, SplitMul>(v, tw);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) Y[((4 * i + rq) * PITCH + k2) * TR + col] = v[i];
+    }
+    __syncthreads();
+    float2* dst = dop + ((size_t)t * C + c) * K * ldr + r;
+    for (int g = tid / TR; g < 8 * N2; g += GT) {
+      const int k2 = g % N2, j = g / N2;
+      float2 a[4];                                   // positions j + 8 q
+#pragma unroll
+      for (int q = 0; q < 4; ++q) a[q] = Y[((4 * j + (((q & 1) << 1) | (q >> 1))) * PITCH + k2) * TR + col];
+      auto fly = [&](float2& x, float2& y, int m, bool one) {   // x, y <- x + W^m y, x - W^m y
+        const float2 b = one ? y : SplitMul()(y, tw[m]);
+        y = make_float2(x.x - b.x, x.y - b.y);
+        x = make_float2(x.x + b.x, x.y + b.y);
+      };
+      fly(a[0], a[1], j * (K / 16), j == 0);
+      fly(a[2], a[3], j * (K / 16), j == 0);
+      fly(a[0], a[2], j * (K / 32), j == 0);
+      fly(a[1], a[3], (j + 8) * (K / 32), false);
+      if (r < R)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int k = k2 + N2 * (j + 8 * q);
+          if (in_bounds(((long long)t * C + c) * K * ldr + r + (long long)k * ldr,
+                        ((long long)C * TW * K - 1) * ldr + R, kSiteDopplerOut))
+            dst[(size_t)k * ldr] = a[q];
+        }
+    }
+    return;
+  }
   // ---- pass B: thread (col, k2), N1-point FFT over n1 ----
   if (tid < TR * N2) {
     const int col = tid % TR, k2 = tid / TR;
     const int r = r0 + col;
     float2 u[N1];
 #pragma unroll
-    for (int n1 = 0; n1 < N1; ++n1) u[n1] = Y[(n1 * N2 + k2) * TR + col];
+    for (int n1 = 0; n1 < N1; ++n1) u[n1] = Y[(n1 * PITCH + k2) * TR + col];
     fft_reg<N1, K>(u, tw);
     if (r < R) {
       float2* dst = dop + ((size_t)t * C + c) * K * ldr + r;
@@ -150,139 +229,15 @@ __device__ __forceinline__ void doppler_body(const DopplerParams& prm, int bx, i
   }
 }
 
-// Long transforms (K >= 512) in three passes of 8 and 16 points, K = N1 N2 N3:
-//   n = n1 + N1 (n2 + N2 n3),  k = k3 + N3 (k2 + N2 k1),
-//   pass 1: sum over n3, times W_K^{N1 n2 k3};  pass 2: sum over n2, times
-//   W_K^{n1 (k3 + N3 k2)};  pass 3: sum over n1.
-// The two-pass form needs 32 points in registers here (86 of them: two
-// 256-thread CTAs per SM, half of whose threads have no second pass); eight
-// points leave room for three times the warps (TR = 8: one butterfly per
-// thread and pass), which a transform that streams its input from HBM needs
-// more than it minds the second trip through shared memory.  Pass 2 replaces
-// its inputs in place.  K 512, C32 P512 R4096: 315 -> 246 us (4.4 TB/s of the
-// cube and the result; 16 cells per CTA 261); K 1024, C8 P1000 R4096: 181 -> 150
-// (16 cells 171).
 template <int LOGK, int TR>
-struct Long {
-  static constexpr int K = 1 << LOGK, N3 = 8, N2 = 8, N1 = K / 64;
-  static constexpr int THREADS = 512;
-  static constexpr int MINB = LOGK == 9 && TR == 8 ? 3 : 2;   // CTAs per SM that the registers allow
-  // one more row of TR columns per N3 rows where a warp's pass-1 writes (four
-  // groups of N3 rows) would otherwise meet on half the banks
-  static constexpr int PAD = TR == 8 ? 1 : 0;
-  static constexpr int ROWS = K + PAD * (K / N3);
-  __device__ static int row(int s) { return s + PAD * (s / N3); }   // s = (n1 N2 + n2) N3 + k3
-};
-
-template <int LOGK, int TR>
-__device__ __forceinline__ void doppler_long_body(const DopplerParams& prm, int bx, int by) {
-  using G = Long<LOGK, TR>;
-  constexpr int K = G::K, N1 = G::N1, N2 = G::N2, N3 = G::N3, GT = G::THREADS / TR;
-  const float2* __restrict__ cube = prm.cube;
-  float2* __restrict__ dop = prm.dop;
-  const float* __restrict__ win = prm.win;
-  const int P = prm.P, R = prm.R, ldr = prm.ldr, C = prm.C, TW = prm.TW, PW = prm.PW;
-  extern __shared__ float2 smem[];
-  float2* tw = smem;        // [K]
-  float2* Y = smem + K;     // [ROWS][TR]
-  const int tid = threadIdx.x, col = tid % TR, g0 = tid / TR;
-  const int c = by / TW, t = by - c * TW;   // channel, sub-window
-  const int r = bx * TR + col;
-  for (int m = tid; m < K; m += G::THREADS) tw[m] = prm.tw[m];
-  __syncthreads();
-  const float2* src = cube + (size_t)c * P * ldr + r;
-#pragma unroll (TR == 8 ? 1 : 2)
-  for (int g = g0; g < N1 * N2; g += GT) {         // g = n1 + N1 n2
-    const int n1 = g % N1, n2 = g / N1;
-    float2 v[N3];
-#pragma unroll
-    for (int n3 = 0; n3 < N3; ++n3) {
-      const int n = g + N1 * N2 * n3;
-      float2 x = make_float2(0.f, 0.f);
-      if (r < R && n >= t && n < t + PW &&
-          in_bounds((long long)c * P * ldr + r + (long long)n * ldr, (long long)(C * P - 1) * ldr + R,
-                    kSiteDopplerIn)) {
-        x = __ldg(src + (size_t)n * ldr);
-        const float h = __ldg(win + (n - t));
-        x.x *= h;
-        x.y *= h;
-      }
-      v[n3] = x;
-    }
-    fft_reg<N3, K>(v, tw);
-#pragma unroll
-    for (int k3 = 0; k3 < N3; ++k3)
-      Y[G::row((n1 * N2 + n2) * N3 + k3) * TR + col] = k3 == 0 ? v[0] : cmulf(v[k3], tw[N1 * n2 * k3]);
-  }
-  __syncthreads();
-#pragma unroll (TR == 8 ? 1 : 2)
-  for (int g = g0; g < N1 * N3; g += GT) {         // g = n1 N3 + k3
-    const int n1 = g / N3, k3 = g % N3;
-    float2 v[N2];
-#pragma unroll
-    for (int n2 = 0; n2 < N2; ++n2) v[n2] = Y[G::row((n1 * N2 + n2) * N3 + k3) * TR + col];
-    fft_reg<N2, K>(v, tw);
-#pragma unroll
-    for (int k2 = 0; k2 < N2; ++k2)
-      Y[G::row((n1 * N2 + k2) * N3 + k3) * TR + col] = cmulf(v[k2], tw[n1 * (k3 + N3 * k2)]);
-  }
-  __syncthreads();
-  float2* dst = dop + ((size_t)t * C + c) * K * ldr + r;
-#pragma unroll (TR == 8 ? 1 : 2)
-  for (int g = g0; g < N2 * N3; g += GT) {         // g = k3 + N3 k2
-    float2 v[N1];
-#pragma unroll
-    for (int n1 = 0; n1 < N1; ++n1) v[n1] = Y[G::row(n1 * N2 * N3 + g) * TR + col];
-    fft_reg<N1, K>(v, tw);
-    if (r < R)
-#pragma unroll
-      for (int k1 = 0; k1 < N1; ++k1)
-        if (in_bounds(((long long)t * C + c) * K * ldr + r + (long long)(g + N2 * N3 * k1) * ldr,
-                      ((long long)C * TW * K - 1) * ldr + R, kSiteDopplerOut))
-          dst[(size_t)(g + N2 * N3 * k1) * ldr] = v[k1];
-  }
-}
-
-template <int LOGK, int TR>
-__global__ void __launch_bounds__(512, Long<LOGK, TR>::MINB)
-doppler_long_kernel(DopplerParams p) {
-  doppler_long_body<LOGK, TR>(p, blockIdx.x, blockIdx.y);
-}
-
-template <int LOGK, int TR>
-__global__ void __launch_bounds__(512, Long<LOGK, TR>::MINB)
-doppler_long_batched(BatchCtl ctl) {
-  batched_loop<DopplerParams>(ctl, [&](const DopplerParams& p, int bx, int by, int) {
-    doppler_long_body<LOGK, TR>(p, bx, by);
-  });
-}
-
-template <int LOGK, int TR>
-cudaError_t launch_long(const float2* cube, float2* dop, const float* win, const float2* tw, int C,
-                        int TW, int P, int R, int ldr, cudaStream_t s) {
-  using G = Long<LOGK, TR>;
-  const size_t smem = (size_t)(G::K + G::ROWS * TR) * sizeof(float2);
-  if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  static int set_bytes[64] = {0}, set_bytes_b[64] = {0};
-  cudaError_t e = ensure_smem(doppler_long_kernel<LOGK, TR>, smem, set_bytes);
-  if (e == cudaSuccess) e = ensure_smem(doppler_long_batched<LOGK, TR>, smem, set_bytes_b);
-  if (e != cudaSuccess) return e;
-  dim3 grid((R + TR - 1) / TR, C * TW);
-  const DopplerParams p{cube, dop, win, tw, P, R, ldr, C, TW, P - TW + 1, (int)grid.x};
-  return launch_params(reinterpret_cast<const void*>(doppler_long_kernel<LOGK, TR>),
-                       reinterpret_cast<const void*>(doppler_long_batched<LOGK, TR>), grid, G::THREADS,
-                       smem, s, p);
-}
-
-template <int LOGK, int TR>
-__global__ void __launch_bounds__(TR * (1 << ((LOGK + 1) / 2)))
+__global__ void __launch_bounds__(TR * (1 << ((LOGK + 1) / 2)), Rows<LOGK, TR>::MINB)
 doppler_fft_kernel(DopplerParams p) {
   doppler_body<LOGK, TR>(p, blockIdx.x, blockIdx.y);
 }
 
 // the same transform as a persistent launch over the CPIs of a batch
 template <int LOGK, int TR>
-__global__ void __launch_bounds__(TR * (1 << ((LOGK + 1) / 2)))
+__global__ void __launch_bounds__(TR * (1 << ((LOGK + 1) / 2)), Rows<LOGK, TR>::MINB)
 doppler_fft_batched(BatchCtl ctl) {
   batched_loop<DopplerParams>(ctl, [&](const DopplerParams& p, int bx, int by, int) {
     doppler_body<LOGK, TR>(p, bx, by);
@@ -294,7 +249,7 @@ cudaError_t launch_logk_tr(const float2* cube, float2* dop, const float* win, co
                            int TW, int P, int R, int ldr, cudaStream_t s) {
   constexpr int K = 1 << LOGK;
   constexpr int N1 = 1 << ((LOGK + 1) / 2);
-  const size_t smem = (size_t)K * sizeof(float2) * (1 + TR);
+  const size_t smem = ((size_t)K + (size_t)N1 * Rows<LOGK, TR>::PITCH * TR) * sizeof(float2);
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
   static int set_bytes[64] = {0}, set_bytes_b[64] = {0};
   cudaError_t e = ensure_smem(doppler_fft_kernel<LOGK, TR>, smem, set_bytes);
@@ -313,14 +268,6 @@ cudaError_t launch_logk_tr(const float2* cube, float2* dop, const float* win, co
 template <int LOGK>
 cudaError_t launch_logk(const float2* cube, float2* dop, const float* win, const float2* tw, int C,
                         int TW, int P, int R, int ldr, cudaStream_t s, int tr) {
-  if constexpr (LOGK >= 9) {
-    switch (tr == 0 ? 8 : tr) {
-      case 8: return launch_long<LOGK, 8>(cube, dop, win, tw, C, TW, P, R, ldr, s);
-      case 16: return launch_long<LOGK, 16>(cube, dop, win, tw, C, TW, P, R, ldr, s);
-      case 32: return launch_long<LOGK, 32>(cube, dop, win, tw, C, TW, P, R, ldr, s);
-      default: return cudaErrorInvalidValue;
-    }
-  }
   constexpr int N1 = 1 << ((LOGK + 1) / 2);
   if (tr == 0) tr = N1 >= 16 ? 8 : 32;
   switch (tr) {

@@ -1,4 +1,4 @@
-"""The Doppler transform's long form (K >= 512) at every tile width, and the
+"""The Doppler transform's longest lengths (K = 512 in split passes) at every tile width, and the
 front end's three forms, against 64-bit sums."""
 import numpy as np
 import pytest
