@@ -70,8 +70,10 @@ typedef enum {
  *                about 2^-21 relative to the block's largest magnitude.
  * The tensor-core apply needs B | 128 or 128 | B and at most 256 real weight
  * rows (2 per steering vector and block) per 128-cell tile, and falls back
- * to the FP32 apply otherwise; stap_plan_autotune keeps the FP32 kernel of a
- * step where that is faster (small D). */
+ * to the FP32 apply otherwise; for D <= 24 the FP32 apply -- the more accurate
+ * one -- is the faster and the default (S <= 32; FP16_SCALED: any S).
+ * stap_plan_autotune keeps the FP32 kernel of a step where timing finds it
+ * faster, and stap_plan_set_tuning can name either. */
 typedef enum {
   STAP_PREC_FP32 = 0,        /* FP32 FFT; covariance accumulated error-free in
                                 FP32 pairs (two-product / compensated sum); FP32

@@ -52,7 +52,7 @@
 //   [wr_0, wi_0, wr_1, wi_1, ...] -> Re y,  [-wi_0, wr_0, -wi_1, wr_1, ...] -> Im y.
 // One accumulator; lane m (cell r0 + m) reads the columns of its own block.
 //
-// Pipeline per CTA (256 threads, persistent over tiles): the operand chunk
+// Pipeline per CTA (256 or 512 threads, persistent over tiles): the operand chunk
 // is staged into one of two shared-memory stages (K-major core matrices, no
 // swizzle) by all threads, thread 0 issues the chunk's MMAs and commits them
 // to that stage's mbarrier, and the next chunk is staged into the other
@@ -93,7 +93,12 @@ struct Fmt<kFP16S> {
 __device__ __forceinline__ int prod_a(int i) { return i < 3 ? (i == 2 ? 1 : 0) : (i == 3 ? 0 : (i == 4 ? 1 : 2)); }
 __device__ __forceinline__ int prod_b(int i) { return i < 3 ? (i == 1 ? 1 : 0) : (i == 3 ? 2 : (i == 4 ? 1 : 0)); }
 
-constexpr int kThreads = 256;                 // 8 warps stage; warp w reads TMEM lanes 32 (w % 4) ..
+// Covariance: 16 warps, all of which stage; warp w reads TMEM lanes 32 (w % 4)
+// .. 32 (w % 4) + 31.  The phases of a tile (scale pass, staging, epilogue) wait on
+// memory more than on issue; with 8 warps FP16S took 1115 us instead of 888 at
+// D = 128 (C32 T4 K512 R2048 B256, one CTA per SM) and 521 instead of 467 at D = 64
+// (C16 T4 K256 R4096 B128, two CTAs per SM).
+constexpr int kWarps = 16, kThreads = 32 * kWarps;
 constexpr int kWaitIter = kDefaultWaitPolls;  // drain waits before TMEM is freed
 
 // ---- splitting ---------------------------------------------------------------
@@ -164,7 +169,7 @@ __host__ __device__ constexpr uint32_t idesc_for(int N) {
 // of G = floor(64 / D8) systems, two accumulators of NA <= 64 columns) and
 // split (D8 > 64: four accumulators, 512 columns).  A piece of a stage holds
 // ROWS operand rows of RB bytes (16 KB either way).
-constexpr int kCovU = 8;                      // staging units per warp and chunk (<= 64 units / 8 warps)
+constexpr int kCovU = 64 / kWarps;            // staging units per warp and chunk (at most 64 units)
 constexpr int kCovPiece = 16384;              // bytes of one piece of one stage
 
 template <bool STK>
@@ -180,7 +185,7 @@ template <int PREC>
 constexpr size_t cov_smem() { return 2 * (size_t)Fmt<PREC>::NPC * kCovPiece; }
 
 template <int PREC, bool STK>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kThreads, STK ? 2 : 1)
 covariance_tcx_kernel(const float2* __restrict__ dop, double2* __restrict__ cov, int C, int K,
                       int ldr, int T, int B, int NB, int D8, int G, long long ntiles, int lower_only,
                       DeviceStatus* __restrict__ status, int wait_polls) {
@@ -267,10 +272,10 @@ covariance_tcx_kernel(const float2* __restrict__ dop, double2* __restrict__ cov,
     // A unit is one core matrix (8 rows x 16 bytes) of the Xr rows and the
     // matching one of the Xi rows; lane l takes row 8 rg + l/4 and CPL cells
     // and writes one 32-bit word per piece into each.  Warp w takes units
-    // w, w + 8, ... (at most kCovU of them).  The next chunk's loads are
+    // w, w + kWarps, ... (at most kCovU of them).  The next chunk's loads are
     // issued before this chunk's barrier and MMAs, so their latency overlaps
     // both.
-    // Per tile, each lane's unit uu covers row (warp + 8 uu) / NCM * 8 + l/4
+    // Per tile, each lane's unit uu covers row (warp + kWarps uu) / NCM * 8 + l/4
     // (its dop offset and, for FP16S, its system's scale fetched here once)
     // and the same cells of every chunk ((warp % NCM) CPW + (l & 3) CPL on).
     long long rbase[kCovU];
@@ -396,7 +401,7 @@ covariance_tcx_kernel(const float2* __restrict__ dop, double2* __restrict__ cov,
     if (!ok) break;
     tc::fence_after_sync();
     // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 (rows i of the
-    // tile); warps w and w + 4 take alternate column blocks of 8
+    // tile); warps w, w + 4, ... take alternate column blocks of 8
     const int q4 = warp & 3, hf = warp >> 2;
     const uint32_t lb = (uint32_t)(q4 * 32) << 16;
     const float invB = 1.f / (float)B;
@@ -411,7 +416,7 @@ covariance_tcx_kernel(const float2* __restrict__ dop, double2* __restrict__ cov,
         const int ii = q4 * 32 + lane - GD;
         const bool xi = ii >= 0 && ii < GD;
         const int g = xi ? ii / D8 : 0, a = ii - g * D8;
-        for (int cb = hf * 8; cb < NA; cb += 16) {
+        for (int cb = hf * 8; cb < NA; cb += 2 * kWarps) {
           float x0[8], x1[8];
           in_bounds(NA + cb + 7, Fm::COLS, kSiteTcTmem);   // recorded only
           tc::tmem_ld8x2(tmem + lb + cb, tmem + lb + NA + cb, x0, x1);
@@ -439,7 +444,7 @@ covariance_tcx_kernel(const float2* __restrict__ dop, double2* __restrict__ cov,
       const int gw0 = (q4 * 32) / D8;
       const int gw1 = min(G - 1, (q4 * 32 + 31) / D8);
       for (int gg = gw0; gg <= gw1; ++gg) {
-        for (int cb = hf * 8; cb < D8; cb += 16) {   // warp-uniform bounds
+        for (int cb = hf * 8; cb < D8; cb += 2 * kWarps) {   // warp-uniform bounds
           // one system per tile: a block of columns left of the warp's first
           // row has no l >= a entry
           if (G == 1 && cb + 8 <= q4 * 32) continue;
@@ -507,14 +512,15 @@ covariance_tcx_kernel(const float2* __restrict__ dop, double2* __restrict__ cov,
 constexpr int kAppRB = 64;                    // bytes of one operand row per chunk (4 core matrices)
 constexpr int kAppA = 128 * kAppRB;           // A piece: 128 cells (8 KB)
 constexpr int kAppB = 256 * kAppRB;           // B piece: at most 256 weight rows (16 KB)
-constexpr int kAppU = 16;                     // staging units per warp and chunk: (64 A + at most 64 B units) / 8 warps
 
 // two stages of the pieces of 128 cell rows and NP weight rows
 template <int PREC>
 constexpr size_t apply_smem(int NP) { return 2 * (size_t)Fmt<PREC>::NPC * (kAppA + (size_t)NP * kAppRB); }
 
-template <int PREC>
-__global__ void __launch_bounds__(kThreads, 2)   // two CTAs per SM (TMEM <= 256 columns each)
+// NW warps per CTA: 8, of which two CTAs or more share an SM and overlap their
+// phases, or 16 in one CTA (launch_app chooses)
+template <int PREC, int NW>
+__global__ void __launch_bounds__(32 * NW, NW == 8 ? 2 : 1)
 apply_tcx_kernel(const float2* __restrict__ dop, const float2* __restrict__ wts,
                  float* __restrict__ out, int C, int K, int R, int ldr, int T, int B, int S, int NB,
                  int NP, int tmem_cols, long long ntiles, DeviceStatus* __restrict__ status,
@@ -546,7 +552,7 @@ apply_tcx_kernel(const float2* __restrict__ dop, const float2* __restrict__ wts,
   // weight element written to the vector's two rows
   const int unitsA = 16 * NCM, units = unitsA + (NP / 8) * (NCM / 2);
 
-  for (int i = tid; i < 2 * STAGE / 4; i += kThreads) reinterpret_cast<uint32_t*>(sm)[i] = 0u;
+  for (int i = tid; i < 2 * STAGE / 4; i += (32 * NW)) reinterpret_cast<uint32_t*>(sm)[i] = 0u;
   if (warp == 0) tc::tmem_alloc(&tmem_base, tmem_cols);
   if (tid == 0) {
     tc::mbar_init(&mbar[0], 1);
@@ -572,15 +578,15 @@ apply_tcx_kernel(const float2* __restrict__ dop, const float2* __restrict__ wts,
     }
     {
       const int q = tid >> 1, j = q / S, s = q - j * S;
-      wbase[tid] = (tid < NP && q < Nq && b0 + j < NB) ? ((((long long)k * NB + b0 + j) * S + s) * D) : -1;
+      if (tid < 256) wbase[tid] = (tid < NP && q < Nq && b0 + j < NB) ? ((((long long)k * NB + b0 + j) * S + s) * D) : -1;
     }
     if (PREC == kFP16S && tid == 0) xmax = 0;
     __syncthreads();
     if constexpr (PREC == kFP16S) {   // the tile's largest |x| component, each vector's largest |w|
       float m = 0.f;
       const int rn = min(128, R - r0);
-#pragma unroll 8
-      for (int e = tid; e < D * 128; e += kThreads) {   // entry d = e / 128 of cell e % 128
+#pragma unroll 16
+      for (int e = tid; e < D * 128; e += (32 * NW)) {   // entry d = e / 128 of cell e % 128
         const int d = e >> 7, mm = e & 127;
         if (mm < rn) {
           const float2 v = __ldg(dop + colbase[d] + r0 + mm);
@@ -589,7 +595,7 @@ apply_tcx_kernel(const float2* __restrict__ dop, const float2* __restrict__ wts,
       }
       m = warp_max(m);
       if (lane == 0) atomicMax(&xmax, __float_as_int(m));
-      for (int q = warp; q < Nq; q += kThreads / 32) {
+      for (int q = warp; q < Nq; q += (32 * NW) / 32) {
         const long long wb = wbase[2 * q];
         float mw = 0.f;
         if (wb >= 0)
@@ -613,15 +619,15 @@ apply_tcx_kernel(const float2* __restrict__ dop, const float2* __restrict__ wts,
     // one 8-row group: lane l takes weight vector 4 rg + (l / 4) % 4 and word
     // l & 3 of both its rows, [wr, wi] (even) and [-wi, wr] (odd), from one
     // load and one split (pieces of -x are minus those of x).  Warp w takes
-    // units w, w + 8, ... (at most kAppU); the next chunk's loads are issued
+    // units w, w + 8, ... (at most 128 / NW); the next chunk's loads are issued
     // before this chunk's barrier and MMAs.
     // With NCM = 4 the 64 A units are units 0-63: warp w's unit uu < 8 is
     // row group (w >> 2) + 2 uu, core matrix w & 3.  Its B unit vb (unit
     // 64 + w + 8 vb) is row group (w >> 1) + 4 vb, core matrices 2 (w & 1) + h.
     // Row offsets, weight-vector offsets and scales are fixed per tile; the
     // snapshot entry and the weight element per chunk.
-    static_assert(NCM == 4 && kAppU == 16, "unit layout");
-    constexpr int kAU = 8, kBU = kAppU - kAU;
+    static_assert(NCM == 4 && NW % 4 == 0, "unit layout");
+    constexpr int kAU = 64 / NW, kBU = 64 / NW;
     const int unitsB = units - unitsA;
     const int cmA = warp & 3, h = lane >> 4, q4 = (lane >> 2) & 3;
     const int cmB = 2 * (warp & 1) + h;
@@ -629,12 +635,12 @@ apply_tcx_kernel(const float2* __restrict__ dop, const float2* __restrict__ wts,
     float wscq[kBU];
 #pragma unroll
     for (int vb = 0; vb < kBU; ++vb) {
-      const int ub = warp + 8 * vb;
-      const int q = ((warp >> 1) + 4 * vb) * 4 + q4;
+      const int ub = warp + NW * vb;
+      const int q = ((warp >> 1) + NW / 2 * vb) * 4 + q4;
       wbq[vb] = ub < unitsB ? wbase[2 * q] : -1;
       wscq[vb] = (PREC == kFP16S && ub < unitsB && q < Nq) ? wsc[q] : 1.f;
     }
-    float2 v[kAppU];
+    float2 v[kAU + kBU];
     auto load_chunk = [&](int ch) {
       const int kap0 = ch * KC;
       const int dA = PREC == kTF32X3 ? (kap0 + cmA * 4 + (lane & 3)) >> 1 : (kap0 + cmA * 8 + (lane & 3) * 2) >> 1;
@@ -642,7 +648,7 @@ apply_tcx_kernel(const float2* __restrict__ dop, const float2* __restrict__ wts,
       const long long baseA = dA < D ? colbase[dA] + r0 : -1;
 #pragma unroll
       for (int uu = 0; uu < kAU; ++uu) {
-        const int row = (warp >> 2) * 8 + 16 * uu + (lane >> 2);
+        const int row = ((warp >> 2) + NW / 4 * uu) * 8 + (lane >> 2);
         v[uu] = (baseA >= 0 && r0 + row < R &&
                  in_bounds(baseA + row, ((long long)C * K - 1) * ldr + R, kSiteTcIn))
                     ? __ldg(dop + baseA + row) : make_float2(0.f, 0.f);
@@ -671,7 +677,7 @@ apply_tcx_kernel(const float2* __restrict__ dop, const float2* __restrict__ wts,
 #pragma unroll
       for (int uu = 0; uu < kAU; ++uu) {   // A: cell rows
         const float2 e = v[uu];
-        const int off = ((warp >> 2) + 2 * uu) * SBO + cmA * 128 + (lane >> 2) * 16 + (lane & 3) * 4;
+        const int off = ((warp >> 2) + NW / 4 * uu) * SBO + cmA * 128 + (lane >> 2) * 16 + (lane & 3) * 4;
         if (!in_bounds(off + 3, kAppA, kSiteTcSmem)) continue;   // the word's last byte
         if constexpr (PREC == kTF32X3) {
           const int kap = kap0 + cmA * 4 + (lane & 3);
@@ -693,9 +699,9 @@ apply_tcx_kernel(const float2* __restrict__ dop, const float2* __restrict__ wts,
       }
 #pragma unroll
       for (int vb = 0; vb < kBU; ++vb) {   // B: weight rows
-        if (warp + 8 * vb >= unitsB) continue;
+        if (warp + NW * vb >= unitsB) continue;
         const float2 e = v[kAU + vb];
-        const int rg = (warp >> 1) + 4 * vb;
+        const int rg = (warp >> 1) + NW / 2 * vb;
         const int offE = kAppA + rg * SBO + cmB * 128 + (2 * q4) * 16 + (lane & 3) * 4;
         const int offO = offE + 16;   // the odd row of the same vector
         if (!in_bounds(offO + 3, PIECE, kSiteTcSmem)) continue;
@@ -783,7 +789,7 @@ apply_tcx_kernel(const float2* __restrict__ dop, const float2* __restrict__ wts,
         // blocks of 8 columns starting on a multiple of 8 (column 2 jj S is
         // even, so a (Re, Im) pair never straddles two blocks)
         const int c_lo = 2 * jj * S, c_hi = c_lo + 2 * S;
-        for (int cb = (c_lo & ~7) + hf * 8; cb < c_hi; cb += 16) {   // warp-uniform bounds
+        for (int cb = (c_lo & ~7) + hf * 8; cb < c_hi; cb += 2 * NW) {   // warp-uniform bounds
           float a[8];
           in_bounds(cb + 7, tmem_cols, kSiteTcTmem);   // recorded only
           tc::tmem_ld8(tmem + lb + cb, a);
@@ -855,8 +861,8 @@ cudaError_t launch_cov(const float2* dop, double2* cov, int C, int K, int R, int
   return launch_cov_form<PREC, false>(dop, cov, C, K, R, ldr, T, B, lower_only, status, s, wait_polls);
 }
 
-template <int PREC>
-cudaError_t launch_app(const float2* dop, const float2* wts, float* out, int C, int K, int R, int ldr,
+template <int PREC, int NW>
+cudaError_t launch_app_nw(const float2* dop, const float2* wts, float* out, int C, int K, int R, int ldr,
                        int T, int B, int S, DeviceStatus* status, cudaStream_t s, int wait_polls) {
   const int NB = R / B;
   const int nbt = B < 128 ? 128 / B : 1;
@@ -868,20 +874,32 @@ cudaError_t launch_app(const float2* dop, const float2* wts, float* out, int C, 
   const long long ntiles = (long long)K * ((R + 127) / 128);
   const size_t smem = apply_smem<PREC>(NP);
   static int set_bytes[64] = {0};
-  cudaError_t e = ensure_smem(apply_tcx_kernel<PREC>, smem, set_bytes);
+  cudaError_t e = ensure_smem(apply_tcx_kernel<PREC, NW>, smem, set_bytes);
   if (e != cudaSuccess) return e;
   // resident CTAs per SM: registers and shared memory (occupancy query),
   // and no more than the SM's 512 TMEM columns hold
-  int per_sm = resident_ctas(apply_tcx_kernel<PREC>, kThreads, smem);
+  int per_sm = resident_ctas(apply_tcx_kernel<PREC, NW>, 32 * NW, smem);
   if (per_sm > 512 / cols) per_sm = 512 / cols;
   const long long cap = 152LL * per_sm;
   const long long blocks = ntiles < cap ? ntiles : cap;
   return launch_or_defer(s, [=](cudaStream_t st) {
-    apply_tcx_kernel<PREC><<<(unsigned)blocks, kThreads, smem, st>>>(dop, wts, out, C, K, R, ldr, T, B, S,
+    apply_tcx_kernel<PREC, NW><<<(unsigned)blocks, 32 * NW, smem, st>>>(dop, wts, out, C, K, R, ldr, T, B, S,
                                                                    NB, NP, cols, ntiles, status,
                                                                    wait_polls);
     return cudaGetLastError();
   });
+}
+
+template <int PREC>
+cudaError_t launch_app(const float2* dop, const float2* wts, float* out, int C, int K, int R, int ldr,
+                       int T, int B, int S, DeviceStatus* status, cudaStream_t s, int wait_polls) {
+  // FP16S reads a tile twice (its scale first): from D = 64 on, one CTA of 16
+  // warps, whose reads are short of latency hiding, not of other CTAs' phases
+  // (C32 T4 K512 R2048 B256 S64: 1281 us with 8 warps, 1089 with 16; BF16X3 C16 T4
+  // K256 R4096 B128 S32: 320 with 8, 464 with 16)
+  if (PREC == kFP16S && C * T >= 64)
+    return launch_app_nw<PREC, 16>(dop, wts, out, C, K, R, ldr, T, B, S, status, s, wait_polls);
+  return launch_app_nw<PREC, 8>(dop, wts, out, C, K, R, ldr, T, B, S, status, s, wait_polls);
 }
 
 }  // namespace

@@ -299,6 +299,19 @@ stap_status do_doppler(stap_plan p, const Cpi& c, const void* cube, void* dop, c
       d.n_range, st, c.tune));
 }
 
+// Whether a mixed-precision plan's default apply is the (more accurate) FP32
+// kernel: for short snapshots, which fit a thread's registers, while the
+// tensor-core kernel's time is the splitting of the snapshots whatever S is (K
+// 128 R 4096 B 128, FP32 / BF16X3 / TF32X3 / FP16S, us: D = 12 S = 16 30 / 60 / 71 /
+// 96, D = 24 S = 32 87 / 103 / 105 / 208, D = 24 S = 64 155 / 139 / 130 / 278).  Beyond
+// D = 24 the FP32 kernel would win for S <= 8 to 32 by up to a quarter, but the
+// outputs would move by up to a few 1e-5 of their norm, where strong clutter
+// cancels in the filter; the autotuner, which is asked to, still picks it.
+// By the CPI's shape alone: range slabs, batches and single runs agree.
+bool fp32_apply_default(const Cpi& c, int precision) {
+  return c.D <= 24 && (c.d.n_steering <= 32 || precision == STAP_PREC_FP16_SCALED);
+}
+
 // lower: the chain's own buffer, of which the solve reads only the lower
 // triangle (the kernels then skip the upper one)
 stap_status do_covariance(stap_plan p, const Cpi& c, const void* dop, void* cov, cudaStream_t st,
@@ -342,7 +355,7 @@ stap_status do_apply(stap_plan p, const Cpi& c, const void* dop, const void* wts
   const int R = nr < 0 ? d.n_range : nr;
   if (stap::tc_precision(p->opt.precision) &&
       stap::apply_tc_supported(d.training_block, d.n_steering) &&
-      (c.tune.apply_kind == 0 || c.tune.apply_kind == 3))
+      (c.tune.apply_kind == 3 || (c.tune.apply_kind == 0 && !fp32_apply_default(c, p->opt.precision))))
     return check_launch(stap::launch_apply_tc(static_cast<const float2*>(dop),
                                               static_cast<const float2*>(wts), out, c.Cd,
                                               d.n_dop, R, d.n_range, c.Td, d.training_block,
