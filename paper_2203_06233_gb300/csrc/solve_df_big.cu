@@ -8,7 +8,7 @@ cudaError_t launch_solve_df_big(const SolveDfParams& p, cudaStream_t s) {
   if (D <= 48) return launch_df<16, 3, 256, false>(p, s);
   if (D <= 64) return launch_df<16, 4, 256, false>(p, s);
   if (D <= 96) return launch_df<16, 6, 512, false>(p, s);
-  return launch_df<16, 8, 512, false>(p, s);
+  return launch_df<32, 4, 512, false>(p, s);
 }
 
 cudaError_t check_record_solve_df_big(CheckRecord* out) { return read_check_record(out); }

@@ -17,7 +17,14 @@
 // Knuth's TwoSum, every rounding error and the cross terms collected in a
 // second float; the pair is renormalised every LR columns, so the collected
 // errors stay small against the sum.  Relative to the terms' running sums
-// that is about 2^-44, against FP64's 2^-50 over as many terms.
+// that is about 2^-44, against FP64's 2^-50 over as many terms.  Where a bound
+// on the partial sums is known and close, the sum runs on a fixed grid at half
+// the instructions (gmac): from D = 33 on, the factorisation (an entry's sums
+// stay below sqrt(Rl_ii Rl_ll)) and the substitutions' blocks off the diagonal
+// (|x| + max |l| sum |y|, formed per row and block).  Not the residual: its only
+// cheap bound, sqrt(Rl_ii) sum sqrt(Rl_jj) |u_j|, is far above the sums where
+// the solutions of the separable basis cancel (measured: one system in eight
+// 3.6e-6 off instead of 2.9e-8), though it would be a third faster.
 //
 // Where it may stand in for FP64.  The weights are stored as complex64
 // (2^-25), and the solution's relative error is at most kappa(Rl) times the
@@ -47,13 +54,19 @@
 // issued 74% of the slots against 62% for eight warps of 255 with two
 // right-hand sides per thread; packed FP32 pairs (FFMA2) of two right-hand
 // sides, or of real and imaginary part, needed so many moves to form the pairs
-// that they were no faster.
+// that they were no faster.  With the grids a warp per right-hand side is the
+// faster split at D > 96 (2048 systems of 128 rows: half a warp 10230 us, a warp
+// 9470; without grids 10820, 10890), half a warp below (96 rows: 4958, 5540).
 //
-// Measured (GB300; before: the FP64 kernels, after), us:
-//   D = 128, 16384 systems, C 32 S 64    266533 -> 82200
-//   D =  64, 8192 systems,  C 16 S 32     15859 ->  5300
-//   D =  12, 16384 systems, C 4  S 16       324 ->   170
-//   D =  12, 256 systems,   C 4  S 4      103.5 ->  26.5
+// Measured (GB300; the FP64 kernels, double-float without grids, as it is), us:
+//   D = 128, 16384 systems, C 32 S 64    266533, 82470, 71420
+//   D =  64, 8192 systems,  C 16 S 32     15859,  5403,  5234
+//   D =  15, 3840 systems,  C 5  S 11       258,   117 (no grids)
+//   D =  12, 16384 systems, C 4  S 16       324,   160 (no grids)
+//   D =  12, 256 systems,   C 4  S 4      103.5,    21 (no grids)
+// What bounds it at D = 128: 62% of the issue slots in use, half of the rest
+// fixed-latency waits at four warps per scheduler (shared memory holds one
+// system per SM), then shared-memory latency and barriers.
 //
 // F32F (STAP_SOLVE_MIXED_IR): the factor and the substitutions in FP32, the
 // residual and the solution in double-float as above.
@@ -69,6 +82,11 @@ namespace stap {
 namespace {
 
 constexpr int KC = 8;   // columns of Rl per residual chunk
+
+// Whether the factorisation and the substitutions' off-diagonal blocks run on
+// grids: from D = 33 on.
+template <int TEAM, bool F32F>
+__host__ __device__ constexpr bool grids() { return !F32F && TEAM >= 256; }
 
 // One complex value: running sums (rs, is) and the errors collected beside
 // them (re, ie); in shared memory (re hi, im hi, re lo, im lo).
@@ -108,6 +126,48 @@ __device__ __forceinline__ void cms(Cdf& x, float4 l, float4 y) {
   mac(x.is, x.ie, -l.x, -l.z, y.y, y.w);
   mac(x.rs, x.re, l.y, l.w, y.y, y.w);
   mac(x.is, x.ie, -l.y, -l.w, y.x, y.z);
+}
+
+// A sum whose partial sums a bound M is known for runs from sig = 3 P, P the
+// power of two above M, instead of from zero: it stays in (2 P, 4 P), where
+// floats have one spacing, so that t - s and the rest a b - (t - s) are exact
+// and need no TwoSum: 6 instructions instead of 12 per real product.  The error
+// is about 2^-46 of M where it was about 2^-47 of the running sums.
+__device__ __forceinline__ void gmac(float& s, float& e, float ah, float al, float bh, float bl) {
+  const float t = __fmaf_rn(ah, bh, s);
+  float q = __fmaf_rn(ah, bh, __fsub_rn(s, t));
+  q = __fmaf_rn(ah, bl, q);
+  q = __fmaf_rn(al, bh, q);
+  s = t;
+  e = __fadd_rn(e, q);
+}
+__device__ __forceinline__ void gcms(Cdf& x, float4 l, float4 y) {
+  gmac(x.rs, x.re, -l.x, -l.z, y.x, y.z);
+  gmac(x.is, x.ie, -l.x, -l.z, y.y, y.w);
+  gmac(x.rs, x.re, l.y, l.w, y.y, y.w);
+  gmac(x.is, x.ie, -l.y, -l.w, y.x, y.z);
+}
+__device__ __forceinline__ float sigma(float m) {
+  return __fmul_rn(__uint_as_float(__float_as_uint(m) & 0x7F800000u), 6.f);
+}
+// onto sig's grid, the rest of s to e; and back (normalised)
+__device__ __forceinline__ void bias2(float& s, float& e, float sig) {
+  const float t = __fadd_rn(s, sig);
+  e = __fadd_rn(e, __fsub_rn(s, __fsub_rn(t, sig)));
+  s = t;
+}
+__device__ __forceinline__ void unbias2(float& s, float& e, float sig) {
+  norm2(s, e);                       // |e| <= spacing / 2: the difference is 0 or larger
+  s = __fsub_rn(s, sig);
+  norm2(s, e);
+}
+__device__ __forceinline__ void bias(Cdf& x, float sig) {
+  bias2(x.rs, x.re, sig);
+  bias2(x.is, x.ie, sig);
+}
+__device__ __forceinline__ void unbias(Cdf& x, float sig) {
+  unbias2(x.rs, x.re, sig);
+  unbias2(x.is, x.ie, sig);
 }
 
 // a b of two normalised double-floats
@@ -210,8 +270,8 @@ __device__ __forceinline__ double lanes_sum(double v) {
 // visited, with the block indices compile-time constants.  Only the diagonal
 // block decides per lane; rows past D read whatever lies after their column
 // (inside the team's shared memory) into registers that nothing reads.
-template <int LR, int RPL, bool BACK>
-__device__ __forceinline__ void subst(Cdf (&x)[RPL], const float4* L, int D, int li, int gbase) {
+template <int LR, int RPL, bool BACK, bool GRID>
+__device__ __forceinline__ void subst(Cdf (&x)[RPL], const float4* L, const float* lmax, int D, int li, int gbase) {
 #pragma unroll
   for (int bb = 0; bb < RPL; ++bb) {
     const int qb = BACK ? RPL - 1 - bb : bb;
@@ -231,7 +291,7 @@ __device__ __forceinline__ void subst(Cdf (&x)[RPL], const float4* L, int D, int
       const float4* cj = L + cstart(j, D) - j + li;
 #pragma unroll
       for (int q = 0; q < RPL; ++q) {
-        if (BACK ? (q > qb) : (q < qb)) continue;         // compile-time
+        if (GRID ? q != qb : (BACK ? (q > qb) : (q < qb))) continue;   // compile-time
         if (LR * q >= D) continue;                        // team-uniform
         float4 l = make_float4(0.f, 0.f, 0.f, 0.f);
         if (q != qb || (BACK ? li < jo : (li > jo && li + LR * q < D)))
@@ -239,24 +299,62 @@ __device__ __forceinline__ void subst(Cdf (&x)[RPL], const float4* L, int D, int
         cms(x[q], l, pack(y));
       }
     }
+    if constexpr (!GRID) {
 #pragma unroll
-    for (int q = 0; q < RPL; ++q)
-      if (BACK ? q < qb : q > qb) norm(x[q]);
+      for (int q = 0; q < RPL; ++q)
+        if (BACK ? q < qb : q > qb) norm(x[q]);
+    } else if (BACK ? qb > 0 : LR * (qb + 1) < D) {
+      // the block's entries are final: the other rows on a grid whose bound is
+      // |x| + max |l| sum |y|
+      norm(x[qb]);
+      float ys = li < jn ? fabsf(x[qb].rs) + fabsf(x[qb].is) : 0.f;
+#pragma unroll
+      for (int o = LR / 2; o > 0; o >>= 1) ys += __shfl_xor_sync(0xffffffffu, ys, o);
+      ys *= 1.001f;
+      float sig[RPL];
+#pragma unroll
+      for (int q = 0; q < RPL; ++q) {
+        if (BACK ? q >= qb : q <= qb) continue;
+        if (LR * q >= D) continue;
+        const int i = min(li + LR * q, D - 1);
+        sig[q] = sigma(fmaf(lmax[(BACK ? RPL + qb : qb) * D + i], ys, fmaxf(fabsf(x[q].rs), fabsf(x[q].is))));
+        bias(x[q], sig[q]);
+      }
+#pragma unroll (LR * RPL > 64 ? 2 : 1)
+      for (int jo = 0; jo < jn; ++jo) {
+        const int j = LR * qb + jo;
+        const Cdf y{__shfl_sync(0xffffffffu, x[qb].rs, gbase + jo), __shfl_sync(0xffffffffu, x[qb].re, gbase + jo),
+                    __shfl_sync(0xffffffffu, x[qb].is, gbase + jo), __shfl_sync(0xffffffffu, x[qb].ie, gbase + jo)};
+        const float4* cj = L + cstart(j, D) - j + li;
+#pragma unroll
+        for (int q = 0; q < RPL; ++q) {
+          if (BACK ? q >= qb : q <= qb) continue;
+          if (LR * q >= D) continue;
+          gcms(x[q], BACK ? conj4(L[b0 + j + b1 * q - q * q * (LR * LR / 2)]) : cj[LR * q], pack(y));
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < RPL; ++q) {
+        if (BACK ? q >= qb : q <= qb) continue;
+        if (LR * q >= D) continue;
+        unbias(x[q], sig[q]);
+      }
+    }
   }
 }
 
 // x <- Rl^{-1} x with Rl = Lu Dg Lu^H (rd: the pivot reciprocals).
-template <int LR, int RPL>
-__device__ __forceinline__ void ldl_solve(Cdf (&x)[RPL], const float4* L, const float2* rd, int D, int li,
-                                          int gbase) {
-  subst<LR, RPL, false>(x, L, D, li, gbase);
+template <int LR, int RPL, bool GRID>
+__device__ __forceinline__ void ldl_solve(Cdf (&x)[RPL], const float4* L, const float* lmax, const float2* rd, int D,
+                                          int li, int gbase) {
+  subst<LR, RPL, false, GRID>(x, L, lmax, D, li, gbase);
 #pragma unroll
   for (int q = 0; q < RPL; ++q) {
     const int i = li + LR * q;
     const float2 r = rd[i < D ? i : D - 1];
     x[q] = i < D ? scale(x[q], ff::F2{r.x, r.y}) : Cdf{0.f, 0.f, 0.f, 0.f};
   }
-  subst<LR, RPL, true>(x, L, D, li, gbase);
+  subst<LR, RPL, true, GRID>(x, L, lmax, D, li, gbase);
 #pragma unroll
   for (int q = 0; q < RPL; ++q) norm(x[q]);
 }
@@ -381,7 +479,9 @@ __device__ __forceinline__ ff::F2 pivot(ff::F2 d, int* okf) {
 }
 
 // Copy Rl's lower triangle into shared memory and factor it: Rl = Lu Dg Lu^H,
-// right-looking, two columns per round.  Phase 1: the thread of row i scales
+// right-looking, two columns per round (on grids the trailing triangle takes
+// two rounds' columns at once: one pass over it in shared memory per four
+// columns; 410k cycles per 128-row system without grids, 325k with, 287k by four columns).  Phase 1: the thread of row i scales
 // column j, brings its entry of column j+1 up to date and scales that; each
 // thread forms the two pivots' reciprocals itself.  Phase 2: the rank-2 update
 // of the trailing triangle, its columns spread over groups of RW threads, a
@@ -394,14 +494,35 @@ __device__ __forceinline__ void factor(const System y, int D) {
   using LT = typename SH::LT;
   char* base = reinterpret_cast<char*>(smdf) + y.off;
   LT* L = reinterpret_cast<LT*>(base + sh.l);
-  LT* colb = reinterpret_cast<LT*>(base + sh.col);
-  LT* colb2 = colb + D;
   float2* rd = reinterpret_cast<float2*>(base + sh.rd);
   int* okf = reinterpret_cast<int*>(base + sh.ok);
   const int tt = team_thread<TEAM>();
+  // On grids: h_i = sqrt(Rl_ii); |Rl_il| and every partial sum of the entry's
+  // updates are at most h_i h_l where Rl is positive definite (h_i in rd[i]
+  // until the pivot's reciprocal comes)
+  constexpr bool GRID = grids<TEAM, F32F>();
+  if constexpr (GRID) {
+    for (int i = tt; i < D; i += TEAM) rd[i].x = 1.0001f * sqrtf(fmaxf(entry(y, D, i, i).x, 0.f));
+    team_sync<TEAM>();
+  }
+  auto take = [](Cdf& x, float hh) {               // an entry's finished sum
+    if constexpr (GRID) unbias(x, sigma(hh));
+    else norm(x);
+  };
+  auto less = [](Cdf& x, float4 l, float4 v) {
+    if constexpr (GRID) gcms(x, l, v);
+    else cms(x, l, v);
+  };
   auto put = [&](int i, int l, float4 v) {
-    if constexpr (F32F) L[cstart(l, D) + i - l] = make_float2(__fadd_rn(v.x, v.z), __fadd_rn(v.y, v.w));
-    else L[cstart(l, D) + i - l] = v;
+    if constexpr (F32F) {
+      L[cstart(l, D) + i - l] = make_float2(__fadd_rn(v.x, v.z), __fadd_rn(v.y, v.w));
+    } else if constexpr (GRID) {
+      Cdf b = unpack(v);
+      bias(b, sigma(rd[i].x * rd[l].x));
+      L[cstart(l, D) + i - l] = pack(b);
+    } else {
+      L[cstart(l, D) + i - l] = v;
+    }
     if constexpr (SH::FULL) {
       float4* As = reinterpret_cast<float4*>(base + sh.as);
       if constexpr (!SQUARE) {
@@ -429,7 +550,9 @@ __device__ __forceinline__ void factor(const System y, int D) {
 
   for (int j = 0; j < D; j += 2) {
     const int j1 = j + 1;
-    const bool pair = j1 < D;
+    const bool pair = j1 < D, second = GRID && (j & 2) != 0;
+    LT* colb = reinterpret_cast<LT*>(base + sh.col) + (second ? 2 * D : 0);
+    LT* colb2 = colb + D;
     const int cj = cstart(j, D), c1 = pair ? cstart(j1, D) : cj;
     if constexpr (F32F) {
       const float rj = pivot<F32F>({L[cj].x, 0.f}, okf).hi;
@@ -469,27 +592,27 @@ __device__ __forceinline__ void factor(const System y, int D) {
       team_sync<TEAM>();
       if (own1) L[cj + 1] = own;
     } else {
+      const float hj = GRID ? rd[j].x : 0.f, h1 = GRID && pair ? rd[j1].x : 0.f;
       Cdf dj = unpack(L[cj]);
-      norm2(dj.rs, dj.re);
+      take(dj, hj * hj);
       const ff::F2 rj = pivot<F32F>({dj.rs, dj.re}, okf);
       Cdf a1j{0.f, 0.f, 0.f, 0.f};
       ff::F2 r1{1.f, 0.f};
       if (pair) {
         a1j = unpack(L[cj + 1]);
-        norm(a1j);
-        const Cdf l1j = scale(a1j, rj);
+        take(a1j, hj * h1);
         Cdf d1 = unpack(L[c1]);
-        mac(d1.rs, d1.re, -l1j.rs, -l1j.re, a1j.rs, a1j.re);
-        mac(d1.rs, d1.re, -l1j.is, -l1j.ie, a1j.is, a1j.ie);
-        norm2(d1.rs, d1.re);
+        less(d1, pack(scale(a1j, rj)), conj4(pack(a1j)));
+        take(d1, h1 * h1);
         r1 = pivot<F32F>({d1.rs, d1.re}, okf);
       }
       const float4 a1c = conj4(pack(a1j));
       float4 own = make_float4(0.f, 0.f, 0.f, 0.f);
       bool own1 = false;
       for (int i = j1 + tt; i < D; i += TEAM) {
+        const float hi = GRID ? rd[i].x : 0.f;
         Cdf v = unpack(L[cj + i - j]);
-        norm(v);
+        take(v, hi * hj);
         colb[i] = conj4(pack(v));                // stored conjugated
         const float4 lij = pack(scale(v, rj));
         if (i == j1) {
@@ -498,18 +621,50 @@ __device__ __forceinline__ void factor(const System y, int D) {
         } else {
           L[cj + i - j] = lij;
           Cdf w = unpack(L[c1 + i - j1]);
-          cms(w, lij, a1c);
-          norm(w);
+          less(w, lij, a1c);
+          take(w, hi * h1);
           colb2[i] = conj4(pack(w));
           L[c1 + i - j1] = pack(scale(w, r1));
         }
       }
+      team_sync<TEAM>();
       if (tt == 0) {
         rd[j] = make_float2(rj.hi, rj.lo);
         if (pair) rd[j1] = make_float2(r1.hi, r1.lo);
       }
-      team_sync<TEAM>();
       if (own1) L[cj + 1] = own;
+    }
+    if constexpr (GRID) {
+      if (!second) {                               // the next pair of columns only
+        const int l = j + 2 + tt / (TEAM / 2), i = l + tt % (TEAM / 2);
+        if (i < D) {
+          LT* e = L + cstart(l, D) + i - l;
+          Cdf acc = unpack(*e);
+          gcms(acc, L[cj + i - j], colb[l]);
+          gcms(acc, L[c1 + i - j1], colb2[l]);
+          norm(acc);
+          *e = pack(acc);
+        }
+      } else {                                     // the rest, by both pairs
+        constexpr int RW = TEAM == 512 ? 32 : 16;
+        const LT* la = L + cstart(j - 2, D) + 2 - j;
+        const LT* lb = L + cstart(j - 1, D) + 1 - j;
+        for (int l = j + 2 + tt / RW; l < D; l += TEAM / RW) {
+          const LT ya = colb[l - 2 * D], yb = colb[l - D], yc = colb[l], yd = colb2[l];
+          LT* cl = L + cstart(l, D) - l;
+          for (int i = l + tt % RW; i < D; i += RW) {
+            Cdf acc = unpack(cl[i]);
+            gcms(acc, la[i], ya);
+            gcms(acc, lb[i], yb);
+            gcms(acc, L[cj + i - j], yc);
+            gcms(acc, L[c1 + i - j1], yd);
+            norm(acc);
+            cl[i] = pack(acc);
+          }
+        }
+      }
+      team_sync<TEAM>();
+      continue;
     }
     constexpr int RW = TEAM == 512 ? 32 : (TEAM >= 128 ? 16 : (TEAM >= 32 ? 8 : 4));
     for (int l = j + 2 + tt / RW; l < D; l += TEAM / RW) {
@@ -530,8 +685,8 @@ __device__ __forceinline__ void factor(const System y, int D) {
           cl[i] = acc;
         } else {
           Cdf acc = unpack(cl[i]);
-          cms(acc, lij, alj);
-          cms(acc, mij, blj);
+          less(acc, lij, alj);
+          less(acc, mij, blj);
           norm(acc);
           cl[i] = pack(acc);
         }
@@ -557,6 +712,7 @@ __device__ __forceinline__ void solve_rhs(const SolveDfParams& prm, const System
   float4* As = reinterpret_cast<float4*>(base + sh.as);
   const typename SH::LT* L = reinterpret_cast<const typename SH::LT*>(base + sh.l);
   const float2* rd = reinterpret_cast<const float2*>(base + sh.rd);
+  constexpr bool GRID = grids<TEAM, F32F>();
   const int tt = team_thread<TEAM>(), li = tt % LR, g = tt / LR;
   const int gbase = (threadIdx.x & 31) - li;       // first lane of this thread's group
   // a CTA team's warps past the last right-hand side only help convert
@@ -580,9 +736,27 @@ __device__ __forceinline__ void solve_rhs(const SolveDfParams& prm, const System
 #pragma unroll
   for (int q = 0; q < RPL; ++q) x[q] = b_at(li + LR * q);
   for (int it = 0;; ++it) {
+    // the largest entry of each row block of a column and column block of a
+    // row, in the chunk's place
+    float* lmax = reinterpret_cast<float*>(As);
+    if constexpr (GRID) {
+      __syncthreads();
+      for (int f = tt; f < 2 * RPL * D; f += TEAM) {
+        const int b = f / D, i = f - b * D, j0 = LR * (b < RPL ? b : b - RPL);
+        const int j1 = min(j0 + LR, D);
+        float m = 0.f;
+        if (b < RPL ? i >= j1 : i < j0)
+          for (int j = j0; j < j1; ++j) {
+            const float4 l = L[b < RPL ? cstart(j, D) - j + i : cstart(i, D) - i + j];
+            m = fmaxf(m, fmaxf(fabsf(l.x), fabsf(l.y)));
+          }
+        lmax[f] = m;
+      }
+      __syncthreads();
+    }
     if (work) {
       if constexpr (F32F) ldl_solve_f32<LR, RPL>(x, L, rd, D, li, gbase);
-      else ldl_solve<LR, RPL>(x, L, rd, D, li, gbase);
+      else ldl_solve<LR, RPL, GRID>(x, L, lmax, rd, D, li, gbase);
 #pragma unroll
       for (int q = 0; q < RPL; ++q) {
         const int i = li + LR * q;
@@ -698,7 +872,7 @@ __device__ __noinline__ void emit(const SolveDfParams& prm, int off, long long s
 }
 
 // Separable steering: u_s = sum_c a_s[c] U_c from the team's basis solutions U
-// (at byte `off` of shared memory) and the normalised weights. 
+// (at byte `off` of shared memory) and the normalised weights.
 template <int LR, int RPL, int TEAM>
 __device__ __noinline__ void combine(const SolveDfParams& prm, int off, long long sys, bool valid, bool ok, int e) {
   constexpr int NG = TEAM / LR;
@@ -726,43 +900,43 @@ __device__ __noinline__ void combine(const SolveDfParams& prm, int off, long lon
     constexpr int QB = RPL % 4 == 0 ? 4 : (RPL % 3 == 0 ? 3 : 2);   // rows per pass over the basis
 #pragma unroll
     for (int q0 = 0; q0 < RPL; q0 += QB) {
-    if (LR * q0 >= D) continue;
-    Cdf PR[QB], TQ[QB];                        // (P, R) and (T, Q) of each row
+      if (LR * q0 >= D) continue;
+      Cdf PR[QB], TQ[QB];                        // (P, R) and (T, Q) of each row
 #pragma unroll
-    for (int q = 0; q < QB; ++q) PR[q] = TQ[q] = Cdf{0.f, 0.f, 0.f, 0.f};
-    for (int c = 0; c < C; ++c) {
-      const float4 a = __ldg(as + c);
+      for (int q = 0; q < QB; ++q) PR[q] = TQ[q] = Cdf{0.f, 0.f, 0.f, 0.f};
+      for (int c = 0; c < C; ++c) {
+        const float4 a = __ldg(as + c);
 #pragma unroll
-      for (int q = 0; q < QB; ++q) {
-        const int i = li + LR * (q0 + q);
-        const float4 u = U[(size_t)c * D + (i < D ? i : D - 1)];
-        mac(PR[q].rs, PR[q].re, a.x, a.y, u.x, u.z);
-        mac(TQ[q].is, TQ[q].ie, a.z, a.w, u.y, u.w);
-        mac(PR[q].is, PR[q].ie, a.x, a.y, u.y, u.w);
-        mac(TQ[q].rs, TQ[q].re, a.z, a.w, u.x, u.z);
+        for (int q = 0; q < QB; ++q) {
+          const int i = li + LR * (q0 + q);
+          const float4 u = U[(size_t)c * D + (i < D ? i : D - 1)];
+          mac(PR[q].rs, PR[q].re, a.x, a.y, u.x, u.z);
+          mac(TQ[q].is, TQ[q].ie, a.z, a.w, u.y, u.w);
+          mac(PR[q].is, PR[q].ie, a.x, a.y, u.y, u.w);
+          mac(TQ[q].rs, TQ[q].re, a.z, a.w, u.x, u.z);
+        }
       }
-    }
 #pragma unroll
-    for (int q = q0; q < q0 + QB; ++q) {
-      const int i = li + LR * q;
-      norm(PR[q - q0]);
-      norm(TQ[q - q0]);
-      const ff::F2 P{PR[q - q0].rs, PR[q - q0].re}, R{PR[q - q0].is, PR[q - q0].ie};
-      const ff::F2 T{TQ[q - q0].rs, TQ[q - q0].re}, Q{TQ[q - q0].is, TQ[q - q0].ie};
-      const ff::F2 ur1 = ff::sub2(P, Q), ui1 = ff::add2(R, T);
-      const ff::F2 ur2 = ff::add2(P, Q), ui2 = ff::sub2(R, T);
-      if (i < D) {
-        const float4 b1 = __ldg(v1 + i), b2 = __ldg(v2 + i);
-        mac(q1s, q1e, b1.x, b1.y, ur1.hi, ur1.lo);
-        mac(q1s, q1e, b1.z, b1.w, ui1.hi, ui1.lo);
-        mac(q2s, q2e, b2.x, b2.y, ur2.hi, ur2.lo);
-        mac(q2s, q2e, b2.z, b2.w, ui2.hi, ui2.lo);
+      for (int q = q0; q < q0 + QB; ++q) {
+        const int i = li + LR * q;
+        norm(PR[q - q0]);
+        norm(TQ[q - q0]);
+        const ff::F2 P{PR[q - q0].rs, PR[q - q0].re}, R{PR[q - q0].is, PR[q - q0].ie};
+        const ff::F2 T{TQ[q - q0].rs, TQ[q - q0].re}, Q{TQ[q - q0].is, TQ[q - q0].ie};
+        const ff::F2 ur1 = ff::sub2(P, Q), ui1 = ff::add2(R, T);
+        const ff::F2 ur2 = ff::add2(P, Q), ui2 = ff::sub2(R, T);
+        if (i < D) {
+          const float4 b1 = __ldg(v1 + i), b2 = __ldg(v2 + i);
+          mac(q1s, q1e, b1.x, b1.y, ur1.hi, ur1.lo);
+          mac(q1s, q1e, b1.z, b1.w, ui1.hi, ui1.lo);
+          mac(q2s, q2e, b2.x, b2.y, ur2.hi, ur2.lo);
+          mac(q2s, q2e, b2.z, b2.w, ui2.hi, ui2.lo);
+        }
+        w1r[q] = ur1;
+        w1i[q] = ui1;
+        w2r[q] = ur2;
+        w2i[q] = ui2;
       }
-      w1r[q] = ur1;
-      w1i[q] = ui1;
-      w2r[q] = ur2;
-      w2i[q] = ui2;
-    }
     }
     const ff::F2 d1 = lanes_sum2<LR>(q1s, q1e), d2 = lanes_sum2<LR>(q2s, q2e);
     const bool good1 = ok && usable(d1), good2 = ok && usable(d2);

@@ -116,6 +116,23 @@ def test_any_power_of_the_input_scale_gives_the_same_weights(scale):
         assert np.all(~np.isfinite(w.real) | (np.abs(w.real) > 1e30)) if scale < 1 else np.all(np.abs(w) < 1e-30)
 
 
+@pytest.mark.parametrize("refine", [0, 1])
+@pytest.mark.parametrize("C,T", [(11, 3), (16, 4), (13, 5), (32, 3), (97, 1), (32, 4)])
+def test_rows_of_uneven_power(C, T, refine):
+    """From 33 rows on the factor's sums run on grids set by the diagonal, the
+    substitutions' by the factor's entries and the solution: diagonals over
+    six decades, and a row that the others do not touch."""
+    D, S = C * T, 7
+    R = _covariances(8, D, seed=D)
+    r = 10.0 ** np.random.default_rng(D).uniform(-3, 0, D)
+    R = R * r[:, None] * r[None, :]
+    R[:, D // 2, :D // 2] = R[:, D // 2, D // 2 + 1:] = 0
+    R[:, :D // 2, D // 2] = R[:, D // 2 + 1:, D // 2] = 0
+    w, status = _solve(R, C, T, S, refine_steps=refine)
+    assert status == (stap.STAP_OK, 0)
+    _check(w, _reference(R, _default_steering(C, T, S), 1e-3))
+
+
 def test_weak_loads_take_the_fp64_kernels():
     """Nothing bounds the condition number without a load: such plans keep the
     FP64 kernels bit for bit (solve_kind 3 names one of them)."""
