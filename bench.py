@@ -1,12 +1,12 @@
 """Benchmark of the STAP path on GB300: range-Doppler cells per second.
 
 One step = one whole CPI through ``stap_run_cpi`` (Doppler transform,
-covariance, FP64 loading/LDL^H/solves/refinement, apply).  The headline is the
+covariance, loading/LDL^H/solves/refinement, apply).  The headline is the
 large CPI (C=32 channels, P=512 pulses, K=512 Doppler bins, R=32768 range
 cells, T=4 so D=128, B=256-cell training blocks, S=64 steering vectors; a
 seeded synthetic 4.3 GB cube: unit noise, 40 dB CNR clutter ridge, 32
 targets) on the mixed path (FP16 per-block-scaled split products on the tensor
-cores for the covariance and the apply, FP64 solve), with the plain FP32 path
+cores for the covariance and the apply, double-float solve), with the plain FP32 path
 timed on the same cube beside it.  The D = 64 CPI, the standard D = 12 CPI and
 the 512-CPI batch are keys of the same line, each with its mixed and plain
 legs; every single-CPI workload also runs the mixed-precision refinement
@@ -42,22 +42,13 @@ L2_FLUSH_BYTES = 256 << 20
 
 # DRAM bytes (read + write) per launch of the solve kernel (dram__bytes_read.sum
 # + dram__bytes_write.sum of one unslabbed launch, from an ncu capture
-# summarised in profiles/), keyed by a hash of the kernel source, the solve
-# kernel the tuning chose (1 register-resident, 2 shared-memory teams, 3 one
-# system per CTA) and the workload, so that a changed or different kernel
-# reports null until re-measured.  The large CPI's entry is an eighth of it
-# (8192 of its 65536 systems, same kernel and launch shape: 1151412224 bytes
-# read + 510120448 written, the capture summarised in profiles/) scaled by 8, the
-# traffic being per system (its lower triangle read, its weights written).
-# The second key is solve.cu after a change confined to the refinement
-# option's team kernel (solve_mir_kernel, its shared-memory strides and size
-# function, and a helper they use): solve_big_kernel's source is the same, so
-# the same capture applies.
-SOLVE_TRAFFIC = {("ece189e7f5967c5d", 3, "large"): 8 * (1151412224 + 510120448),
-                 ("077ece954fb9fac1", 3, "large"): 8 * (1151412224 + 510120448)}
-SOLVE_KERNELS = {1: "solve_reg_kernel (register-resident FP64 LDL^H, solves, refinement)",
-                 2: "solve_kernel (shared-memory FP64 Cholesky teams, solves, refinement)",
-                 3: "solve_big_kernel (one system per CTA: FP64 LDL^H, solves, refinement)"}
+# summarised in profiles/), keyed by a hash of the kernel source and the
+# workload, so that a changed kernel reports null until re-measured.  The large
+# CPI's entry is an eighth of it (8192 of its 65536 systems, same kernel and
+# launch shape) scaled by 8, the traffic being per system (its lower triangle
+# read, its weights written).
+SOLVE_TRAFFIC = {("cf777efc75b6551f", "large"): 8 * (1147238144 + 512322816)}
+SOLVE_KERNEL = "solve_df_kernel (double-float LDL^H, solves, refinement on the FP32 pipe)"
 
 
 def peaks():
@@ -96,20 +87,32 @@ def workload_config(spec, name=None):
 
 
 def solve_flops(spec, refine=1, separable=True):
-    """Algorithmic FP64 flops of the loading/Cholesky/solve kernel (8 flops per
+    """Algorithmic flops of the loading/factorisation/solve step (8 flops per
     complex multiply-add): Cholesky D^3/6, then (1 + 2 refine) forward/back
     solve pairs of D^2 each (one solve, then per refinement step a residual
     and a solve) for each right-hand side -- the C basis vectors when the
     steering set is separable, otherwise the S steering vectors, followed by
     their FP64 normalisations (D real products each).  The separable path's
-    combination of the basis solutions and its normalisations run in
-    double-float on the FP32 pipe and are not FP64 work."""
+    combination of the basis solutions and its normalisations are left out."""
     C, P, K, R, T, B, S = spec.dims()
     D, NB = C * T, R // B
     if separable:
         per = 8.0 * (D ** 3 / 6.0 + (1 + 2 * refine) * C * D * D)
     else:
         per = 8.0 * (D ** 3 / 6.0 + (1 + 2 * refine) * S * D * D) + 4.0 * S * D
+    return K * NB * per
+
+
+def solve_instr(spec, refine=1):
+    """FP32 instructions (per lane) that the double-float solve cannot do
+    without: 48 per complex multiply-add (four real ones of 12: the product
+    and its error, TwoSum, the cross terms), 24 where the sum runs on a fixed
+    grid -- from D = 33 on, the factorisation and the substitutions.  The
+    combination into the steering vectors and the normalisation are left out."""
+    C, P, K, R, T, B, S = spec.dims()
+    D, NB = C * T, R // B
+    g = 24.0 if D > 32 else 48.0
+    per = g * (D ** 3 / 6.0 + (1 + refine) * C * D * D) + 48.0 * refine * C * D * D
     return K * NB * per
 
 
@@ -232,7 +235,8 @@ PREC_TEXT = {
     3: "mixed: FP16 two-piece split products (3) with per-block power-of-two scaling on the tensor "
        "cores for covariance and apply, FP32 accumulation; FP32 FFT",
 }
-SOLVE_TEXT = "FP64 diagonal load, LDL^H factorisation and substitutions, 1 refinement step"
+SOLVE_TEXT = ("FP64 diagonal load; LDL^H factorisation, substitutions and 1 refinement step in "
+              "double-float (two FP32, about 2^-44)")
 MIR_TEXT = ("mixed-precision refinement solve: FP64 diagonal load, FP32 LDL^H and substitutions, "
             "2 refinement steps with double-float residuals (STAP_SOLVE_MIXED_IR)")
 
@@ -296,20 +300,21 @@ def kernel_figures(spec, prec, kt, pk, refine=1, solver=0, used=None):
     C, P, K, R, T, B, S = spec.dims()
     D, NB = C * T, R // B
     dop_bytes = 8.0 * C * R * (P + K)
-    sf = solve_flops(spec, refine=refine)
+    sf, si = solve_flops(spec, refine=refine), solve_instr(spec, refine=refine)
     out = {
         "doppler": {"ms": kt["doppler"], "bound": "hbm", "bytes": dop_bytes,
                     "achieved_gbs": dop_bytes / kt["doppler"] / 1e6,
                     "frac": dop_bytes / kt["doppler"] / 1e6 / pk["hbm_gbs"]},
-        "solve": {"ms": kt["solve"], "bound": "alu", "fp64_flops": sf,
-                  "achieved_tflops": sf / kt["solve"] / 1e9,
-                  "frac": sf / kt["solve"] / 1e9 / pk["fp64_tflops"]},
+        "solve": {"ms": kt["solve"], "bound": "alu", "fp32_instr": si,
+                  "achieved_tinstr": si / kt["solve"] / 1e9,
+                  "frac": si / kt["solve"] / 1e9 / (pk["fp32_tflops"] / 2),
+                  "fp64_equivalent_tflops": sf / kt["solve"] / 1e9},
     }
     if solver == 1:   # FP32 factor and substitutions, double-float residuals: no FP64 roofline
         out["solve"] = {"ms": kt["solve"], "bound": "fp32 issue",
                         "fp64_equivalent_tflops": sf / kt["solve"] / 1e9,
-                        "note": "FP64-solve flop count over this solve's time, for comparison with "
-                                "the FP64 solve; the kernel itself runs on the FP32 and integer pipes"}
+                        "note": "the solve's flop count over its time; the kernel itself runs on the "
+                                "FP32 and integer pipes"}
     # covariance through the step call (full Hermitian c128 output)
     cov_bytes = 8.0 * C * K * R + 16.0 * K * NB * D * D
     apply_bytes = 8.0 * C * K * R + 8.0 * K * NB * S * D + 4.0 * S * K * R
@@ -318,8 +323,8 @@ def kernel_figures(spec, prec, kt, pk, refine=1, solver=0, used=None):
     fp32_app = prec == 0 or used.get("apply", "").startswith("FP32")
     if fp32_cov:
         cplx = 1.0 * K * NB * B * (T * C * C - C * (C - 1) // 2)
-        out["covariance"] = {"ms": kt["covariance"], "bound": "alu", "fp32_instr": 20.0 * cplx,
-                             "frac": 20.0 * cplx / kt["covariance"] / 1e9 / (pk["fp32_tflops"] / 2),
+        out["covariance"] = {"ms": kt["covariance"], "bound": "alu", "fp32_instr": 16.0 * cplx,
+                             "frac": 16.0 * cplx / kt["covariance"] / 1e9 / (pk["fp32_tflops"] / 2),
                              "hbm_frac": cov_bytes / kt["covariance"] / 1e6 / pk["hbm_gbs"]}
     if fp32_app:
         af = 8.0 * K * R * S * D
@@ -521,18 +526,18 @@ def run_gpu(args):
         total_ms, value = aggregate(mleg["ms_per_step"] * sub.steps, cells * sub.steps, world, dev)
         ms_per_step = total_ms / sub.steps
         kern = kernel_figures(spec, mprec, mleg["kernels_ms"], pk, used=mleg["kernels_used"])
-        solve_kind = 3 if C * T > 32 else list(mleg["tuning"].values())[0][7]
-        roofline = {"kernel": SOLVE_KERNELS.get(solve_kind, "solve"),
-                    "bound": "alu", "achieved": kern["solve"]["achieved_tflops"],
-                    "peak": pk["fp64_tflops"], "unit": "TFLOP/s", "frac": kern["solve"]["frac"],
-                    "traffic": SOLVE_TRAFFIC.get((kernel_hash(), solve_kind, name)),
-                    "basis": "8 K NB (D^3/6 + (1 + 2 refine) C D^2) FP64 flops per launch: the "
+        roofline = {"kernel": SOLVE_KERNEL,
+                    "bound": "alu", "achieved": kern["solve"]["achieved_tinstr"],
+                    "peak": pk["fp32_tflops"] / 2, "unit": "T FP32 instructions/s",
+                    "frac": kern["solve"]["frac"],
+                    "traffic": SOLVE_TRAFFIC.get((kernel_hash(), name)),
+                    "basis": "K NB (24 (D^3/6 + (1 + refine) C D^2) + 48 refine C D^2) FP32 lane "
+                             "instructions per launch (48 throughout for D <= 32): the "
                              "factorisation plus, for each of the C basis right-hand sides of the "
                              "separable steering (v_s = g (x) a_s), one forward/back solve pair and "
-                             "per refinement step a residual and a solve pair; the combination into "
-                             "the S steering vectors and their normalisation run on the FP32 pipe",
-                    "peak_src": "FP64: 152 SMs x 2 DFMA/clk x 2 flops x 2.07 GHz (unit count and max "
-                                "clock; a DFMA microbenchmark measured 1.20 TFLOP/s at 1987 MHz)"}
+                             "per refinement step a residual and a solve pair",
+                    "fp64_equivalent_tflops": kern["solve"]["fp64_equivalent_tflops"],
+                    "peak_src": "FP32: 152 SMs x 128 lanes x 2.07 GHz (unit count and max clock)"}
         # ---- end to end through the public API from pinned host buffers ----
         ring = 4 if cube_h.nbytes <= (1 << 30) else 2
         cube_pin = torch.from_numpy(cube_h).pin_memory()
@@ -757,8 +762,8 @@ def batch_legs(args, dev, stream, flush):
             "value": cells / (ms * 1e-3), "ms_per_step": ms, "steps": steps, "autotune_s": tune_s,
             "schedule": sched_names[chosen], "ms_per_step_by_schedule": schedules,
             "gpu_launches_per_step": 4 * len(specs),
-            "fp64_solve_frac_of_step": sum(solve_flops(s) for s in specs) / (ms * 1e-3) / 1e12 /
-            peaks()["fp64_tflops"]}
+            "solve_frac_of_step": sum(solve_instr(s) for s in specs) / (ms * 1e-3) / 1e12 /
+            (peaks()["fp32_tflops"] / 2)}
         plan.close()
         del plan, outs
         torch.cuda.empty_cache()
@@ -834,15 +839,15 @@ def run_batch(args):
     cells = sum(s.cells for s in specs)
     total_ms, value = aggregate(sum(times), cells * args.steps, world, dev)
     ms_per_step = total_ms / args.steps
-    sf = sum(solve_flops(s, refine=1) for s in specs)
+    si = sum(solve_instr(s, refine=1) for s in specs)
     pk = peaks()
-    achieved = sf / (ms_per_step * 1e-3) / 1e12
-    roofline = {"kernel": "all solve kernels of the batch (FP64)", "bound": "alu",
-                "achieved": achieved, "peak": pk["fp64_tflops"], "unit": "TFLOP/s",
-                "frac": achieved / pk["fp64_tflops"], "traffic": None,
-                "basis": "FP64 solve flops of all 512 CPIs / whole step time (a lower bound for "
+    achieved = si / (ms_per_step * 1e-3) / 1e12
+    roofline = {"kernel": "all solve kernels of the batch (double-float)", "bound": "alu",
+                "achieved": achieved, "peak": pk["fp32_tflops"] / 2, "unit": "T FP32 instructions/s",
+                "frac": achieved / (pk["fp32_tflops"] / 2), "traffic": None,
+                "basis": "FP32 solve instructions of all 512 CPIs / whole step time (a lower bound for "
                          "the solve kernels: the step also runs the other 1536 launches)",
-                "peak_src": "FP64: 152 SMs x 2 DFMA/clk x 2 flops x 2.07 GHz (unit count and max clock)"}
+                "peak_src": "FP32: 152 SMs x 128 lanes x 2.07 GHz (unit count and max clock)"}
 
     # end to end: every cube from pinned host memory, every output back
     h2d = sum(c.numel() * 8 for c in cubes)
@@ -1034,7 +1039,7 @@ def host_mem_available():
 def kernel_hash():
     import hashlib
     h = hashlib.sha256()
-    with open(os.path.join(ROOT, "paper_2203_06233_gb300", "csrc", "solve.cu"), "rb") as f:
+    with open(os.path.join(ROOT, "paper_2203_06233_gb300", "csrc", "solve_df_kernel.cuh"), "rb") as f:
         h.update(f.read())
     return h.hexdigest()[:16]
 

@@ -285,7 +285,7 @@ stap_status stap_apply(stap_plan plan, const void* dop_c64, const void* wts_c64,
  * With n_cpi == 1 and a tuned slab count above 1 (stap_plan_autotune or
  * stap_plan_set_tuning), the range axis is cut into that many slabs of whole
  * training blocks and each slab's chain runs on its own internal stream,
- * earlier slabs at higher priority, so that the FP64 solve of one slab
+ * earlier slabs at higher priority, so that the solve of one slab
  * overlaps the other steps of the next; the result is the same.  Those
  * streams are created by the first such call and joined back into the plan's
  * stream before the call returns.
@@ -313,9 +313,8 @@ stap_status stap_run_cpi(stap_plan plan, const void* const* cubes, float* const*
  *                          bins or systems) from an atomic counter over a
  *                          device array of per-CPI parameter blocks, with no
  *                          waits between CTAs; kernels without a persistent
- *                          form (the mixed-precision refinement solves, the
- *                          training averages, the tensor-core kernels) run
- *                          one launch per CPI in that phase.  The default.
+ *                          form (the training averages, the tensor-core
+ *                          kernels) run one launch per CPI in that phase.  The default.
  *   STAP_BATCH_STREAMS     each CPI's four-step chain on one of several
  *                          internal streams, so that CPIs overlap.
  * Either way the whole sequence is captured into a CUDA graph and replayed

@@ -5,8 +5,8 @@
 // Muller et al., "Handbook of Floating-Point Arithmetic", ch. 4 and 14.
 //
 // GB300 runs FP32 at 62x the FP64 rate, so work that needs more than FP32
-// but is not itself a triangular solve (combinations and normalisations of
-// FP64 solutions) is cheaper here than on the FP64 pipe.
+// is cheaper here than on the FP64 pipe: the solves whose condition number is
+// bounded, and the combinations and normalisations of FP64 solutions.
 #pragma once
 
 #include <cstdint>
@@ -49,15 +49,9 @@ __device__ __forceinline__ F2 add2(F2 a, F2 b) {
 }
 __device__ __forceinline__ F2 sub2(F2 a, F2 b) { return add2(a, {-b.hi, -b.lo}); }
 
-// a + b with a a double-float and b a float
-__device__ __forceinline__ F2 add(F2 a, float b) {
-  const F2 s = two_sum(a.hi, b);
-  return fast_two_sum(s.hi, __fadd_rn(s.lo, a.lo));
-}
-
 // ---- conversions on the integer pipe -------------------------------------
 // On this GPU every float <-> double conversion instruction occupies the FP64
-// pipe, the one the solve is bound by.  Both directions are exact or
+// pipe, the one the FP64 solves are bound by.  Both directions are exact or
 // correctly rounded re-encodings of IEEE-754 fields, done here with integer
 // operations.
 
@@ -111,14 +105,7 @@ __device__ __forceinline__ float round_to_float(uint64_t n, int e2, uint32_t sig
 }
 
 // Split a double into hi = nearest float, lo = nearest float to the rest
-// (x - hi is exact in double), with the conversion instructions: for kernels
-// bound by the FP32 or integer issue rather than by the FP64 pipe.
-__device__ __forceinline__ F2 from_double_cvt(double x) {
-  const float hi = __double2float_rn(x);
-  return {hi, __double2float_rn(x - (double)hi)};
-}
-
-// The same split on the integer pipe (bit-identical), for kernels bound by the
+// (x - hi is exact in double), on the integer pipe, for kernels bound by the
 // FP64 pipe: |x| in [2^-70, 2^126), where hi and a nonzero lo are normal
 // floats; the conversion instructions elsewhere (zero, tiny, huge,
 // non-finite).

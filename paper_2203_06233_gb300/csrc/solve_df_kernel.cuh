@@ -479,13 +479,14 @@ __device__ __forceinline__ ff::F2 pivot(ff::F2 d, int* okf) {
 }
 
 // Copy Rl's lower triangle into shared memory and factor it: Rl = Lu Dg Lu^H,
-// right-looking, two columns per round (on grids the trailing triangle takes
-// two rounds' columns at once: one pass over it in shared memory per four
-// columns; 410k cycles per 128-row system without grids, 325k with, 287k by four columns).  Phase 1: the thread of row i scales
+// right-looking, two columns per round.  Phase 1: the thread of row i scales
 // column j, brings its entry of column j+1 up to date and scales that; each
 // thread forms the two pivots' reciprocals itself.  Phase 2: the rank-2 update
 // of the trailing triangle, its columns spread over groups of RW threads, a
-// group's threads over a column's rows.
+// group's threads over a column's rows.  On grids every other phase 2 updates
+// the next two columns only and the one after it takes four columns at once,
+// half the passes over the triangle in shared memory (128 rows: 410k cycles
+// without grids, 325k with, 287k by four columns).
 template <int TEAM, bool F32F, bool SQUARE>
 __device__ __forceinline__ void factor(const System y, int D) {
   extern __shared__ float4 smdf[];
