@@ -150,30 +150,6 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
-// FP16S: the work of a CTA is a run of consecutive tiles of the order (group of
-// `lc` bins, column, bin): the next tile of a run is the next bin of the same
-// range cells, which shares all but one of its T bins, so that its maximum
-// needs a pass over that one bin's rows only.  lc is a CTA's number of tiles, so
-// that neighbouring CTAs walk the same bins beside each other and share
-// weights and Doppler rows in L2.
-// D = 128 (C32 T4 K512 R2048 B256 S64): covariance 888 -> 858 us; apply, with four
-// weight vectors' loads in flight per warp, 1089 -> 1005 us; the same bits.
-__device__ __forceinline__ void run_tile(long long o, int K, int ncol, int lc, int& k, int& col) {
-  const long long grp = (long long)lc * ncol, q = o / grp;
-  const int k0 = (int)q * lc, len = min(lc, K - k0), rem = (int)(o - q * grp);
-  col = rem / len;
-  k = k0 + rem - col * len;
-}
-
-// Tiles per run for `ntiles` tiles on `blocks` CTAs, or 0 where runs share
-// nothing (one bin per snapshot, or fewer than two tiles per CTA).
-template <int PREC>
-int run_length(long long ntiles, long long blocks, int K, int T) {
-  if (PREC != kFP16S || T < 2 || ntiles < 2 * blocks) return 0;
-  const long long lc = (ntiles + blocks - 1) / blocks;
-  return (int)(lc < K ? lc : K);
-}
-
 template <int PREC>
 __device__ __forceinline__ void issue_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, bool acc) {
   if constexpr (PREC == kTF32X3)
@@ -205,6 +181,22 @@ struct CovForm {
   static constexpr int GROWS = STK ? 64 : 128;   // rows of Xr a tile takes (G D8 <= GROWS)
 };
 
+// FP16S split form: a CTA's tiles are consecutive in the order (group of `lc`
+// bins, range block, bin), so that the next tile is mostly the next bin of the
+// same cells, which shares all but one of its T bins: its scale pass reads that
+// one bin's rows only.  lc is a CTA's number of tiles, so that neighbouring CTAs
+// walk the same bins beside each other and share their rows in L2.  D = 128:
+// C32 T4 K512 R2048 B256 891 -> 858 us, B64 (K256) 1134 -> 1094, D = 96 B200
+// 471 -> 422; the same bits (a maximum is exact).  The stacked form, whose two
+// CTAs per SM hide the pass, and the apply, whose output and weights lie the
+// other way, lost 2 to 30% in that order.
+__device__ __forceinline__ long long run_system(long long o, int K, int NB, int lc) {
+  const long long grp = (long long)lc * NB, q = o / grp;
+  const int k0 = (int)q * lc, len = min(lc, K - k0), rem = (int)(o - q * grp);
+  const int b = rem / len;
+  return (long long)(k0 + rem - b * len) * NB + b;
+}
+
 template <int PREC>
 constexpr size_t cov_smem() { return 2 * (size_t)Fmt<PREC>::NPC * kCovPiece; }
 
@@ -220,12 +212,13 @@ covariance_tcx_kernel(const float2* __restrict__ dop, double2* __restrict__ cov,
   constexpr int STAGE = F::NPC * kCovPiece;
   constexpr int CPW = 16 / F::ESZ;           // cells per core-matrix row
   constexpr int CPL = CPW / 4;               // cells per lane in a staging unit
+  constexpr bool RUNS = PREC == kFP16S && !STK;   // G = 1
   extern __shared__ __align__(1024) uint8_t sm[];
   __shared__ __align__(8) uint64_t mbar[2];
   __shared__ uint32_t tmem_base;
   __shared__ long long rowbase[128];          // dop offset of Xr/Xi row p, or -1
   __shared__ float sscale[128];               // per system scale (FP16S)
-  __shared__ int smax[128];                   // per system, or (in runs) per bin of the one system
+  __shared__ int smax[128];                   // per system; RUNS: per bin of the one system
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int D = C * T;
   const int GD = G * D8;                     // Xr rows of the tile (Xi rows follow)
@@ -250,23 +243,13 @@ covariance_tcx_kernel(const float2* __restrict__ dop, double2* __restrict__ cov,
   bool ok = true;
   long long gch = 0;                          // chunks issued by this CTA (stage = gch & 1)
 
-  // runs of bins (lc > 0: FP16S, one system per tile), or tiles dealt out in turn
-  if (PREC != kFP16S) lc = 0;
-  const long long t0 = lc ? ntiles * blockIdx.x / gridDim.x : blockIdx.x;
-  const long long t1 = lc ? ntiles * (blockIdx.x + 1) / gridDim.x : ntiles;
-  int last_k = -2, last_b = -1;
-  for (long long tile = t0; tile < t1 && ok; tile += lc ? 1 : gridDim.x) {
-    long long sys0 = tile * G;
-    int first_row = 0, shift = 0;             // rows whose maximum is not known yet
-    if (lc) {
-      int k, b;
-      run_tile(tile, K, NB, lc, k, b);
-      sys0 = (long long)k * NB + b;
-      shift = b == last_b && k == last_k + 1;
-      if (shift) first_row = (T - 1) * C;
-      last_k = k;
-      last_b = b;
-    }
+  const long long tile0 = RUNS ? ntiles * blockIdx.x / gridDim.x : blockIdx.x;
+  const long long tile1 = RUNS ? ntiles * (blockIdx.x + 1) / gridDim.x : ntiles;
+  long long last = -1 - (long long)NB;        // RUNS: the system before
+  for (long long tile = tile0; tile < tile1 && ok; tile += RUNS ? 1 : gridDim.x) {
+    const long long sys0 = RUNS ? run_system(tile, K, NB, lc) : tile * G;
+    const bool next_bin = RUNS && sys0 == last + NB;
+    last = sys0;
     if (tid < GD) {  // row p = g D8 + a: entry a of system sys0 + g
       long long base = -1;
       const int g = tid / D8, a = tid - g * D8;
@@ -278,25 +261,25 @@ covariance_tcx_kernel(const float2* __restrict__ dop, double2* __restrict__ cov,
       }
       rowbase[tid] = base;
     }
-    if (PREC == kFP16S && warp == 0) {
-      if (lc) {   // the bins move down by one
+    if constexpr (RUNS) {   // the bins move down by one, or start again
+      if (warp == 0) {
         int m[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const int t = lane + 32 * i;
-          m[i] = shift && t + 1 < T ? smax[t + 1] : 0;
+          m[i] = next_bin && t + 1 < T ? smax[t + 1] : 0;
         }
         __syncwarp();
 #pragma unroll
         for (int i = 0; i < 4; ++i) smax[lane + 32 * i] = m[i];
-      } else {
-        for (int g = lane; g < G; g += 32) smax[g] = 0;
       }
+    } else {
+      if (PREC == kFP16S && tid < G) smax[tid] = 0;
     }
     __syncthreads();
     if constexpr (PREC == kFP16S) {   // each system's largest |re|, |im| over its B cells
       // two rows per warp and pass, so that both rows' loads are in flight together
-      for (int p0 = first_row + warp; p0 < GD; p0 += 2 * (kThreads / 32)) {
+      for (int p0 = (next_bin ? (T - 1) * C : 0) + warp; p0 < GD; p0 += 2 * (kThreads / 32)) {
         const int p1 = p0 + kThreads / 32;
         const long long base0 = rowbase[p0], base1 = p1 < GD ? rowbase[p1] : -1;
         float m0 = 0.f, m1 = 0.f;
@@ -314,15 +297,20 @@ covariance_tcx_kernel(const float2* __restrict__ dop, double2* __restrict__ cov,
         m0 = warp_max(m0);
         m1 = warp_max(m1);
         if (lane == 0) {   // m >= 0: int order
-          const int rows = lc ? C : D8;
-          if (base0 >= 0) atomicMax(&smax[p0 / rows], __float_as_int(m0));
-          if (base1 >= 0) atomicMax(&smax[p1 / rows], __float_as_int(m1));
+          if constexpr (RUNS) {   // (rows past D lie past the last bin)
+            if (p0 < D) atomicMax(&smax[p0 / C], __float_as_int(m0));
+            if (p1 < D) atomicMax(&smax[p1 / C], __float_as_int(m1));
+          } else {
+            atomicMax(&smax[p0 / D8], __float_as_int(m0));
+            if (p1 < GD) atomicMax(&smax[p1 / D8], __float_as_int(m1));
+          }
         }
       }
       __syncthreads();
       if (tid < G) {
         int m = smax[tid];
-        for (int t = 1; lc && t < T; ++t) m = max(m, smax[t]);
+        if constexpr (RUNS)
+          for (int t = 1; t < T; ++t) m = max(m, smax[t]);
         sscale[tid] = block_scale(__int_as_float(m));
       }
       __syncthreads();
@@ -581,7 +569,7 @@ template <int PREC, int NW>
 __global__ void __launch_bounds__(32 * NW, NW == 8 ? 2 : 1)
 apply_tcx_kernel(const float2* __restrict__ dop, const float2* __restrict__ wts,
                  float* __restrict__ out, int C, int K, int R, int ldr, int T, int B, int S, int NB,
-                 int NP, int tmem_cols, long long ntiles, int lc, DeviceStatus* __restrict__ status,
+                 int NP, int tmem_cols, long long ntiles, DeviceStatus* __restrict__ status,
                  int wait_polls) {
   using F = Fmt<PREC>;
   constexpr int KC = kAppRB / F::ESZ;         // K elements per chunk: 16 (tf32) or 32 (16-bit)
@@ -597,7 +585,7 @@ apply_tcx_kernel(const float2* __restrict__ dop, const float2* __restrict__ wts,
   __shared__ float wsc[128];                  // per weight vector scale (FP16S)
   __shared__ float winv[128];                 // its inverse times the tile's (exact: powers of two)
   __shared__ float xsc_s;
-  __shared__ int xmax[128];                   // per bin of the snapshot
+  __shared__ int xmax;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int D = C * T;
   const int K2 = 2 * D;
@@ -626,21 +614,9 @@ apply_tcx_kernel(const float2* __restrict__ dop, const float2* __restrict__ wts,
   bool ok = true;
   long long gch = 0;
 
-  // runs of bins (lc > 0: FP16S), or tiles dealt out in turn
-  if (PREC != kFP16S) lc = 0;
-  const long long t0 = lc ? ntiles * blockIdx.x / gridDim.x : blockIdx.x;
-  const long long t1 = lc ? ntiles * (blockIdx.x + 1) / gridDim.x : ntiles;
-  int last_k = -2, last_r0 = -1;
-  for (long long tile = t0; tile < t1 && ok; tile += lc ? 1 : gridDim.x) {
-    int k = (int)(tile / tiles_per_k);
-    int r0 = (int)(tile - (long long)k * tiles_per_k) * 128;
-    if (lc) {
-      run_tile(tile, K, tiles_per_k, lc, k, r0);
-      r0 *= 128;
-    }
-    const bool shift = r0 == last_r0 && k == last_k + 1;   // all bins but the last are known
-    last_k = k;
-    last_r0 = r0;
+  for (long long tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+    const int k = (int)(tile / tiles_per_k);
+    const int r0 = (int)(tile - (long long)k * tiles_per_k) * 128;
     const int b0 = r0 / B;
     if (tid < D) {
       const int t = tid / C, c = tid - t * C;
@@ -650,60 +626,34 @@ apply_tcx_kernel(const float2* __restrict__ dop, const float2* __restrict__ wts,
       const int q = tid >> 1, j = q / S, s = q - j * S;
       if (tid < 256) wbase[tid] = (tid < NP && q < Nq && b0 + j < NB) ? ((((long long)k * NB + b0 + j) * S + s) * D) : -1;
     }
-    if (PREC == kFP16S && warp == 0) {   // the bins move down by one, or start again
-      int m[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int t = lane + 32 * i;
-        m[i] = shift && t + 1 < T ? xmax[t + 1] : 0;
-      }
-      __syncwarp();
-#pragma unroll
-      for (int i = 0; i < 4; ++i) xmax[lane + 32 * i] = m[i];
-    }
+    if (PREC == kFP16S && tid == 0) xmax = 0;
     __syncthreads();
     if constexpr (PREC == kFP16S) {   // the tile's largest |x| component, each vector's largest |w|
+      float m = 0.f;
       const int rn = min(128, R - r0);
-      // a warp per row: 4 cells per lane
-      for (int d = (shift ? (T - 1) * C : 0) + warp; d < D; d += NW) {
-        const float2* x = dop + colbase[d] + r0;
-        float m = 0.f;
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          if (lane + 32 * i < rn) {
-            const float2 v = __ldg(x + lane + 32 * i);
-            m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
-          }
-        m = warp_max(m);
-        if (lane == 0) atomicMax(&xmax[d / C], __float_as_int(m));   // m >= 0: int order
+#pragma unroll 16
+      for (int e = tid; e < D * 128; e += (32 * NW)) {   // entry d = e / 128 of cell e % 128
+        const int d = e >> 7, mm = e & 127;
+        if (mm < rn) {
+          const float2 v = __ldg(dop + colbase[d] + r0 + mm);
+          m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
+        }
       }
-      // four vectors per warp at once, so that their loads are in flight together
-      for (int q = warp; q < Nq; q += 4 * NW) {
-        long long wb[4];
-        float mw[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          wb[i] = q + NW * i < Nq ? wbase[2 * (q + NW * i)] : -1;
-          mw[i] = 0.f;
-        }
-#pragma unroll 2
-        for (int d = lane; d < D; d += 32)
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (wb[i] >= 0) {
-              const float2 w = __ldg(wts + wb[i] + d);
-              mw[i] = fmaxf(mw[i], fmaxf(fabsf(w.x), fabsf(w.y)));
-            }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          mw[i] = warp_max(mw[i]);
-          if (lane == 0 && q + NW * i < Nq) wsc[q + NW * i] = block_scale(mw[i]);
-        }
+      m = warp_max(m);
+      if (lane == 0) atomicMax(&xmax, __float_as_int(m));
+      for (int q = warp; q < Nq; q += (32 * NW) / 32) {
+        const long long wb = wbase[2 * q];
+        float mw = 0.f;
+        if (wb >= 0)
+          for (int d = lane; d < D; d += 32) {
+            const float2 w = __ldg(wts + wb + d);
+            mw = fmaxf(mw, fmaxf(fabsf(w.x), fabsf(w.y)));
+          }
+        mw = warp_max(mw);
+        if (lane == 0) wsc[q] = block_scale(mw);
       }
       __syncthreads();
-      int xm = xmax[0];
-      for (int t = 1; t < T; ++t) xm = max(xm, xmax[t]);
-      const float xs = block_scale(__int_as_float(xm));
+      const float xs = block_scale(__int_as_float(xmax));
       if (tid == 0) xsc_s = xs;
       if (tid < Nq) winv[tid] = 1.f / (wsc[tid] * xs);   // powers of two: exact
       __syncthreads();
@@ -941,7 +891,8 @@ cudaError_t launch_cov_form(const float2* dop, double2* cov, int C, int K, int R
   if (per_sm > 512 / CovForm<STK>::COLS) per_sm = 512 / CovForm<STK>::COLS;
   const long long cap = 152LL * per_sm;
   const long long blocks = ntiles < cap ? ntiles : cap;
-  const int lc = G == 1 ? run_length<PREC>(ntiles, blocks, K, T) : 0;
+  const long long per_cta = (ntiles + blocks - 1) / blocks;
+  const int lc = (int)(per_cta < K ? per_cta : K);
   return launch_or_defer(s, [=](cudaStream_t st) {
     covariance_tcx_kernel<PREC, STK><<<(unsigned)blocks, kThreads, smem, st>>>(
         dop, cov, C, K, ldr, T, B, NB, D8, G, ntiles, lc, lower_only ? 1 : 0, status, wait_polls);
@@ -979,10 +930,9 @@ cudaError_t launch_app_nw(const float2* dop, const float2* wts, float* out, int 
   if (per_sm > 512 / cols) per_sm = 512 / cols;
   const long long cap = 152LL * per_sm;
   const long long blocks = ntiles < cap ? ntiles : cap;
-  const int lc = run_length<PREC>(ntiles, blocks, K, T);
   return launch_or_defer(s, [=](cudaStream_t st) {
     apply_tcx_kernel<PREC, NW><<<(unsigned)blocks, 32 * NW, smem, st>>>(dop, wts, out, C, K, R, ldr, T, B, S,
-                                                                   NB, NP, cols, ntiles, lc, status,
+                                                                   NB, NP, cols, ntiles, status,
                                                                    wait_polls);
     return cudaGetLastError();
   });

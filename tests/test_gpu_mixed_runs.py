@@ -1,7 +1,7 @@
-"""FP16S tensor-core kernels on runs of bins: a CTA that walks consecutive bins
-of the same range cells keeps the maxima of the bins that the snapshots share.
-A maximum is exact, so the results equal, bit for bit, those of small pieces of
-the range axis, where every tile finds its own."""
+"""The FP16S covariance's runs of bins: a CTA that walks consecutive bins of the
+same range cells keeps the maxima of the bins that the snapshots share.  A
+maximum is exact, so the results (and the apply's) equal, bit for bit, those of
+small pieces of the range axis, where a CTA has one tile."""
 import numpy as np
 import pytest
 import torch
@@ -21,11 +21,11 @@ def _plan(dims):
     return plan
 
 
-# split and stacked forms, several systems per tile (no runs in the covariance),
-# tiles across blocks, runs as long as the bins with every bin in each snapshot
+# split and stacked forms, several systems per tile, tiles across blocks, every
+# bin in each snapshot with runs as long as the bins
 @pytest.mark.parametrize("C,T,K,R,B,S", [(32, 4, 128, 1024, 128, 8), (16, 4, 128, 1280, 64, 5),
                                          (9, 5, 64, 4608, 96, 3), (4, 3, 64, 8192, 64, 4),
-                                         (8, 8, 8, 16384, 128, 6), (30, 3, 64, 2560, 256, 33)])
+                                         (8, 8, 8, 16384, 128, 6), (12, 8, 8, 16384, 128, 3), (30, 3, 64, 2560, 256, 33)])
 def test_runs_equal_small_pieces(C, T, K, R, B, S):
     rng = np.random.default_rng(C * K)
     dop = (rng.standard_normal((C, K, R)) + 1j * rng.standard_normal((C, K, R)))
