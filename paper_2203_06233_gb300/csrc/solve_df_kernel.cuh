@@ -64,9 +64,11 @@
 //   D =  15, 3840 systems,  C 5  S 11       258,   117 (no grids)
 //   D =  12, 16384 systems, C 4  S 16       324,   160 (no grids)
 //   D =  12, 256 systems,   C 4  S 4      103.5,    21 (no grids)
-// What bounds it at D = 128: 62% of the issue slots in use, half of the rest
-// fixed-latency waits at four warps per scheduler (shared memory holds one
-// system per SM), then shared-memory latency and barriers.
+// What bounds it at D = 128: issue, 74% of the slots in use by four warps per
+// scheduler (shared memory holds one system per SM), the sums' own
+// instructions a third of all slots; masked lanes of the diagonal blocks,
+// renormalisations, the shuffles that broadcast a column's entry and the loads
+// take the rest.
 //
 // F32F (STAP_SOLVE_MIXED_IR): the factor and the substitutions in FP32, the
 // residual and the solution in double-float as above.
