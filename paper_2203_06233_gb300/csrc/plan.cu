@@ -1368,11 +1368,12 @@ stap_status stap_plan_autotune(stap_plan p, const void* const* cubes, float* con
       if (mixed) c.tune.cov_kind = 1;   // tune the FP32 kernel first
       std::vector<int> kts;
       for (int kt = 1; kt <= 32 && kt <= d.n_dop; kt *= 2) kts.push_back(kt);
+      // as the run writes them: lower triangles
       pick([](stap::Tune& t, int v) { t.cov_kt = v; }, kts,
-           [&] { return do_covariance(p, c, dop, cov, p->stream); });
+           [&] { return do_covariance(p, c, dop, cov, p->stream, -1, true); });
       if (mixed)   // then keep the tensor cores only where they are faster
         pick([](stap::Tune& t, int v) { t.cov_kind = v; }, {2, 1},
-             [&] { return do_covariance(p, c, dop, cov, p->stream); });
+             [&] { return do_covariance(p, c, dop, cov, p->stream, -1, true); });
     }
     if ((st = do_covariance(p, c, dop, cov, p->stream)) != STAP_OK) break;
     // FP64 solves have launch choices; the double-float ones (faster wherever
@@ -1446,8 +1447,8 @@ stap_status stap_plan_autotune(stap_plan p, const void* const* cubes, float* con
         return ms;
       };
       constexpr int kRounds = 7;
-      constexpr int kCands = 6;
-      const int cands[kCands] = {1, 2, 3, 4, 6, 8};
+      constexpr int kCands = 4;
+      const int cands[kCands] = {1, 2, 4, 8};
       float per_round[kCands][kRounds];
       // a CPI of tens of milliseconds gains nothing from overlapping its
       // short steps: one cold run decides whether to look at all
