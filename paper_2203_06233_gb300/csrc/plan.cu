@@ -48,6 +48,7 @@ struct Cpi {
   std::vector<double> steer;    // [S][D][2]
   // steer[s] = g (x) a_s for the default table: temporal factor g [T][2] and
   // spatial factors a [S][C][2]; cleared when the caller replaces the table
+  // (all of them scaled: finish_steering)
   bool separable = false;
   bool sep_sym = false;   // sep_a_ff[S-1-s] is conj(sep_a_ff[s]) bit for bit
   std::vector<double> sep_g, sep_a;
@@ -111,6 +112,56 @@ bool conj_symmetric(const std::vector<float>& a_ff, int S, int C) {
   return true;
 }
 
+// The exponent of the largest |re|, |im| of n numbers (0 where they are all
+// zero, or not all finite), and the numbers with that exponent taken out.
+int top_exponent(const double* x, size_t n) {
+  double m = 0.0;
+  for (size_t i = 0; i < n; ++i) m = std::max(m, std::fabs(x[i]));
+  return m > 0.0 && std::isfinite(m) ? std::ilogb(m) : 0;
+}
+void scale_down(double* x, size_t n, int e) {
+  for (size_t i = 0; i < n; ++i) x[i] = std::scalbn(x[i], -e);
+}
+
+// The weights u / sqrt(v^H u) do not depend on the steering vector's scale, so
+// every table is kept with the power of two of its largest entry taken out:
+// exact, nothing to undo, and neither the double-floats that the solves read
+// nor the products v^H u, which are FP32 products there, leave FP32's range
+// whatever the magnitudes that the caller's table or front end has.
+//
+// An arbitrary table: each vector by itself.
+void finish_steering(Cpi& c) {
+  const size_t n = 2 * (size_t)c.D;
+  for (int s = 0; s < c.d.n_steering; ++s) {
+    double* v = c.steer.data() + s * n;
+    scale_down(v, n, top_exponent(v, n));
+  }
+  to_ff(c.steer, c.steer_ff);
+  c.separable = false;
+}
+
+// v_s = g (x) a_s from the temporal and spatial factors, each scaled.
+void finish_separable(Cpi& c) {
+  const int C = c.d.n_chan, S = c.d.n_steering, T = c.d.tdof, D = c.D;
+  scale_down(c.sep_g.data(), 2 * (size_t)T, top_exponent(c.sep_g.data(), 2 * (size_t)T));
+  for (int s = 0; s < S; ++s) {
+    double* a = &c.sep_a[2 * (size_t)s * C];
+    scale_down(a, 2 * (size_t)C, top_exponent(a, 2 * (size_t)C));
+    for (int t = 0; t < T; ++t)
+      for (int ch = 0; ch < C; ++ch) {
+        const double gr = c.sep_g[2 * t], gi = c.sep_g[2 * t + 1], ar = a[2 * ch], ai = a[2 * ch + 1];
+        double* v = &c.steer[2 * ((size_t)s * D + t * C + ch)];
+        v[0] = gr * ar - gi * ai;
+        v[1] = gr * ai + gi * ar;
+      }
+  }
+  to_ff(c.steer, c.steer_ff);
+  to_ff(c.sep_a, c.sep_a_ff);
+  to_ff(c.sep_g, c.g_ff);
+  c.separable = true;
+  c.sep_sym = conj_symmetric(c.sep_a_ff, S, C);
+}
+
 void make_tables(Cpi& c) {
   const stap_dims& d = c.d;
   const int K = d.n_dop, T = d.tdof, C = d.n_chan, S = d.n_steering;
@@ -142,8 +193,7 @@ void make_tables(Cpi& c) {
     gr[t] = sr;
     gi[t] = si;
   }
-  const int D = c.D;
-  c.steer.assign(2 * (size_t)S * D, 0.0);
+  c.steer.assign(2 * (size_t)S * c.D, 0.0);
   c.sep_g.assign(2 * (size_t)T, 0.0);
   c.sep_a.assign(2 * (size_t)S * C, 0.0);
   for (int t = 0; t < T; ++t) {
@@ -158,19 +208,8 @@ void make_tables(Cpi& c) {
       c.sep_a[2 * ((size_t)s * C + ch)] = std::cos(a);
       c.sep_a[2 * ((size_t)s * C + ch) + 1] = std::sin(a);
     }
-    for (int t = 0; t < T; ++t)
-      for (int ch = 0; ch < C; ++ch) {
-        const double ar = c.sep_a[2 * ((size_t)s * C + ch)], ai = c.sep_a[2 * ((size_t)s * C + ch) + 1];
-        double* v = &c.steer[2 * ((size_t)s * D + t * C + ch)];
-        v[0] = gr[t] * ar - gi[t] * ai;
-        v[1] = gr[t] * ai + gi[t] * ar;
-      }
   }
-  c.separable = true;
-  to_ff(c.steer, c.steer_ff);
-  to_ff(c.sep_a, c.sep_a_ff);
-  to_ff(c.sep_g, c.g_ff);
-  c.sep_sym = conj_symmetric(c.sep_a_ff, S, C);
+  finish_separable(c);
 }
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
@@ -1011,8 +1050,7 @@ stap_status stap_plan_set_steering(stap_plan p, int32_t cpi, const double* host_
   for (size_t i = 0; i < c.steer.size(); ++i)
     if (!std::isfinite(host_c128[i])) return STAP_ERR_INVALID_ARG;
   std::memcpy(c.steer.data(), host_c128, c.steer.size() * sizeof(double));
-  to_ff(c.steer, c.steer_ff);
-  c.separable = false;  // an arbitrary table: solve for every steering vector
+  finish_steering(c);   // an arbitrary table: solve for every steering vector
   drop_graph(p);        // the captured launches chose the solve variant
   return upload_tables(p, cpi);
 }
@@ -1170,7 +1208,7 @@ stap_status stap_plan_set_front_end(stap_plan p, int32_t n_elem, const double* W
   if (p->ws || p->fe_N) return STAP_ERR_INVALID_ARG;   // once, before the workspace
   Cpi& c = p->cpis[0];
   const stap_dims& d = c.d;
-  const int C = d.n_chan, N = n_elem, S = d.n_steering, T = d.tdof, D = c.D;
+  const int C = d.n_chan, N = n_elem, S = d.n_steering;
   const size_t PR8 = (size_t)d.n_pulses * d.n_range * 8;
   if ((size_t)N * PR8 > ((size_t)1 << 44)) return STAP_ERR_UNSUPPORTED;
   for (size_t i = 0; i < 2 * (size_t)C * N; ++i)
@@ -1198,19 +1236,8 @@ stap_status stap_plan_set_front_end(stap_plan p, int32_t n_elem, const double* W
       c.sep_a[2 * ((size_t)s * C + ch)] = br;
       c.sep_a[2 * ((size_t)s * C + ch) + 1] = bi;
     }
-    for (int t = 0; t < T; ++t)
-      for (int ch = 0; ch < C; ++ch) {
-        const double gr = c.sep_g[2 * t], gi = c.sep_g[2 * t + 1];
-        const double ar = c.sep_a[2 * ((size_t)s * C + ch)], ai = c.sep_a[2 * ((size_t)s * C + ch) + 1];
-        double* v = &c.steer[2 * ((size_t)s * D + t * C + ch)];
-        v[0] = gr * ar - gi * ai;
-        v[1] = gr * ai + gi * ar;
-      }
   }
-  c.separable = true;
-  to_ff(c.steer, c.steer_ff);
-  to_ff(c.sep_a, c.sep_a_ff);
-  c.sep_sym = conj_symmetric(c.sep_a_ff, S, C);
+  finish_separable(c);
   p->fe_w.resize(2 * (size_t)C * N);
   for (size_t i = 0; i < p->fe_w.size(); ++i) p->fe_w[i] = (float)W[i];
   p->fe_N = N;

@@ -1,0 +1,51 @@
+"""The weight solve where the double-float kernels could leave the 64-bit
+weights: steering tables and loads of any magnitude, beams that point along the
+interference (the separable combination cancels), the weakest loads they
+accept, and Hermitian inputs that are not quite covariances."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2203_06233_gb300 import stap
+
+from test_gpu_solve_df import TOL, _check, _covariances, _default_steering, _reference, _solve
+
+pytestmark = pytest.mark.gpu
+
+BIG_AND_SMALL = [(4, 3), (5, 3), (16, 4), (32, 4)]
+
+
+@pytest.mark.parametrize("solver", [stap.STAP_SOLVE_FP64, stap.STAP_SOLVE_MIXED_IR], ids=["default", "mixed_ir"])
+@pytest.mark.parametrize("C,T", BIG_AND_SMALL)
+def test_weights_do_not_depend_on_the_steering_tables_scale(C, T, solver):
+    """w = u / sqrt(v^H u): every finite table gives the weights of its
+    directions, to the tolerance of the unscaled one."""
+    D, S = C * T, 5
+    R = _covariances(8, D, seed=D)
+    v = _default_steering(C, T, S) * np.exp(1j * np.arange(D))
+    ref = _reference(R, v, 1e-3)
+    scales = [np.full(S, s) for s in (1e-320, 1e-300, 1e-30, 1e-20, 1e20, 1e30, 1e300)]
+    scales.append(np.array([1e-30, 1.0, 1e30, 1e-200, 1e200]))     # one table, many magnitudes
+    for s in scales:
+        t = v * 1e10 * (s * 1e-10)[:, None] if s.min() > 1e-305 else v * s[:, None]
+        want = ref if s.min() > 1e-305 else _reference(R, t * 2.0 ** 1000, 1e-3)   # subnormal entries are rounded
+        w, status = _solve(R, C, T, S, t, solver=solver, refine_steps=2)
+        assert status == (stap.STAP_OK, 0)
+        _check(w, want)
+
+
+@pytest.mark.parametrize("gain", [1e-30, 1e-22, 1e22, 1e30])
+def test_weights_do_not_depend_on_the_front_ends_scale(gain):
+    """The separable table of a front end, v_s = g (x) W^H a_s."""
+    C, T, S, N = 4, 3, 9, 12
+    W = np.zeros((C, N))
+    for c in range(C):
+        W[c, 3 * c:3 * c + 3] = 1.0
+    R = torch.from_numpy(_covariances(8, C * T, seed=1).reshape(8, 1, C * T, C * T)).cuda()
+    out = []
+    for g in (1.0, gain):
+        plan = stap.Plan((C, 8, 8, 4, T, 4, S), front_end=W * g)
+        out.append(plan.solve_weights(R).cpu().numpy().reshape(8, S, C * T))
+        assert plan.status() == (stap.STAP_OK, 0)
+        plan.close()
+    _check(out[1], out[0])
