@@ -36,7 +36,7 @@
 // the FP64 kernels' (both are the complex64 rounding).
 //
 // Range.  Floats span 2^+-126 only, so each system is scaled by the even
-// power of two 2^-e that brings its trace into [1, 4): the conversion from
+// power of two 2^-e that brings Rl's trace into [1, 4): the conversion from
 // FP64 adds -e to the exponent field (no instruction more), and the weights
 // take 2^(-e/2) back with their normalisation.  Entries below 2^-73 of the
 // trace become zero; an infinity or NaN becomes a NaN, which no pivot test
@@ -987,8 +987,8 @@ __device__ __forceinline__ void solve_df_body(const SolveDfParams& prm, long lon
       if (in_bounds(y.a0 + (long long)j * D + j, y.aext, kSiteSolveIn)) tr += __ldg(&y.A[(size_t)j * D + j].x);
     tr = lanes_sum<TW>(tr);
     y.delta = prm.load_factor * tr * (1.0 / D);
-    // scale 2^-e, e even, trace 2^-e in [1, 4)
-    const int et = (int)(((uint32_t)__double2hiint(tr) >> 20) & 0x7FF);
+    // scale 2^-e, e even, trace of Rl 2^-e in [1, 4)
+    const int et = (int)(((uint32_t)__double2hiint(fma(prm.load_factor, tr, tr)) >> 20) & 0x7FF);
     const int e = et == 0 || et == 0x7FF ? 0 : (et - 1023) & ~1;
     y.sbase = 896 + e;
     factor<TEAM, F32F, square<LR, RPL>()>(y, D);

@@ -49,3 +49,17 @@ def test_weights_do_not_depend_on_the_front_ends_scale(gain):
         assert plan.status() == (stap.STAP_OK, 0)
         plan.close()
     _check(out[1], out[0])
+
+
+@pytest.mark.parametrize("lf", [1e3, 1e20, 1e38, 1e42, 1e100])
+@pytest.mark.parametrize("C,T", BIG_AND_SMALL)
+def test_loads_of_any_strength(C, T, lf):
+    """Rl is scaled by its own trace, load included; R is scaled so that the
+    weights stay inside complex64."""
+    D, S = C * T, 5
+    R = _covariances(8, D, seed=D) / lf
+    for steer in (None, _default_steering(C, T, S) * np.exp(1j * np.arange(D))):
+        v = _default_steering(C, T, S) if steer is None else steer
+        w, status = _solve(R, C, T, S, steer, load_factor=lf)
+        assert status == (stap.STAP_OK, 0)
+        _check(w, _reference(R, v, lf))
