@@ -51,6 +51,7 @@ struct Cpi {
   // (all of them scaled: finish_steering)
   bool separable = false;
   bool sep_sym = false;   // sep_a_ff[S-1-s] is conj(sep_a_ff[s]) bit for bit
+  double g_norm = 0.0, steer_sum = 0.0;   // |g|_2, the largest sum of |re| + |im| of a v_s (rounded up)
   std::vector<double> sep_g, sep_a;
   std::vector<float> steer_ff, sep_a_ff, g_ff;   // the tables as double-floats [..][4]
   size_t steer_ff_off = 0, a_ff_off = 0, g_ff_off = 0;
@@ -154,6 +155,14 @@ void finish_separable(Cpi& c) {
         v[0] = gr * ar - gi * ai;
         v[1] = gr * ai + gi * ar;
       }
+  }
+  c.g_norm = c.steer_sum = 0.0;
+  for (double x : c.sep_g) c.g_norm += x * x;
+  c.g_norm = 1.0001 * std::sqrt(c.g_norm);
+  for (int s = 0; s < S; ++s) {
+    double sum = 0.0;
+    for (int i = 0; i < 2 * D; ++i) sum += std::fabs(c.steer[2 * (size_t)s * D + i]);
+    c.steer_sum = std::max(c.steer_sum, 1.0001 * sum);
   }
   to_ff(c.steer, c.steer_ff);
   to_ff(c.sep_a, c.sep_a_ff);
@@ -384,7 +393,7 @@ stap_status do_solve(stap_plan p, const Cpi& c, const void* cov, void* wts, cuda
       c.separable ? p->at<const float4>(c.a_ff_off) : nullptr,
       c.separable ? p->at<const float4>(c.g_ff_off) : nullptr, (long long)d.n_dop * nb, c.D,
       d.n_steering, d.n_chan, p->opt.load_factor, p->opt.refine_steps, p->opt.solver, p->status(),
-      st, c.tune, c.separable && c.sep_sym));
+      st, c.tune, c.separable && c.sep_sym, c.g_norm, c.steer_sum));
 }
 
 stap_status do_apply(stap_plan p, const Cpi& c, const void* dop, const void* wts, float* out,
@@ -1405,7 +1414,7 @@ stap_status stap_plan_autotune(stap_plan p, const void* const* cubes, float* con
     if ((st = do_covariance(p, c, dop, cov, p->stream)) != STAP_OK) break;
     // FP64 solves have launch choices; the double-float ones (faster wherever
     // they may stand in) have none
-    if (stap::solve_df_eligible(p->opt.solver, p->opt.load_factor, c.D)) {
+    if (stap::solve_df_eligible(p->opt.solver, p->opt.load_factor, c.D, p->opt.refine_steps)) {
       c.tune.solve_kind = c.tune.solve_ts = c.tune.solve_nw = c.tune.solve_lr = 0;
     } else if (c.D <= stap::kSmallMaxD) {
       const int nrhs = c.separable ? d.n_chan : d.n_steering;

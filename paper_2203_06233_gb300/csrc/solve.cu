@@ -31,6 +31,8 @@
 // from S to C right-hand sides.  The combination stays in FP64: u_s can be
 // two orders of magnitude smaller than the terms it sums (steering vectors
 // near the clutter ridge), so FP32 there costs ~1e-4 in the weights.
+#include <algorithm>
+
 #include "df64.cuh"
 #include "batch.cuh"
 #include "checked.cuh"
@@ -1186,14 +1188,15 @@ cudaError_t launch_solve(const double2* cov, float2* wts, const double2* steer,
                          const double2* sep_g, const double2* sep_a, const float4* steer_ff,
                          const float4* sep_a_ff, const float4* g_ff, long long nsys, int D, int S,
                          int C, double load_factor, int refine_steps, int solver,
-                         DeviceStatus* status, cudaStream_t s, const Tune& tn, bool sep_sym) {
+                         DeviceStatus* status, cudaStream_t s, const Tune& tn, bool sep_sym, double g_norm,
+                         double steer_sum) {
   if (nsys <= 0) return cudaSuccess;
   if (D < 1 || D > kMaxD || S < 1) return cudaErrorInvalidValue;
   const bool sep = sep_g != nullptr && sep_a != nullptr && steer_ff != nullptr && sep_a_ff != nullptr &&
                    C >= 1 && C <= 32 && D % C == 0;
   // the double-float kernels where the load allows them (solve_df.cuh), unless
   // the tuning names one of the FP64 kernels (solve_kind 1 to 3)
-  if (solve_df_eligible(solver, load_factor, D) && (solver == 1 || tn.solve_kind == 0) &&
+  if (solve_df_eligible(solver, load_factor, D, refine_steps) && (solver == 1 || tn.solve_kind == 0) &&
       steer_ff != nullptr) {
     // the C basis right-hand sides where they are fewer than the S steering vectors
     const bool dsep = sep && g_ff != nullptr && C < S;
@@ -1210,6 +1213,9 @@ cudaError_t launch_solve(const double2* cov, float2* wts, const double2* steer,
     p.sep = dsep ? 1 : 0;
     p.sym = dsep && sep_sym ? 1 : 0;
     p.load_factor = load_factor;
+    p.cancel = (float)std::min(1.0 / (2097152.0 * load_factor), 1e30);   // half a complex64 rounding of u_s
+    p.cancel_q = (float)std::min(C * g_norm * steer_sum * p.cancel, 1e38);
+    p.steer_sum = (float)steer_sum;
     p.refine_steps = refine_steps;
     p.status = status;
     if (solver == 1) return D <= kSmallMaxD ? launch_solve_df_small_ir(p, s) : launch_solve_df_big_ir(p, s);

@@ -12,10 +12,14 @@ namespace stap {
 constexpr double kDfMaxKappa = 524288.0;   // 2^19
 
 // Whether a plan's solve takes these kernels: the refinement option, and the
-// default solver where the load bounds the condition number.
-inline bool solve_df_eligible(int solver, double load_factor, int D) {
+// default solver where the load bounds the condition number.  Without a
+// refinement step, on grids (D > 32), the bound is a quarter of that: a vector
+// along strong interference loses up to kappa 2^-42 (measured at D = 128: 3e-7 at
+// kappa 2^19, 8e-8 at 2^17).
+inline bool solve_df_eligible(int solver, double load_factor, int D, int refine_steps) {
+  const double most = refine_steps == 0 && D > kSmallMaxD ? kDfMaxKappa / 4 : kDfMaxKappa;
   return solver == STAP_SOLVE_MIXED_IR ||
-         (load_factor > 0.0 && (double)D / load_factor + 1.0 <= kDfMaxKappa);
+         (load_factor > 0.0 && (double)D / load_factor + 1.0 <= most);
 }
 
 // Parameters of one launch (one CPI); gx = the launch's grid size.
@@ -25,6 +29,11 @@ struct SolveDfParams {
   const float4* steer_ff;  // [S][D] steering vectors (re hi, re lo, im hi, im lo)
   const float4* g_ff;      // [T] temporal factors (separable steering)
   const float4* sep_a_ff;  // [S][C] spatial factors (separable steering)
+  // separable steering: a u_s whose largest entry is below `cancel` times the
+  // sum of the basis solutions' largest needs a solve of its own; one with q =
+  // Re v^H u of cancel_q / delta or more cannot be
+  float cancel, cancel_q;
+  float steer_sum;         // the largest sum of |re| + |im| over a steering vector
   long long nsys;
   int D, S, C;
   int sep;                 // solve the C basis right-hand sides g (x) e_c

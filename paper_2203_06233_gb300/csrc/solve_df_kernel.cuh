@@ -260,6 +260,12 @@ __device__ __forceinline__ ff::F2 lanes_sum2(float s, float e) {
 __device__ __forceinline__ bool usable(ff::F2 q) { return q.hi > 0.f && isfinite(q.hi); }
 
 template <int W>
+__device__ __forceinline__ float lanes_max(float v) {
+  for (int o = W / 2; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+
+template <int W>
 __device__ __forceinline__ double lanes_sum(double v) {
   for (int o = W / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
@@ -417,8 +423,9 @@ __device__ __forceinline__ void ldl_solve_f32(Cdf (&x)[RPL], const float2* L, co
 // than 12 rows, where that would cost a third of the resident warps (D = 15:
 // 197 -> 160 us per 3840 systems), as the lower triangle packed like the factor), the two pivot columns before division
 // [2][D] (in the chunk's place: the factorisation is over before the first
-// residual), the factor [Dp] (column-major packed), the pivot reciprocals [D]
-// and the pivot flag.
+// residual), the factor
+// [Dp] (column-major packed), the pivot reciprocals [D], the pivot flag and
+// whether a steering vector's combination cancels.
 template <int LR, int RPL>
 __host__ __device__ constexpr bool square() { return LR * RPL <= 12; }
 
@@ -548,7 +555,7 @@ __device__ __forceinline__ void factor(const System y, int D) {
       while (l > i) l -= ++i;
     }
   }
-  if (tt == 0) *okf = 1;
+  if (tt == 0) okf[0] = 1, okf[1] = 0;
   team_sync<TEAM>();
 
   for (int j = 0; j < D; j += 2) {
@@ -699,16 +706,22 @@ __device__ __forceinline__ void factor(const System y, int D) {
   }
 }
 
-// Solve and refine the right-hand sides r0 .. r0 + TEAM / LR - 1, one per group
-// of LR lanes, into U (row rhs of it, or row g where U holds one pass only).
+// What a group of LR lanes solves in a pass: steering vector rhs itself
+// (direct) or basis vector rhs, into row `row` of U; a group without one of its
+// own (!live) computes a copy that is never stored.
+struct Rhs {
+  int rhs, row;
+  bool live, direct;
+  bool work;   // a CTA team's warps without right-hand sides only help convert
+};
+
+// Solve and refine a pass of right-hand sides, one per group of LR lanes.
 template <int LR, int RPL, int TEAM, bool F32F>
-__device__ __forceinline__ void solve_rhs(const SolveDfParams& prm, const System y, int r0) {
+__device__ __forceinline__ void solve_rhs(const SolveDfParams& prm, const System y, const Rhs z) {
   constexpr int EPT = (KC * LR * RPL + TEAM - 1) / TEAM;   // chunk entries per thread
   using SH = Shared<TEAM, F32F, square<LR, RPL>()>;
   extern __shared__ float4 smdf[];
-  const int D = prm.D, C = prm.C, refine_steps = prm.refine_steps;
-  const bool sep = prm.sep != 0;
-  const int nrhs = sep ? C : prm.S;
+  const int D = prm.D, C = prm.C;
   const SH sh(D, y.nu);
   char* base = reinterpret_cast<char*>(smdf) + y.off;
   float4* U = reinterpret_cast<float4*>(base + sh.u);
@@ -716,21 +729,19 @@ __device__ __forceinline__ void solve_rhs(const SolveDfParams& prm, const System
   const typename SH::LT* L = reinterpret_cast<const typename SH::LT*>(base + sh.l);
   const float2* rd = reinterpret_cast<const float2*>(base + sh.rd);
   constexpr bool GRID = grids<TEAM, F32F>();
-  const int tt = team_thread<TEAM>(), li = tt % LR, g = tt / LR;
+  const int tt = team_thread<TEAM>(), li = tt % LR;
   const int gbase = (threadIdx.x & 31) - li;       // first lane of this thread's group
-  // a CTA team's warps past the last right-hand side only help convert
-  const bool work = TEAM <= 32 || r0 + (tt >> 5) * (32 / LR) < nrhs;
-  const bool live = r0 + g < nrhs;
-  const int rhs = live ? r0 + g : nrhs - 1;    // a spare group computes a copy, never stored
-  float4* Ur = U + (size_t)(sep ? rhs : g) * D;   // its solution
+  const bool work = z.work, live = z.live;
+  const int rhs = z.rhs;
+  float4* Ur = U + (size_t)z.row * D;              // its solution
   auto b_at = [&](int i) -> Cdf {              // right-hand side entry
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);   // tables: (re hi, re lo, im hi, im lo)
     if (i < D) {
-      if (sep) {
+      if (z.direct) {
+        v = __ldg(prm.steer_ff + (size_t)rhs * D + i);
+      } else {
         const int t = i / C;
         if (i - t * C == rhs) v = __ldg(prm.g_ff + t);
-      } else {
-        v = __ldg(prm.steer_ff + (size_t)rhs * D + i);
       }
     }
     return Cdf{v.x, v.y, v.z, v.w};
@@ -769,7 +780,9 @@ __device__ __forceinline__ void solve_rhs(const SolveDfParams& prm, const System
         }
       }
     }
-    if (it == refine_steps) break;
+    // (a vector whose combination cancels takes one refinement step at least: its
+    // small solution loses up to kappa(Rl) 2^-46 to the unrefined solve)
+    if (it == (!F32F && z.direct && prm.sep != 0 ? max(prm.refine_steps, 1) : prm.refine_steps)) break;
     // x = b - Rl u
 #pragma unroll
     for (int q = 0; q < RPL; ++q) x[q] = b_at(li + LR * q);
@@ -838,16 +851,14 @@ __device__ __forceinline__ void solve_rhs(const SolveDfParams& prm, const System
 // and combine() are calls: inlined, their registers cost the substitutions
 // theirs; 3% on a D = 128 system.)
 template <int LR, int RPL, int TEAM>
-__device__ __noinline__ void emit(const SolveDfParams& prm, int off, long long sys, bool valid, bool ok, int e,
-                                  int r0) {
+__device__ __noinline__ void emit(const SolveDfParams& prm, int off, long long sys, bool store, bool ok, int e,
+                                  int rhs, int row) {
   extern __shared__ float4 smdf[];
-  const int D = prm.D, S = prm.S, nrhs = S;
+  const int D = prm.D, S = prm.S;
   const long long nsys = prm.nsys;
   float2* __restrict__ wts = prm.wts;
-  const int tt = team_thread<TEAM>(), li = tt % LR, g = tt / LR;
-  const bool live = r0 + g < nrhs;
-  const int rhs = live ? r0 + g : nrhs - 1;
-  const float4* Ur = smdf + off / 16 + (size_t)g * D;
+  const int tt = team_thread<TEAM>(), li = tt % LR;
+  const float4* Ur = smdf + off / 16 + (size_t)row * D;
   float qs = 0.f, qe = 0.f;
 #pragma unroll
   for (int q = 0; q < RPL; ++q) {
@@ -861,7 +872,7 @@ __device__ __noinline__ void emit(const SolveDfParams& prm, int off, long long s
   const ff::F2 qd = lanes_sum2<LR>(qs, qe);
   const bool good = ok && usable(qd);
   const Gain sf = gain(qd, -e / 2);
-  if (valid && live) {
+  if (store) {
     const long long w0 = (sys * S + rhs) * D;
 #pragma unroll
     for (int q = 0; q < RPL; ++q) {
@@ -876,8 +887,26 @@ __device__ __noinline__ void emit(const SolveDfParams& prm, int off, long long s
 
 // Separable steering: u_s = sum_c a_s[c] U_c from the team's basis solutions U
 // (at byte `off` of shared memory) and the normalised weights.
-template <int LR, int RPL, int TEAM>
-__device__ __noinline__ void combine(const SolveDfParams& prm, int off, long long sys, bool valid, bool ok, int e) {
+//
+// Where v_s lies along strong interference, u_s is up to kappa(Rl) times smaller
+// than the terms of that sum and keeps their errors.  Unrefined basis solutions
+// belong to one slightly other matrix, and so does their combination; but a
+// refinement step rounds every residual by itself, 2^-48 of |Rl| |U_c|, which
+// the smallest eigenvalue, the load, turns into about 2^-47 / lf of U_c: measured
+// 6e-15 / lf of sum max |U_c| (spatial factors of magnitude 1) for D = 12 to 128, loads 1e-3 to 2.3e-5 and
+// one or two steps.  (Rank one along v_s, 60 dB and more: errors of 2.5e-7 at D =
+// 12 to 1.8e-5 at D = 128 for load 1e-3, up to 5e-4 for the weakest loads; a solve
+// of v_s itself is below the complex64 rounding.)  A system with a vector whose
+// ratio is 2^21 lf or more (SolveDfParams::cancel), i.e. half a complex64
+// rounding, is marked, and its vectors are solved by themselves.  A clutter
+// ridge does not get there (D = 12 to 128, 40 to 60 dB, load 1e-3: median 3 to 30,
+// largest 300).  (The refinement option keeps the combination.)
+// Most vectors need no look at the sums: |U_c| <= |g| / delta and Re v^H u <= max
+// |u| sum |v|, so that a q of cancel_q / delta or more rules the ratio out (or, once
+// the sum over the basis is there, of steer_sum times that).
+template <int LR, int RPL, int TEAM, bool F32F>
+__device__ __noinline__ void combine(const SolveDfParams& prm, int off, long long sys, bool valid, bool ok, int e,
+                                     float delta) {
   constexpr int NG = TEAM / LR;
   extern __shared__ float4 smdf[];
   const float4* U = smdf + off / 16;
@@ -885,6 +914,10 @@ __device__ __noinline__ void combine(const SolveDfParams& prm, int off, long lon
   const long long nsys = prm.nsys;
   float2* __restrict__ wts = prm.wts;
   const int tt = team_thread<TEAM>(), li = tt % LR, g = tt / LR;
+  const Shared<TEAM, F32F, square<LR, RPL>()> sh(D, C);
+  char* base = reinterpret_cast<char*>(smdf) + off;
+  int* cancels = reinterpret_cast<int*>(base + sh.ok) + 1;
+  float least_q = __fdividef(prm.cancel_q, delta), least = -1.f;
   // u_s = sum_c a_s[c] U_c: a group takes a steering vector s1 -- with
   // conjugate-symmetric factors (a_{S-1-s} = conj(a_s)) the pair s1,
   // S-1-s1 from the four real sums P = sum ar Ur, Q = sum ai Ui,
@@ -942,6 +975,29 @@ __device__ __noinline__ void combine(const SolveDfParams& prm, int off, long lon
       }
     }
     const ff::F2 d1 = lanes_sum2<LR>(q1s, q1e), d2 = lanes_sum2<LR>(q2s, q2e);
+    if (!F32F && __any_sync(0xffffffffu, !(d1.hi >= least_q) || (sym && !(d2.hi >= least_q)))) {
+      float m1 = 0.f, m2 = 0.f;                    // max |u_s1|, max |u_s2|
+#pragma unroll
+      for (int q = 0; q < RPL; ++q)
+        if (li + LR * q < D) {
+          m1 = fmaxf(m1, fmaxf(fabsf(w1r[q].hi), fabsf(w1i[q].hi)));
+          m2 = fmaxf(m2, fmaxf(fabsf(w2r[q].hi), fabsf(w2i[q].hi)));
+        }
+      m1 = lanes_max<LR>(m1);
+      m2 = lanes_max<LR>(m2);
+      if (least < 0.f) {                           // the system's sum of max |U_c|, once
+        least = 0.f;
+        for (int c = 0; c < C; ++c) {
+          float m = 0.f;
+          for (int i = li; i < D; i += LR)
+            m = fmaxf(m, fmaxf(fabsf(U[(size_t)c * D + i].x), fabsf(U[(size_t)c * D + i].y)));
+          least += lanes_max<LR>(m);
+        }
+        least *= prm.cancel;
+        least_q = fminf(least_q, least * prm.steer_sum);
+      }
+      if (ok && li == 0 && p0 + g < n1 && (!(m1 >= least) || (sym && !(m2 >= least)))) *cancels = 1;
+    }
     const bool good1 = ok && usable(d1), good2 = ok && usable(d2);
     const Gain f1 = gain(d1, -e / 2), f2 = gain(d2, -e / 2);
 #pragma unroll
@@ -993,13 +1049,31 @@ __device__ __forceinline__ void solve_df_body(const SolveDfParams& prm, long lon
     y.sbase = 896 + e;
     factor<TEAM, F32F, square<LR, RPL>()>(y, D);
     const bool ok = *okf != 0;
-    const int nrhs = sep ? prm.C : prm.S;
-    for (int r0 = 0; r0 < nrhs; r0 += PASS) {
-      solve_rhs<LR, RPL, TEAM, F32F>(prm, y, r0);
-      if (!sep) emit<LR, RPL, TEAM>(prm, y.off, sys, valid, ok, e, r0);
-      team_sync<TEAM>();   // the next pass reuses U's rows, the combination reads them all
+    // the basis and its combinations, and all the vectors where one cancelled;
+    // or all the vectors
+    bool direct = !sep;
+    for (;;) {
+      const int nrhs = direct ? prm.S : prm.C;
+      const int step = direct && sep ? min(PASS, prm.C) : PASS;   // the rows of U
+      for (int r0 = 0; r0 < nrhs; r0 += step) {
+        const int g = tt / LR, w0 = (tt >> 5) * (32 / LR);        // group in team, its warp's first
+        Rhs z;
+        z.direct = direct;
+        z.live = g < step && r0 + g < nrhs;
+        z.work = TEAM <= 32 || (w0 < step && r0 + w0 < nrhs);
+        z.rhs = z.live ? r0 + g : nrhs - 1;
+        z.row = direct ? min(g, step - 1) : z.rhs;
+        solve_rhs<LR, RPL, TEAM, F32F>(prm, y, z);
+        if (direct)
+          emit<LR, RPL, TEAM>(prm, y.off, sys, valid && z.live && (!sep || okf[1] != 0), ok, e, z.rhs, z.row);
+        team_sync<TEAM>();   // the next pass reuses U's rows, the combination reads them all
+      }
+      if (direct) break;
+      combine<LR, RPL, TEAM, F32F>(prm, y.off, sys, valid, ok, e, split(y.delta, y.sbase).hi);
+      team_sync<TEAM>();
+      if (F32F || (TEAM > 32 ? okf[1] == 0 : !__any_sync(0xffffffffu, okf[1] != 0))) break;   // alike in a warp
+      direct = true;
     }
-    if (sep) combine<LR, RPL, TEAM>(prm, y.off, sys, valid, ok, e);
     if (valid && !ok && tt == 0) atomicAdd(&prm.status->n_failed, 1ULL);
     team_sync<TEAM>();     // the next system reuses the team's shared memory
   }
@@ -1007,17 +1081,19 @@ __device__ __forceinline__ void solve_df_body(const SolveDfParams& prm, long lon
 
 constexpr int cta_threads(int team) { return team > 32 ? team : 128; }
 // CTAs per SM that the registers must allow (shared memory allows about as many)
-constexpr int min_ctas(int team) { return team == 512 ? 1 : (team == 256 ? 3 : (team == 128 ? 6 : (team == 64 ? 12 : 6))); }
+constexpr int min_ctas(int team, bool f32f) {
+  return team == 512 ? 1 : (team == 256 ? 3 : (team == 128 ? 6 : (team == 64 ? 12 : (f32f ? 6 : 5))));
+}
 
 template <int LR, int RPL, int TEAM, bool F32F>
-__global__ void __launch_bounds__(cta_threads(TEAM), min_ctas(TEAM))
+__global__ void __launch_bounds__(cta_threads(TEAM), min_ctas(TEAM, F32F))
 solve_df_kernel(SolveDfParams p) {
   solve_df_body<LR, RPL, TEAM, F32F>(p, blockIdx.x, gridDim.x);
 }
 
 // the same solves as a persistent launch over the CPIs of a batch
 template <int LR, int RPL, int TEAM, bool F32F>
-__global__ void __launch_bounds__(cta_threads(TEAM), min_ctas(TEAM))
+__global__ void __launch_bounds__(cta_threads(TEAM), min_ctas(TEAM, F32F))
 solve_df_batched(BatchCtl ctl) {
   batched_loop<SolveDfParams>(ctl, [&](const SolveDfParams& p, int bx, int, int gx) {
     solve_df_body<LR, RPL, TEAM, F32F>(p, bx, gx);

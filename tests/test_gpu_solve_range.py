@@ -63,3 +63,63 @@ def test_loads_of_any_strength(C, T, lf):
         w, status = _solve(R, C, T, S, steer, load_factor=lf)
         assert status == (stap.STAP_OK, 0)
         _check(w, _reference(R, v, lf))
+
+
+def _weakest(D):
+    """The smallest load that the double-float kernels accept: D / lf + 1 = 2^19."""
+    return D / (2.0 ** 19 - 1.0) * (1 + 1e-9)
+
+
+@pytest.mark.parametrize("refine", [0, 1])
+@pytest.mark.parametrize("C,T", BIG_AND_SMALL)
+def test_the_weakest_load_on_either_side_of_the_rule(C, T, refine):
+    """kappa(Rl) reaches the bound within a factor of 3 (three strong sources)."""
+    D, S = C * T, C + 3
+    R = _covariances(8, D, seed=D)
+    for lf in (_weakest(D), _weakest(D) * 0.99):
+        for steer in (None, _default_steering(C, T, S) * np.exp(1j * np.arange(D))):
+            v = _default_steering(C, T, S) if steer is None else steer
+            w, status = _solve(R, C, T, S, steer, refine_steps=refine, load_factor=lf)
+            assert status == (stap.STAP_OK, 0)
+            _check(w, _reference(R, v, lf))
+
+
+def _along(v, jnr, seed):
+    """Noise and one source along each of v's vectors in turn, jnr per entry."""
+    n, D = v.shape
+    rng = np.random.default_rng(seed)
+    N = rng.standard_normal((n, D, 2 * D)) + 1j * rng.standard_normal((n, D, 2 * D))
+    a = v * np.sqrt(D) / np.linalg.norm(v, axis=1, keepdims=True)
+    R = jnr * a[:, :, None] * a[:, None, :].conj() + N @ N.conj().swapaxes(1, 2) / (4 * D)
+    i = np.arange(D)
+    R[:, i, i] = R[:, i, i].real
+    return R
+
+
+@pytest.mark.parametrize("refine,load", [(1, "default"), (0, "default"), (2, "default"), (1, "weakest"), (0, "weakest")])
+@pytest.mark.parametrize("db", [40, 60, 80])
+@pytest.mark.parametrize("C,T,S", [(4, 3, 16), (4, 2, 100), (5, 3, 11), (8, 3, 16), (16, 4, 32), (32, 3, 40),
+                                   (32, 4, 64)])
+def test_beams_along_the_interference(C, T, S, db, refine, load):
+    """The solution of such a beam is up to kappa(Rl) times smaller than the
+    separable terms that it is combined from."""
+    D = C * T
+    lf = 1e-3 if load == "default" else _weakest(D)
+    for steer in (None, _default_steering(C, T, S) * np.exp(1j * np.arange(D))):
+        v = _default_steering(C, T, S) if steer is None else steer
+        R = _along(v[np.linspace(0, S - 1, 16).astype(int)], 10.0 ** (db / 10), seed=S)
+        w, status = _solve(R, C, T, S, steer, refine_steps=refine, load_factor=lf)
+        assert status == (stap.STAP_OK, 0)
+        _check(w, _reference(R, v, lf))
+
+
+def test_beams_along_the_interference_in_many_small_systems():
+    """Two systems share a warp: one with such a beam, one without."""
+    C, T, S = 4, 3, 16
+    v = _default_steering(C, T, S)
+    n = 8 * 257
+    R = _covariances(n, C * T, seed=2)
+    R[::3] = np.resize(_along(v, 1e6, seed=4), (n, C * T, C * T))[:len(R[::3])]
+    w, status = _solve(R, C, T, S)
+    assert status == (stap.STAP_OK, 0)
+    _check(w, _reference(R, v, 1e-3))
