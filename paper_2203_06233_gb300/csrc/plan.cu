@@ -391,9 +391,9 @@ stap_status do_solve(stap_plan p, const Cpi& c, const void* cov, void* wts, cuda
       p->at<const double2>(c.steer_off), c.separable ? p->at<const double2>(c.g_off) : nullptr,
       c.separable ? p->at<const double2>(c.a_off) : nullptr, p->at<const float4>(c.steer_ff_off),
       c.separable ? p->at<const float4>(c.a_ff_off) : nullptr,
-      c.separable ? p->at<const float4>(c.g_ff_off) : nullptr, (long long)d.n_dop * nb, c.D,
-      d.n_steering, d.n_chan, p->opt.load_factor, p->opt.refine_steps, p->opt.solver, p->status(),
-      st, c.tune, c.separable && c.sep_sym, c.g_norm, c.steer_sum));
+      c.separable ? p->at<const float4>(c.g_ff_off) : nullptr, (long long)d.n_dop * nb,
+      (long long)d.n_dop * c.NB, c.D, d.n_steering, d.n_chan, p->opt.load_factor, p->opt.refine_steps,
+      p->opt.solver, p->status(), st, c.tune, c.separable && c.sep_sym, c.g_norm, c.steer_sum));
 }
 
 stap_status do_apply(stap_plan p, const Cpi& c, const void* dop, const void* wts, float* out,

@@ -1186,8 +1186,8 @@ int pow2ceil(int x) {
 
 cudaError_t launch_solve(const double2* cov, float2* wts, const double2* steer,
                          const double2* sep_g, const double2* sep_a, const float4* steer_ff,
-                         const float4* sep_a_ff, const float4* g_ff, long long nsys, int D, int S,
-                         int C, double load_factor, int refine_steps, int solver,
+                         const float4* sep_a_ff, const float4* g_ff, long long nsys, long long cpi_sys,
+                         int D, int S, int C, double load_factor, int refine_steps, int solver,
                          DeviceStatus* status, cudaStream_t s, const Tune& tn, bool sep_sym, double g_norm,
                          double steer_sum) {
   if (nsys <= 0) return cudaSuccess;
@@ -1207,6 +1207,7 @@ cudaError_t launch_solve(const double2* cov, float2* wts, const double2* steer,
     p.g_ff = g_ff;
     p.sep_a_ff = sep_a_ff;
     p.nsys = nsys;
+    p.cpi_sys = cpi_sys;
     p.D = D;
     p.S = S;
     p.C = C;

@@ -35,6 +35,8 @@ struct SolveDfParams {
   float cancel, cancel_q;
   float steer_sum;         // the largest sum of |re| + |im| over a steering vector
   long long nsys;
+  long long cpi_sys;       // of the whole CPI: a launch may cover a range slab of it.  Where
+                           // kernels round differently this one chooses, so that slabs agree
   int D, S, C;
   int sep;                 // solve the C basis right-hand sides g (x) e_c
   int sym;                 // separable factors with a_{S-1-s} = conj(a_s)

@@ -10,7 +10,7 @@ cudaError_t launch_solve_df_small(const SolveDfParams& p, cudaStream_t s) {
   // whole: 256 systems 34.4 / 26.3 us, 1024 36.5 / 30.3, 4096 58.0 / 65.9).  D = 16:
   // a warp (1024: half 55.5, whole 36.4; 16384: 299, 277).  D = 32: 128 threads
   // (256: 64 threads 82.1, 128 58.0; 16384: 1875, 1817)
-  if (D <= 8 || (D <= 12 && p.nsys >= 2048))
+  if (D <= 8 || (D <= 12 && p.cpi_sys >= 2048))
     return D <= 8 ? launch_df<4, 2, 16, false>(p, s) : launch_df<4, 3, 16, false>(p, s);
   if (D <= 16) return launch_df<8, 2, 32, false>(p, s);
   if (D <= 24) return launch_df<8, 3, 64, false>(p, s);

@@ -123,3 +123,20 @@ def test_beams_along_the_interference_in_many_small_systems():
     w, status = _solve(R, C, T, S)
     assert status == (stap.STAP_OK, 0)
     _check(w, _reference(R, v, 1e-3))
+
+
+def test_range_slabs_take_the_whole_cpis_kernel():
+    """D = 12, 8192 systems: half a warp per system, also in slabs of 1024,
+    which by themselves would take a warp each and round otherwise."""
+    g = torch.Generator().manual_seed(1)
+    cube = torch.randn((4, 128, 1024), dtype=torch.complex64, generator=g).cuda()
+    out = []
+    for slabs in (1, 3, 8):
+        plan = stap.Plan((4, 128, 128, 1024, 3, 16, 8))
+        choices = stap.stap_plan_get_tuning(plan.handle, 0)
+        choices[6] = slabs
+        stap.stap_plan_set_tuning(plan.handle, 0, choices)
+        out.append(plan.run_cpi(cube).clone())
+        assert plan.status() == (stap.STAP_OK, 0)
+        plan.close()
+    assert torch.equal(out[1], out[0]) and torch.equal(out[2], out[0])
