@@ -382,7 +382,7 @@ stap_status do_covariance(stap_plan p, const Cpi& c, const void* dop, void* cov,
 }
 
 stap_status do_solve(stap_plan p, const Cpi& c, const void* cov, void* wts, cudaStream_t st,
-                     int nr = -1) {
+                     int nr = -1, bool any_matrix = false) {
   NvtxRange range("stap_solve_weights");
   const stap_dims& d = c.d;
   const long long nb = nr < 0 ? c.NB : nr / d.training_block;
@@ -393,7 +393,8 @@ stap_status do_solve(stap_plan p, const Cpi& c, const void* cov, void* wts, cuda
       c.separable ? p->at<const float4>(c.a_ff_off) : nullptr,
       c.separable ? p->at<const float4>(c.g_ff_off) : nullptr, (long long)d.n_dop * nb,
       (long long)d.n_dop * c.NB, c.D, d.n_steering, d.n_chan, p->opt.load_factor, p->opt.refine_steps,
-      p->opt.solver, p->status(), st, c.tune, c.separable && c.sep_sym, c.g_norm, c.steer_sum));
+      p->opt.solver, p->status(), st, c.tune, c.separable && c.sep_sym, c.g_norm, c.steer_sum,
+      any_matrix));
 }
 
 stap_status do_apply(stap_plan p, const Cpi& c, const void* dop, const void* wts, float* out,
@@ -884,6 +885,7 @@ stap_status stap_check_report(int64_t* count, int32_t* site, int64_t* index, int
   cudaError_t (*readers[])(stap::CheckRecord*) = {
       stap::check_record_doppler, stap::check_record_covariance, stap::check_record_solve,
       stap::check_record_solve_df_small, stap::check_record_solve_df_big,
+      stap::check_record_solve_df_small_any, stap::check_record_solve_df_big_any,
       stap::check_record_solve_df_small_ir, stap::check_record_solve_df_big_ir,
       stap::check_record_apply,   stap::check_record_mixed,      stap::check_record_train};
   bool first = true;
@@ -1159,7 +1161,7 @@ stap_status stap_solve_weights(stap_plan p, const void* cov, void* wts) {
   if (!cov || !wts) return STAP_ERR_INVALID_ARG;
   if (!aligned16(cov) || !aligned16(wts)) return STAP_ERR_MISALIGNED;
   if ((st = ready(p, p->step_bytes)) != STAP_OK) return st;
-  return do_solve(p, p->cpis[0], cov, wts, p->stream);
+  return do_solve(p, p->cpis[0], cov, wts, p->stream, -1, true);
 }
 
 stap_status stap_apply(stap_plan p, const void* dop, const void* wts, float* out) {

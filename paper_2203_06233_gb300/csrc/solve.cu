@@ -1135,6 +1135,41 @@ cudaError_t launch_big(const double2* cov, float2* wts, const double2* steer, co
                        dim3((unsigned)blocks), NT, smem, s, p, nsys);
 }
 
+// The systems that the double-float kernels marked (kUnsolved), again in FP64.
+// A thread looks at one system's mark, so that a launch with nothing to do costs
+// one read of each.
+template <int LR, int NT, int RPL>
+__global__ void __launch_bounds__(NT, NT >= 256 ? 1 : 3)
+solve_marked_kernel(SolveParams p) {
+  auto marked = [&](long long sys) {
+    return sys < p.nsys &&
+           __ldcg(reinterpret_cast<const unsigned*>(p.wts + (size_t)sys * p.S * p.D)) == kUnsolved;
+  };
+  const long long gx = gridDim.x;
+  for (long long s0 = blockIdx.x; s0 < p.nsys; s0 += gx * NT) {
+    if (!__syncthreads_or(marked(s0 + gx * threadIdx.x))) continue;
+    // (no other CTA writes these weights, and this one not before barriers that
+    // every thread reaches after its look)
+    for (int t = 0; t < NT && s0 + gx * t < p.nsys; ++t)
+      if (marked(s0 + gx * t)) solve_big_kernel_body<false, LR, NT, RPL>(p, s0 + gx * t, p.nsys);
+  }
+}
+
+template <int LR, int NT, int RPL>
+cudaError_t launch_marked(const double2* cov, float2* wts, const double2* steer, long long nsys, int D, int S, int C,
+                          double lf, int refine, DeviceStatus* status, cudaStream_t s) {
+  const size_t smem = ((size_t)D * (D + 1) / 2 + 2 * D) * sizeof(double2) + D * sizeof(double) + 16;
+  static int set_bytes[64] = {0};
+  const cudaError_t e = ensure_smem(solve_marked_kernel<LR, NT, RPL>, smem, set_bytes);
+  if (e != cudaSuccess) return e;
+  const int per_sm = (int)(228 * 1024 / (smem + 1024));
+  const long long blocks = std::min(nsys, 152LL * std::max(1, std::min(per_sm, 4)));
+  const SolveParams p{cov, wts, steer, nullptr, nullptr, nullptr, nullptr, nsys, D, S, C, 0, lf, refine, status,
+                      (int)nsys, 0};
+  solve_marked_kernel<LR, NT, RPL><<<(unsigned)blocks, NT, smem, s>>>(p);
+  return cudaGetLastError();
+}
+
 template <int D, bool SEP>
 cudaError_t launch_reg(const double2* cov, float2* wts, const double2* steer, const double2* sep_g,
                        const float4* steer_ff, const float4* sep_a_ff, long long nsys, int S, int C,
@@ -1189,7 +1224,7 @@ cudaError_t launch_solve(const double2* cov, float2* wts, const double2* steer,
                          const float4* sep_a_ff, const float4* g_ff, long long nsys, long long cpi_sys,
                          int D, int S, int C, double load_factor, int refine_steps, int solver,
                          DeviceStatus* status, cudaStream_t s, const Tune& tn, bool sep_sym, double g_norm,
-                         double steer_sum) {
+                         double steer_sum, bool any_matrix) {
   if (nsys <= 0) return cudaSuccess;
   if (D < 1 || D > kMaxD || S < 1) return cudaErrorInvalidValue;
   const bool sep = sep_g != nullptr && sep_a != nullptr && steer_ff != nullptr && sep_a_ff != nullptr &&
@@ -1220,7 +1255,12 @@ cudaError_t launch_solve(const double2* cov, float2* wts, const double2* steer,
     p.refine_steps = refine_steps;
     p.status = status;
     if (solver == 1) return D <= kSmallMaxD ? launch_solve_df_small_ir(p, s) : launch_solve_df_big_ir(p, s);
-    return D <= kSmallMaxD ? launch_solve_df_small(p, s) : launch_solve_df_big(p, s);
+    if (!any_matrix) return D <= kSmallMaxD ? launch_solve_df_small(p, s) : launch_solve_df_big(p, s);
+    p.max_correction = (float)(std::max(D / load_factor + 1.0, 1024.0) / 8796093022208.0);   // 2^-43 kappa
+    const cudaError_t e = D <= kSmallMaxD ? launch_solve_df_small_any(p, s) : launch_solve_df_big_any(p, s);
+    if (e != cudaSuccess) return e;
+    return D <= 64 ? launch_marked<16, 128, 4>(cov, wts, steer, nsys, D, S, C, load_factor, refine_steps, status, s)
+                   : launch_marked<16, 256, 8>(cov, wts, steer, nsys, D, S, C, load_factor, refine_steps, status, s);
   }
   if (solver == 1) return cudaErrorNotSupported;
   // one system per CTA, lanes over rows: above D = 32, and below where the

@@ -8,8 +8,19 @@
 namespace stap {
 
 // Largest bound D / load_factor + 1 on the loaded matrix's condition number
-// at which the double-float kernels stand in for the FP64 ones.
+// at which the double-float kernels stand in for the FP64 ones.  What it
+// guarantees: for R positive semidefinite, as a sample covariance is, kappa(Rl)
+// is at most this and each weight vector is off by less than its complex64
+// rounding, whether it was solved by itself or combined from the basis
+// solutions (those whose combination cancels are solved by themselves).  For
+// any other Hermitian R, as a caller may pass one, nothing bounds kappa:
+// the kernels for any matrix then look at what the first refinement step corrects.
 constexpr double kDfMaxKappa = 524288.0;   // 2^19
+
+// A system that the kernels for any matrix cannot answer for has this in
+// the first word of its weights until the FP64 kernel has solved it: a NaN that
+// no arithmetic gives.
+constexpr unsigned kUnsolved = 0x7FD5A3E1u;
 
 // Whether a plan's solve takes these kernels: the refinement option, and the
 // default solver where the load bounds the condition number.  Without a
@@ -42,20 +53,27 @@ struct SolveDfParams {
   int sym;                 // separable factors with a_{S-1-s} = conj(a_s)
   double load_factor;
   int refine_steps;
+  float max_correction;    // any matrix: systems that fail, or whose first correction is above
+                           // this part of the solution, are marked instead of counted
   DeviceStatus* status;
   int gx;
 };
 
-// D <= 32 and D > 32, double-float throughout; and with the FP32 factor and
-// substitutions of STAP_SOLVE_MIXED_IR (double-float residuals and solutions).
-// One translation unit each.
+// D <= 32 and D > 32: double-float throughout, of covariances and of any
+// Hermitian matrices; and with the FP32 factor and substitutions of
+// STAP_SOLVE_MIXED_IR (double-float residuals and solutions).  One translation
+// unit each.
 cudaError_t launch_solve_df_small(const SolveDfParams& p, cudaStream_t s);
 cudaError_t launch_solve_df_big(const SolveDfParams& p, cudaStream_t s);
+cudaError_t launch_solve_df_small_any(const SolveDfParams& p, cudaStream_t s);
+cudaError_t launch_solve_df_big_any(const SolveDfParams& p, cudaStream_t s);
 cudaError_t launch_solve_df_small_ir(const SolveDfParams& p, cudaStream_t s);
 cudaError_t launch_solve_df_big_ir(const SolveDfParams& p, cudaStream_t s);
 
 cudaError_t check_record_solve_df_small(CheckRecord* out);
 cudaError_t check_record_solve_df_big(CheckRecord* out);
+cudaError_t check_record_solve_df_small_any(CheckRecord* out);
+cudaError_t check_record_solve_df_big_any(CheckRecord* out);
 cudaError_t check_record_solve_df_small_ir(CheckRecord* out);
 cudaError_t check_record_solve_df_big_ir(CheckRecord* out);
 

@@ -70,7 +70,7 @@
 // renormalisations, the shuffles that broadcast a column's entry and the loads
 // take the rest.
 //
-// F32F (STAP_SOLVE_MIXED_IR): the factor and the substitutions in FP32, the
+// kMixedIr (STAP_SOLVE_MIXED_IR): the factor and the substitutions in FP32, the
 // residual and the solution in double-float as above.
 #pragma once
 
@@ -85,10 +85,16 @@ namespace {
 
 constexpr int KC = 8;   // columns of Rl per residual chunk
 
+// Which solve a kernel is: double-float throughout of a covariance; the same of
+// any Hermitian matrix, marking what it cannot answer for (kernels of their own,
+// as the marking costs the others 2 to 3%); the refinement option.
+constexpr int kCovariance = 0, kAnyMatrix = 1, kMixedIr = 2;
+__host__ __device__ constexpr bool f32f(int mode) { return mode == kMixedIr; }   // FP32 factor
+
 // Whether the factorisation and the substitutions' off-diagonal blocks run on
 // grids: from D = 33 on.
-template <int TEAM, bool F32F>
-__host__ __device__ constexpr bool grids() { return !F32F && TEAM >= 256; }
+template <int TEAM, int MODE>
+__host__ __device__ constexpr bool grids() { return !f32f(MODE) && TEAM >= 256; }
 
 // One complex value: running sums (rs, is) and the errors collected beside
 // them (re, ie); in shared memory (re hi, im hi, re lo, im lo).
@@ -367,7 +373,7 @@ __device__ __forceinline__ void ldl_solve(Cdf (&x)[RPL], const float4* L, const 
   for (int q = 0; q < RPL; ++q) norm(x[q]);
 }
 
-// The same in FP32 with the FP32 factor (F32F).
+// The same in FP32 with the FP32 factor (kMixedIr).
 template <int LR, int RPL, bool BACK>
 __device__ __forceinline__ void subst_f32(float2 (&x)[RPL], const float2* L, int D, int li, int gbase) {
 #pragma unroll
@@ -429,10 +435,10 @@ __device__ __forceinline__ void ldl_solve_f32(Cdf (&x)[RPL], const float2* L, co
 template <int LR, int RPL>
 __host__ __device__ constexpr bool square() { return LR * RPL <= 12; }
 
-template <int TEAM, bool F32F, bool SQUARE>
+template <int TEAM, int MODE, bool SQUARE>
 struct Shared {
   static constexpr bool FULL = TEAM <= 32;
-  using LT = typename std::conditional<F32F, float2, float4>::type;   // factor entries
+  using LT = typename std::conditional<f32f(MODE), float2, float4>::type;   // factor entries
   int u, as, col, l, rd, ok, bytes;                // byte offsets, all multiples of 16
   __host__ __device__ Shared(int D, int nu) {
     const int Dp = D * (D + 1) / 2;
@@ -496,10 +502,10 @@ __device__ __forceinline__ ff::F2 pivot(ff::F2 d, int* okf) {
 // the next two columns only and the one after it takes four columns at once,
 // half the passes over the triangle in shared memory (128 rows: 410k cycles
 // without grids, 325k with, 287k by four columns).
-template <int TEAM, bool F32F, bool SQUARE>
+template <int TEAM, int MODE, bool SQUARE>
 __device__ __forceinline__ void factor(const System y, int D) {
   extern __shared__ float4 smdf[];
-  using SH = Shared<TEAM, F32F, SQUARE>;
+  using SH = Shared<TEAM, MODE, SQUARE>;
   const SH sh(D, y.nu);
   using LT = typename SH::LT;
   char* base = reinterpret_cast<char*>(smdf) + y.off;
@@ -510,7 +516,7 @@ __device__ __forceinline__ void factor(const System y, int D) {
   // On grids: h_i = sqrt(Rl_ii); |Rl_il| and every partial sum of the entry's
   // updates are at most h_i h_l where Rl is positive definite (h_i in rd[i]
   // until the pivot's reciprocal comes)
-  constexpr bool GRID = grids<TEAM, F32F>();
+  constexpr bool GRID = grids<TEAM, MODE>();
   if constexpr (GRID) {
     for (int i = tt; i < D; i += TEAM) rd[i].x = 1.0001f * sqrtf(fmaxf(entry(y, D, i, i).x, 0.f));
     team_sync<TEAM>();
@@ -524,7 +530,7 @@ __device__ __forceinline__ void factor(const System y, int D) {
     else cms(x, l, v);
   };
   auto put = [&](int i, int l, float4 v) {
-    if constexpr (F32F) {
+    if constexpr (f32f(MODE)) {
       L[cstart(l, D) + i - l] = make_float2(__fadd_rn(v.x, v.z), __fadd_rn(v.y, v.w));
     } else if constexpr (GRID) {
       Cdf b = unpack(v);
@@ -564,8 +570,8 @@ __device__ __forceinline__ void factor(const System y, int D) {
     LT* colb = reinterpret_cast<LT*>(base + sh.col) + (second ? 2 * D : 0);
     LT* colb2 = colb + D;
     const int cj = cstart(j, D), c1 = pair ? cstart(j1, D) : cj;
-    if constexpr (F32F) {
-      const float rj = pivot<F32F>({L[cj].x, 0.f}, okf).hi;
+    if constexpr (f32f(MODE)) {
+      const float rj = pivot<f32f(MODE)>({L[cj].x, 0.f}, okf).hi;
       float2 a1j = make_float2(0.f, 0.f);
       float r1 = 1.f;
       if (pair) {
@@ -573,7 +579,7 @@ __device__ __forceinline__ void factor(const System y, int D) {
         float d1 = L[c1].x;
         d1 = fmaf(-a1j.x * rj, a1j.x, d1);
         d1 = fmaf(-a1j.y * rj, a1j.y, d1);
-        r1 = pivot<F32F>({d1, 0.f}, okf).hi;
+        r1 = pivot<f32f(MODE)>({d1, 0.f}, okf).hi;
       }
       float2 own = make_float2(0.f, 0.f);
       bool own1 = false;
@@ -605,7 +611,7 @@ __device__ __forceinline__ void factor(const System y, int D) {
       const float hj = GRID ? rd[j].x : 0.f, h1 = GRID && pair ? rd[j1].x : 0.f;
       Cdf dj = unpack(L[cj]);
       take(dj, hj * hj);
-      const ff::F2 rj = pivot<F32F>({dj.rs, dj.re}, okf);
+      const ff::F2 rj = pivot<f32f(MODE)>({dj.rs, dj.re}, okf);
       Cdf a1j{0.f, 0.f, 0.f, 0.f};
       ff::F2 r1{1.f, 0.f};
       if (pair) {
@@ -614,7 +620,7 @@ __device__ __forceinline__ void factor(const System y, int D) {
         Cdf d1 = unpack(L[c1]);
         less(d1, pack(scale(a1j, rj)), conj4(pack(a1j)));
         take(d1, h1 * h1);
-        r1 = pivot<F32F>({d1.rs, d1.re}, okf);
+        r1 = pivot<f32f(MODE)>({d1.rs, d1.re}, okf);
       }
       const float4 a1c = conj4(pack(a1j));
       float4 own = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -682,7 +688,7 @@ __device__ __forceinline__ void factor(const System y, int D) {
       LT* cl = L + cstart(l, D) - l;
       for (int i = l + tt % RW; i < D; i += RW) {
         const LT lij = L[cj + i - j], mij = L[c1 + i - j1];
-        if constexpr (F32F) {
+        if constexpr (f32f(MODE)) {
           float2 acc = cl[i];
           acc.x = fmaf(-lij.x, alj.x, acc.x);
           acc.y = fmaf(-lij.y, alj.x, acc.y);
@@ -716,10 +722,26 @@ struct Rhs {
 };
 
 // Solve and refine a pass of right-hand sides, one per group of LR lanes.
-template <int LR, int RPL, int TEAM, bool F32F>
+//
+// kAnyMatrix: what the first refinement step corrects is the solution's error up
+// to then, kappa(Rl) times the arithmetic's for this right-hand side.  Above
+// max_correction of the solution, 2^-43 of the bound on a covariance's kappa, and
+// above 2^-36 / delta (entries of the right-hand side are about 1: a solution much
+// smaller than 1 / delta, of a vector along strong interference, has an error
+// of up to 2^-40 / delta), the system gets the second bit of the pivot flag.
+// Without refinement steps the correction is formed all the same, but not
+// applied.
+// Refinement steps: a vector whose combination cancels takes one at least, its
+// small solution loses up to kappa(Rl) 2^-46 to the unrefined solve.
+template <int MODE>
+__device__ __forceinline__ int steps(const Rhs& z, const SolveDfParams& prm) {
+  return !f32f(MODE) && z.direct && prm.sep != 0 ? max(prm.refine_steps, 1) : prm.refine_steps;
+}
+
+template <int LR, int RPL, int TEAM, int MODE>
 __device__ __forceinline__ void solve_rhs(const SolveDfParams& prm, const System y, const Rhs z) {
   constexpr int EPT = (KC * LR * RPL + TEAM - 1) / TEAM;   // chunk entries per thread
-  using SH = Shared<TEAM, F32F, square<LR, RPL>()>;
+  using SH = Shared<TEAM, MODE, square<LR, RPL>()>;
   extern __shared__ float4 smdf[];
   const int D = prm.D, C = prm.C;
   const SH sh(D, y.nu);
@@ -728,7 +750,7 @@ __device__ __forceinline__ void solve_rhs(const SolveDfParams& prm, const System
   float4* As = reinterpret_cast<float4*>(base + sh.as);
   const typename SH::LT* L = reinterpret_cast<const typename SH::LT*>(base + sh.l);
   const float2* rd = reinterpret_cast<const float2*>(base + sh.rd);
-  constexpr bool GRID = grids<TEAM, F32F>();
+  constexpr bool GRID = grids<TEAM, MODE>();
   const int tt = team_thread<TEAM>(), li = tt % LR;
   const int gbase = (threadIdx.x & 31) - li;       // first lane of this thread's group
   const bool work = z.work, live = z.live;
@@ -769,20 +791,36 @@ __device__ __forceinline__ void solve_rhs(const SolveDfParams& prm, const System
       __syncthreads();
     }
     if (work) {
-      if constexpr (F32F) ldl_solve_f32<LR, RPL>(x, L, rd, D, li, gbase);
+      if constexpr (f32f(MODE)) ldl_solve_f32<LR, RPL>(x, L, rd, D, li, gbase);
       else ldl_solve<LR, RPL, GRID>(x, L, lmax, rd, D, li, gbase);
+      if (MODE == kAnyMatrix && it == 1) {
+        float c = 0.f, u = 0.f;
 #pragma unroll
-      for (int q = 0; q < RPL; ++q) {
-        const int i = li + LR * q;
-        if (i < D) {
-          if (it > 0) x[q] = add(unpack(Ur[i]), x[q]);   // u += c
-          if (live) Ur[i] = pack(x[q]);
+        for (int q = 0; q < RPL; ++q) {
+          const int i = li + LR * q;
+          if (i < D) {
+            const float4 v = Ur[i];
+            const float a = fabsf(x[q].rs) + fabsf(x[q].is);
+            c = a < INFINITY ? fmaxf(c, a) : INFINITY;   // (a NaN too)
+            u = fmaxf(u, fabsf(v.x) + fabsf(v.y));
+          }
         }
+        c = lanes_max<LR>(c);
+        u = lanes_max<LR>(u);
+        const float some = __fdividef(1.5e-11f, split(y.delta, y.sbase).hi);
+        if (live && li == 0 && !(c <= fmaf(prm.max_correction, u, some))) atomicOr(reinterpret_cast<int*>(base + sh.ok), 2);
       }
+      if (MODE != kAnyMatrix || it <= steps<MODE>(z, prm))
+#pragma unroll
+        for (int q = 0; q < RPL; ++q) {
+          const int i = li + LR * q;
+          if (i < D) {
+            if (it > 0) x[q] = add(unpack(Ur[i]), x[q]);   // u += c
+            if (live) Ur[i] = pack(x[q]);
+          }
+        }
     }
-    // (a vector whose combination cancels takes one refinement step at least: its
-    // small solution loses up to kappa(Rl) 2^-46 to the unrefined solve)
-    if (it == (!F32F && z.direct && prm.sep != 0 ? max(prm.refine_steps, 1) : prm.refine_steps)) break;
+    if (it == (MODE == kAnyMatrix ? max(steps<MODE>(z, prm), 1) : steps<MODE>(z, prm))) break;
     // x = b - Rl u
 #pragma unroll
     for (int q = 0; q < RPL; ++q) x[q] = b_at(li + LR * q);
@@ -903,8 +941,9 @@ __device__ __noinline__ void emit(const SolveDfParams& prm, int off, long long s
 // largest 300).  (The refinement option keeps the combination.)
 // Most vectors need no look at the sums: |U_c| <= |g| / delta and Re v^H u <= max
 // |u| sum |v|, so that a q of cancel_q / delta or more rules the ratio out (or, once
-// the sum over the basis is there, of steer_sum times that).
-template <int LR, int RPL, int TEAM, bool F32F>
+// the sum over the basis is there, of steer_sum times that; a caller's matrix need
+// not keep the first bound).
+template <int LR, int RPL, int TEAM, int MODE>
 __device__ __noinline__ void combine(const SolveDfParams& prm, int off, long long sys, bool valid, bool ok, int e,
                                      float delta) {
   constexpr int NG = TEAM / LR;
@@ -914,10 +953,10 @@ __device__ __noinline__ void combine(const SolveDfParams& prm, int off, long lon
   const long long nsys = prm.nsys;
   float2* __restrict__ wts = prm.wts;
   const int tt = team_thread<TEAM>(), li = tt % LR, g = tt / LR;
-  const Shared<TEAM, F32F, square<LR, RPL>()> sh(D, C);
+  const Shared<TEAM, MODE, square<LR, RPL>()> sh(D, C);
   char* base = reinterpret_cast<char*>(smdf) + off;
   int* cancels = reinterpret_cast<int*>(base + sh.ok) + 1;
-  float least_q = __fdividef(prm.cancel_q, delta), least = -1.f;
+  float least_q = MODE == kAnyMatrix ? INFINITY : __fdividef(prm.cancel_q, delta), least = -1.f;
   // u_s = sum_c a_s[c] U_c: a group takes a steering vector s1 -- with
   // conjugate-symmetric factors (a_{S-1-s} = conj(a_s)) the pair s1,
   // S-1-s1 from the four real sums P = sum ar Ur, Q = sum ai Ui,
@@ -975,7 +1014,7 @@ __device__ __noinline__ void combine(const SolveDfParams& prm, int off, long lon
       }
     }
     const ff::F2 d1 = lanes_sum2<LR>(q1s, q1e), d2 = lanes_sum2<LR>(q2s, q2e);
-    if (!F32F && __any_sync(0xffffffffu, !(d1.hi >= least_q) || (sym && !(d2.hi >= least_q)))) {
+    if (!f32f(MODE) && __any_sync(0xffffffffu, !(d1.hi >= least_q) || (sym && !(d2.hi >= least_q)))) {
       float m1 = 0.f, m2 = 0.f;                    // max |u_s1|, max |u_s2|
 #pragma unroll
       for (int q = 0; q < RPL; ++q)
@@ -1014,7 +1053,7 @@ __device__ __noinline__ void combine(const SolveDfParams& prm, int off, long lon
   }
 }
 
-template <int LR, int RPL, int TEAM, bool F32F>
+template <int LR, int RPL, int TEAM, int MODE>
 __device__ __forceinline__ void solve_df_body(const SolveDfParams& prm, long long bx, long long gx) {
   constexpr int PASS = TEAM / LR;                  // right-hand sides per pass, one per group
   const long long nsys = prm.nsys;
@@ -1026,7 +1065,7 @@ __device__ __forceinline__ void solve_df_body(const SolveDfParams& prm, long lon
   const int tt = team_thread<TEAM>();
   System y;
   y.nu = sep ? prm.C : PASS;
-  const Shared<TEAM, F32F, square<LR, RPL>()> sh(D, y.nu);
+  const Shared<TEAM, MODE, square<LR, RPL>()> sh(D, y.nu);
   y.off = team * sh.bytes;
   y.aext = nsys * (long long)D * D;
   const int* okf = reinterpret_cast<const int*>(reinterpret_cast<char*>(smdf) + y.off + sh.ok);
@@ -1047,7 +1086,7 @@ __device__ __forceinline__ void solve_df_body(const SolveDfParams& prm, long lon
     const int et = (int)(((uint32_t)__double2hiint(fma(prm.load_factor, tr, tr)) >> 20) & 0x7FF);
     const int e = et == 0 || et == 0x7FF ? 0 : (et - 1023) & ~1;
     y.sbase = 896 + e;
-    factor<TEAM, F32F, square<LR, RPL>()>(y, D);
+    factor<TEAM, MODE, square<LR, RPL>()>(y, D);
     const bool ok = *okf != 0;
     // the basis and its combinations, and all the vectors where one cancelled;
     // or all the vectors
@@ -1063,50 +1102,54 @@ __device__ __forceinline__ void solve_df_body(const SolveDfParams& prm, long lon
         z.work = TEAM <= 32 || (w0 < step && r0 + w0 < nrhs);
         z.rhs = z.live ? r0 + g : nrhs - 1;
         z.row = direct ? min(g, step - 1) : z.rhs;
-        solve_rhs<LR, RPL, TEAM, F32F>(prm, y, z);
+        solve_rhs<LR, RPL, TEAM, MODE>(prm, y, z);
         if (direct)
           emit<LR, RPL, TEAM>(prm, y.off, sys, valid && z.live && (!sep || okf[1] != 0), ok, e, z.rhs, z.row);
         team_sync<TEAM>();   // the next pass reuses U's rows, the combination reads them all
       }
       if (direct) break;
-      combine<LR, RPL, TEAM, F32F>(prm, y.off, sys, valid, ok, e, split(y.delta, y.sbase).hi);
+      combine<LR, RPL, TEAM, MODE>(prm, y.off, sys, valid, ok, e, split(y.delta, y.sbase).hi);
       team_sync<TEAM>();
-      if (F32F || (TEAM > 32 ? okf[1] == 0 : !__any_sync(0xffffffffu, okf[1] != 0))) break;   // alike in a warp
+      if (f32f(MODE) || (TEAM > 32 ? okf[1] == 0 : !__any_sync(0xffffffffu, okf[1] != 0))) break;   // alike in a warp
       direct = true;
     }
-    if (valid && !ok && tt == 0) atomicAdd(&prm.status->n_failed, 1ULL);
+    if constexpr (MODE == kAnyMatrix) {            // (the pass and the combination ended with a barrier)
+      if (valid && *okf != 1 && tt == 0) prm.wts[sys * prm.S * D] = make_float2(__uint_as_float(kUnsolved), 0.f);
+    } else {
+      if (valid && !ok && tt == 0) atomicAdd(&prm.status->n_failed, 1ULL);
+    }
     team_sync<TEAM>();     // the next system reuses the team's shared memory
   }
 }
 
 constexpr int cta_threads(int team) { return team > 32 ? team : 128; }
 // CTAs per SM that the registers must allow (shared memory allows about as many)
-constexpr int min_ctas(int team, bool f32f) {
-  return team == 512 ? 1 : (team == 256 ? 3 : (team == 128 ? 6 : (team == 64 ? 12 : (f32f ? 6 : 5))));
+constexpr int min_ctas(int team, int mode) {
+  return team == 512 ? 1 : (team == 256 ? 3 : (team == 128 ? 6 : (team == 64 ? 12 : (f32f(mode) ? 6 : 5))));
 }
 
-template <int LR, int RPL, int TEAM, bool F32F>
-__global__ void __launch_bounds__(cta_threads(TEAM), min_ctas(TEAM, F32F))
+template <int LR, int RPL, int TEAM, int MODE>
+__global__ void __launch_bounds__(cta_threads(TEAM), min_ctas(TEAM, MODE))
 solve_df_kernel(SolveDfParams p) {
-  solve_df_body<LR, RPL, TEAM, F32F>(p, blockIdx.x, gridDim.x);
+  solve_df_body<LR, RPL, TEAM, MODE>(p, blockIdx.x, gridDim.x);
 }
 
 // the same solves as a persistent launch over the CPIs of a batch
-template <int LR, int RPL, int TEAM, bool F32F>
-__global__ void __launch_bounds__(cta_threads(TEAM), min_ctas(TEAM, F32F))
+template <int LR, int RPL, int TEAM, int MODE>
+__global__ void __launch_bounds__(cta_threads(TEAM), min_ctas(TEAM, MODE))
 solve_df_batched(BatchCtl ctl) {
   batched_loop<SolveDfParams>(ctl, [&](const SolveDfParams& p, int bx, int, int gx) {
-    solve_df_body<LR, RPL, TEAM, F32F>(p, bx, gx);
+    solve_df_body<LR, RPL, TEAM, MODE>(p, bx, gx);
   });
 }
 
-template <int LR, int RPL, int TEAM, bool F32F>
+template <int LR, int RPL, int TEAM, int MODE>
 cudaError_t launch_df(SolveDfParams p, cudaStream_t s) {
   constexpr int PASS = TEAM / LR;
   constexpr size_t kMaxSmem = 227 * 1024;
   // the basis form keeps all C solutions in shared memory
-  if (p.sep && Shared<TEAM, F32F, square<LR, RPL>()>(p.D, p.C).bytes > (int)kMaxSmem) p.sep = p.sym = 0;
-  const size_t tb = Shared<TEAM, F32F, square<LR, RPL>()>(p.D, p.sep ? p.C : PASS).bytes;
+  if (p.sep && Shared<TEAM, MODE, square<LR, RPL>()>(p.D, p.C).bytes > (int)kMaxSmem) p.sep = p.sym = 0;
+  const size_t tb = Shared<TEAM, MODE, square<LR, RPL>()>(p.D, p.sep ? p.C : PASS).bytes;
   int threads = TEAM;
   if (TEAM <= 32) {
     // several teams per CTA; with few systems one warp per CTA, so that they
@@ -1118,15 +1161,46 @@ cudaError_t launch_df(SolveDfParams p, cudaStream_t s) {
   const size_t smem = tb * teams;
   if (smem > kMaxSmem) return cudaErrorInvalidValue;
   static int set_bytes[64] = {0}, set_bytes_b[64] = {0};
-  cudaError_t err = ensure_smem(solve_df_kernel<LR, RPL, TEAM, F32F>, smem, set_bytes);
-  if (err == cudaSuccess) err = ensure_smem(solve_df_batched<LR, RPL, TEAM, F32F>, smem, set_bytes_b);
-  if (err != cudaSuccess) return err;
+  cudaError_t err = ensure_smem(solve_df_kernel<LR, RPL, TEAM, MODE>, smem, set_bytes);
   const long long units = (p.nsys + teams - 1) / teams;
   const long long blocks = units < (1LL << 30) ? units : (1LL << 30);
   p.gx = (int)blocks;
-  return launch_params(reinterpret_cast<const void*>(solve_df_kernel<LR, RPL, TEAM, F32F>),
-                       reinterpret_cast<const void*>(solve_df_batched<LR, RPL, TEAM, F32F>),
-                       dim3((unsigned)blocks), threads, smem, s, p, blocks);
+  if constexpr (MODE == kAnyMatrix) {              // one call's launch: no persistent form
+    if (err != cudaSuccess) return err;
+    solve_df_kernel<LR, RPL, TEAM, MODE><<<(unsigned)blocks, threads, smem, s>>>(p);
+    return cudaGetLastError();
+  } else {
+    if (err == cudaSuccess) err = ensure_smem(solve_df_batched<LR, RPL, TEAM, MODE>, smem, set_bytes_b);
+    if (err != cudaSuccess) return err;
+    return launch_params(reinterpret_cast<const void*>(solve_df_kernel<LR, RPL, TEAM, MODE>),
+                         reinterpret_cast<const void*>(solve_df_batched<LR, RPL, TEAM, MODE>),
+                         dim3((unsigned)blocks), threads, smem, s, p, blocks);
+  }
+}
+
+// The splits of the double-float solves: D <= 32, and above.
+template <int MODE>
+cudaError_t launch_small(const SolveDfParams& p, cudaStream_t s) {
+  const int D = p.D;
+  // D <= 12: half a warp per system, or a whole one where the systems are too
+  // few to fill the SMs and the latency of one counts (C 4 S 16, D = 12, half /
+  // whole: 256 systems 34.4 / 26.3 us, 1024 36.5 / 30.3, 4096 58.0 / 65.9).  D = 16:
+  // a warp (1024: half 55.5, whole 36.4; 16384: 299, 277).  D = 32: 128 threads
+  // (256: 64 threads 82.1, 128 58.0; 16384: 1875, 1817)
+  if (D <= 8 || (D <= 12 && p.cpi_sys >= 2048))
+    return D <= 8 ? launch_df<4, 2, 16, MODE>(p, s) : launch_df<4, 3, 16, MODE>(p, s);
+  if (D <= 16) return launch_df<8, 2, 32, MODE>(p, s);
+  if (D <= 24) return launch_df<8, 3, 64, MODE>(p, s);
+  return launch_df<16, 2, 128, MODE>(p, s);
+}
+
+template <int MODE>
+cudaError_t launch_large(const SolveDfParams& p, cudaStream_t s) {
+  const int D = p.D;
+  if (D <= 48) return launch_df<16, 3, 256, MODE>(p, s);
+  if (D <= 64) return launch_df<16, 4, 256, MODE>(p, s);
+  if (D <= 96) return launch_df<16, 6, 512, MODE>(p, s);
+  return launch_df<32, 4, 512, MODE>(p, s);
 }
 
 }  // namespace

@@ -129,13 +129,16 @@ cudaError_t launch_apply_tc(const float2* dop, const float2* wts, float* out, in
 // steer_ff [S][D] and sep_a_ff [S][C] are the same tables as double-floats
 // (re_hi, re_lo, im_hi, im_lo) for the combination on the FP32 pipe, g_norm |sep_g|_2 and
 // steer_sum the largest sum of |re| + |im| over a steering vector.  cpi_sys: the
-// systems of the whole CPI, where nsys are a range slab's.
+// systems of the whole CPI, where nsys are a range slab's.  any_matrix: cov is a
+// caller's and need not be positive semidefinite (a second launch solves what
+// the double-float kernels cannot answer for).
 cudaError_t launch_solve(const double2* cov, float2* wts, const double2* steer,
                          const double2* sep_g, const double2* sep_a, const float4* steer_ff,
                          const float4* sep_a_ff, const float4* g_ff, long long nsys, long long cpi_sys,
                          int D, int S, int C, double load_factor, int refine_steps, int solver,
                          DeviceStatus* status, cudaStream_t s, const Tune& t = Tune(),
-                         bool sep_sym = false, double g_norm = 0.0, double steer_sum = 0.0);
+                         bool sep_sym = false, double g_norm = 0.0, double steer_sum = 0.0,
+                         bool any_matrix = false);
 
 // out[s][k][r] = |w^H x|^2; dop [C][K][R] c64, wts [K][NB][S][D] c64, out [S][K][R] f32.
 cudaError_t launch_apply(const float2* dop, const float2* wts, float* out, int C, int K, int R,

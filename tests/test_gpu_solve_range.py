@@ -140,3 +140,77 @@ def test_range_slabs_take_the_whole_cpis_kernel():
         assert plan.status() == (stap.STAP_OK, 0)
         plan.close()
     assert torch.equal(out[1], out[0]) and torch.equal(out[2], out[0])
+
+
+def _long_reference(R, v, lf):
+    """The weights by an unpivoted LDL^H in long double (64 or more bits)."""
+    n, D = R.shape[0], R.shape[-1]
+    A = R.astype(np.clongdouble)
+    tr = np.einsum("nii->ni", A).real.sum(1)
+    i = np.arange(D)
+    A[:, i, i] = A[:, i, i].real + (np.longdouble(lf) * tr / D)[:, None]
+    u = np.broadcast_to(v.T.astype(np.clongdouble), (n,) + v.T.shape).copy()
+    for j in range(D):                       # [A | u] -> unit upper triangular
+        row = A[:, j, j + 1:] / A[:, j, j, None]
+        ur = u[:, j] / A[:, j, j, None]
+        f = A[:, j + 1:, j, None]
+        A[:, j + 1:, j + 1:] -= f * row[:, None, :]
+        u[:, j + 1:] -= f * ur[:, None, :]
+        A[:, j, j + 1:], u[:, j] = row, ur
+    for j in range(D - 1, 0, -1):
+        u[:, :j] -= A[:, :j, j, None] * u[:, j, None, :]
+    q = np.einsum("sd,nds->ns", v.conj().astype(np.clongdouble), u).real
+    return (np.swapaxes(u, 1, 2) / np.sqrt(q)[:, :, None]).astype(np.complex128)
+
+
+@pytest.mark.parametrize("refine", [0, 1])
+@pytest.mark.parametrize("margin", [0.5, 1e-2, 1e-4, 1e-6])
+@pytest.mark.parametrize("C,T", [(4, 2), (4, 3), (5, 3), (8, 3), (16, 3), (16, 4), (32, 3), (32, 4)])
+def test_matrices_that_are_not_quite_covariances(C, T, margin, refine):
+    """A negative eigenvalue just above minus the load: Rl is positive definite
+    with kappa = 1 / margin times what a covariance's would be.  The weights
+    are as good as 64-bit arithmetic leaves them, sqrt(D) kappa 2^-53 beside the
+    complex64 rounding; covariances among them are not touched."""
+    D, S, n, lf = C * T, 7, 16, 1e-3
+    rng = np.random.default_rng(D)
+    Q, _ = np.linalg.qr(rng.standard_normal((n, D, D)) + 1j * rng.standard_normal((n, D, D)))
+    ev = np.concatenate([[1e4], rng.uniform(0.5, 2.0, D - 2), [0.0]])
+    lo = lf / D * ev.sum() / (1 + lf / D * (1 - margin))      # its share of the trace taken off
+    ev[-1] = -(1 - margin) * lo
+    odd = np.arange(n) % 3 != 1
+    R = (Q * np.where(odd[:, None], ev, np.abs(ev))[:, None, :]) @ Q.conj().swapaxes(1, 2)
+    R = (R + R.conj().swapaxes(1, 2)) / 2
+    kappa = (1e4 + lo) / (margin * lo)
+    tol = TOL + np.sqrt(D) * kappa * 2.0 ** -53
+    v = _default_steering(C, T, S)
+    for steer in (None, v * np.exp(1j * np.arange(D))):
+        w, status = _solve(R, C, T, S, steer, load_factor=lf, refine_steps=refine)
+        assert status == (stap.STAP_OK, 0)
+        ref = _long_reference(R, v if steer is None else steer, lf)
+        err = np.linalg.norm(w - ref, axis=-1) / np.linalg.norm(ref, axis=-1)
+        print(f"indefinite {err[odd].max():.2e} (kappa {kappa:.1e}, bound {tol:.1e}), covariances {err[~odd].max():.2e}")
+        assert err[odd].max() <= tol and err[~odd].max() <= TOL
+
+
+@pytest.mark.parametrize("refine", [0, 1])
+@pytest.mark.parametrize("C,T,S,K,NB", [(3, 2, 5, 8, 3), (4, 3, 16, 8, 3), (4, 3, 16, 64, 33), (5, 3, 40, 8, 5),
+                                        (4, 4, 3, 32, 33), (8, 3, 16, 8, 3), (16, 2, 9, 8, 3), (11, 3, 24, 8, 3),
+                                        (16, 4, 32, 8, 3), (24, 4, 40, 8, 2), (32, 4, 64, 8, 2)])
+def test_runs_and_steps_agree(C, T, S, K, NB, refine):
+    """A run's solve, of its own covariances, and the step's, of any matrix, are
+    kernels of their own: the same bits, also for a beam along interference."""
+    B = 2 * C * T
+    g = torch.Generator().manual_seed(S)
+    cube = torch.randn((C, K, NB * B), dtype=torch.complex64, generator=g)
+    f = 0.5 * np.sin(np.deg2rad(-90.0 + 180.0 * (S // 2 + 0.5) / S))
+    line = np.exp(2j * np.pi * (f * np.arange(C)[:, None] + 3 / K * np.arange(K)[None, :]))
+    cube += 1e3 * torch.from_numpy(line.astype(np.complex64))[:, :, None] * torch.randn(
+        NB * B, dtype=torch.complex64, generator=g)
+    plan = stap.Plan((C, K, K, NB * B, T, B, S), refine_steps=refine)
+    cube = cube.cuda()
+    out = plan.run_cpi(cube).clone()
+    dop = plan.doppler(cube)
+    steps = plan.apply(dop, plan.solve_weights(plan.covariance(dop)))
+    assert plan.status() == (stap.STAP_OK, 0)
+    plan.close()
+    assert torch.equal(out, steps)
