@@ -133,6 +133,7 @@ covariance_ff_kernel(const float2* __restrict__ dop, double2* __restrict__ cov, 
 // Measured, before and after: C16 K256 R4096 T4 B128 (D = 64) 1387 -> 1036 us;
 // C8 K256 R8192 T3 B64 (D = 24) 577 -> 433; C4 K256 R4096 T3 B64 (D = 12) 79.1 ->
 // 69; error against 64 bits at D = 64 5.6e-12 -> 7.6e-13.
+constexpr float kFar = 0x1p40f;         // see the rows' norms
 constexpr int kPairMaxThreads = 1024;   // one thread per entry, up to this
 
 __device__ __forceinline__ float pow2_ceil(float x) {  // smallest power of two >= x, at most 2^126
@@ -214,7 +215,9 @@ __device__ __forceinline__ void covariance_pairs_body(const CovPairsParams& prm,
       if (!(ss > 1e-24f && ss < 1e36f)) {          // warp-uniform: squares may have over- or underflowed
         // again from values scaled by the power of two next to the largest; a
         // row with an infinity or NaN keeps its largest value, its entries are
-        // not finite either
+        // not finite either.  A row whose norm is beyond 2^62 is kept divided by
+        // kFar, with the sign of its norm as the mark, so that the grid and
+        // the sums of any two rows whose own sums FP32 holds stay inside it
         float mx = 0.f;
         for (int cell = lane; cell < cc; cell += 32) mx = fmaxf(mx, fmaxf(fabsf(dst[cell].x), fabsf(dst[cell].y)));
         for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -229,6 +232,14 @@ __device__ __forceinline__ void covariance_pairs_body(const CovPairsParams& prm,
           }
           for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
           n = up * sqrtf(ss);
+          if (n > 0x1p62f) {
+            __syncwarp();
+            for (int cell = lane; cell < cc; cell += 32) {
+              dst[cell].x *= 1.0f / kFar;
+              dst[cell].y *= 1.0f / kFar;
+            }
+            n = -(up * (1.0f / kFar)) * sqrtf(ss);
+          }
         }
       }
       if (lane == 0) m[row] = n;
@@ -258,7 +269,8 @@ __device__ __forceinline__ void covariance_pairs_body(const CovPairsParams& prm,
       const int ra = j1 * C + c1, rb = (j1 + d) * C + c2;
       const float4* xa = reinterpret_cast<const float4*>(X + ra * ld);   // two cells each
       const float4* xb = reinterpret_cast<const float4*>(X + rb * ld);
-      const float s0 = 1.5f * pow2_ceil(2.01f * m[ra] * m[rb]);
+      const float na = m[ra], nb = m[rb];
+      const float s0 = 1.5f * pow2_ceil(fabsf(2.01f * na * nb));
       float sr = s0, si = s0, lr = 0.f, li = 0.f;
 #pragma unroll 4
       for (int p = 0; p < ce / 2; ++p) {
@@ -279,6 +291,11 @@ __device__ __forceinline__ void covariance_pairs_body(const CovPairsParams& prm,
                          ff::f2d_exact(hi * invBf) + ff::f2d_exact(li * invBf));
       } else {
         v = make_double2((ff::f2d_exact(hr) + ff::f2d_exact(lr)) * invB, (ff::f2d_exact(hi) + ff::f2d_exact(li)) * invB);
+      }
+      if (na < 0.f || nb < 0.f) {                  // rows kept divided by kFar
+        const double f = (na < 0.f ? (double)kFar : 1.0) * (nb < 0.f ? (double)kFar : 1.0);
+        v.x *= f;
+        v.y *= f;
       }
       if (c0 > 0) {
         const double2 p = Q[it];

@@ -51,3 +51,18 @@ def test_rows_of_any_magnitude_keep_their_own_precision(spread):
     d = np.sqrt(np.einsum("kbii->kbi", ref).real)
     err = np.abs(cov - ref) / (d[..., :, None] * d[..., None, :])
     assert err[..., ok].max() <= 1e-10
+
+
+@pytest.mark.parametrize("size", [1e18, 1.5e18, 2e18])
+@pytest.mark.parametrize("C,T,B", [(3, 1, 50), (4, 3, 64), (16, 4, 128), (32, 4, 515)])
+def test_rows_at_the_end_of_fp32s_range(C, T, B, size):
+    """Rows whose squares sum to just under FP32's largest number (3.2e38 for the
+    largest), beside rows smaller by 1e28 and by 1e33."""
+    NB, K = 2, 8
+    dop = _dop(C, K, NB * B, B)
+    dop = dop / np.sqrt((np.abs(dop.reshape(C, K, NB, B)) ** 2).sum(3).max()) * size * 9
+    dop[1::3] *= 1e-28
+    dop[2::3] *= 1e-33
+    cov, ref = _run(C, T, B, NB, dop.astype(np.complex64), K)
+    d = np.sqrt(np.einsum("kbii->kbi", ref).real)
+    assert (np.abs(cov - ref) / (d[..., :, None] * d[..., None, :])).max() <= 1e-10
