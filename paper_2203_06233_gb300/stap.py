@@ -447,6 +447,7 @@ class Plan:
         opts = stap_options(float(load_factor), int(refine_steps), int(precision), int(solver),
                             int(training), int(snapshots), int(train_guard), int(train_half))
         self.precision, self.refine_steps, self.solver = int(precision), int(refine_steps), int(solver)
+        self.load_factor = float(load_factor)
         self.training, self.snapshots = int(training), int(snapshots)
         self.train_guard, self.train_half = int(train_guard), int(train_half)
         self.n_elem = 0
@@ -616,6 +617,8 @@ class Plan:
         key = "C%d P%d K%d T%d B%d S%d prec%d ref%d solve%d train%d" % (
             d.n_chan, d.n_pulses, d.n_dop, d.tdof, d.training_block, d.n_steering, self.precision,
             self.refine_steps, self.solver, self.training)
+        # the load decides which solves a plan takes, and so what is tuned
+        key += " load%r" % self.load_factor
         if self.snapshots:
             key += " snap%d" % self.snapshots
         if self.training == STAP_TRAIN_WINDOW:

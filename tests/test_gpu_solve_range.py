@@ -214,3 +214,18 @@ def test_runs_and_steps_agree(C, T, S, K, NB, refine):
     assert plan.status() == (stap.STAP_OK, 0)
     plan.close()
     assert torch.equal(out, steps)
+
+
+def test_the_tuning_cache_tells_loads_apart(tmp_path):
+    """A weak load is solved in FP64, with launch choices of its own; a plan
+    with the default load, tuned into the same cache, does not take them."""
+    dims, cache = (4, 16, 16, 256, 3, 16, 4), str(tmp_path / "tune.json")
+    cube = torch.randn((4, 16, 256), dtype=torch.complex64, device="cuda")
+    keys = []
+    for lf in (1e-6, 1e-3):
+        plan = stap.Plan(dims, load_factor=lf)
+        (key, tuning), = plan.autotune(cube, cache_path=cache).items()
+        keys.append(key)
+        assert (tuning[7] == 0) == (lf == 1e-3), tuning
+        plan.close()
+    assert keys[0] != keys[1]
