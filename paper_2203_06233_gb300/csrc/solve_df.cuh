@@ -26,11 +26,13 @@ constexpr unsigned kUnsolved = 0x7FD5A3E1u;
 // default solver where the load bounds the condition number.  Without a
 // refinement step, on grids (D > 32), the bound is a quarter of that: a vector
 // along strong interference loses up to kappa 2^-42 (measured at D = 128: 3e-7 at
-// kappa 2^19, 8e-8 at 2^17).
+// kappa 2^19, 8e-8 at 2^17).  One or two rows are left to FP64, a lane of which
+// does a whole right-hand side (D = 1, 16384 systems, S = 2: 6.6 us, in
+// double-float 21.6).
 inline bool solve_df_eligible(int solver, double load_factor, int D, int refine_steps) {
   const double most = refine_steps == 0 && D > kSmallMaxD ? kDfMaxKappa / 4 : kDfMaxKappa;
   return solver == STAP_SOLVE_MIXED_IR ||
-         (load_factor > 0.0 && (double)D / load_factor + 1.0 <= most);
+         (load_factor > 0.0 && (double)D / load_factor + 1.0 <= most && D > 2);
 }
 
 // Parameters of one launch (one CPI); gx = the launch's grid size.

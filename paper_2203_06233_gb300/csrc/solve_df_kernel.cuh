@@ -42,8 +42,9 @@
 // trace become zero; an infinity or NaN becomes a NaN, which no pivot test
 // passes.
 //
-// Layout.  A system belongs to a team of TEAM threads: half a warp or a warp
-// (D <= 16) or a CTA of 64, 128 (D <= 32), 256 (D <= 64) or 512 (D <= 128) threads.
+// Layout.  A system belongs to a team of TEAM threads: half a warp, a warp or, of
+// few, 128 threads (D <= 16), a CTA of 64, 128 (D <= 32), 256 (D <= 64) or 512 (D <=
+// 128) threads.
 // LR lanes hold one right-hand side, row li + LR q in register q < RPL.  The
 // factor (column-major packed) and the solutions stay in shared memory, the
 // column's entry is broadcast by shuffles, so a 16-byte read feeds one complex
@@ -1182,14 +1183,23 @@ cudaError_t launch_df(SolveDfParams p, cudaStream_t s) {
 template <int MODE>
 cudaError_t launch_small(const SolveDfParams& p, cudaStream_t s) {
   const int D = p.D;
+  // Few systems with more right-hand sides than a warp's four groups take at
+  // once, or many combinations: 128 threads per system, all of its right-hand
+  // sides in one or two passes (us with a warp / with 128 threads, arbitrary
+  // tables: D = 8 S = 64, 128 systems 100 / 21, 1024 102 / 60; D = 15 S = 16, 128
+  // systems 51 / 22, 512 52 / 38, 1024 68 / 64; D = 16 S = 64, 1024 systems 233 / 185,
+  // 2048 381 / 336; separable: C = 5 S = 16, D = 15, 512 systems 40 / 35, 1024 49 /
+  // 64; C = 4 S = 64, D = 12, 512 systems 38 / 30, 1024 44 / 54)
+  const int nrhs = p.sep ? p.C : p.S;
+  const bool wide = (nrhs > 4 || p.S > 16) && p.cpi_sys <= (nrhs > 16 ? 1024 : 512);
   // D <= 12: half a warp per system, or a whole one where the systems are too
   // few to fill the SMs and the latency of one counts (C 4 S 16, D = 12, half /
   // whole: 256 systems 34.4 / 26.3 us, 1024 36.5 / 30.3, 4096 58.0 / 65.9).  D = 16:
   // a warp (1024: half 55.5, whole 36.4; 16384: 299, 277).  D = 32: 128 threads
   // (256: 64 threads 82.1, 128 58.0; 16384: 1875, 1817)
-  if (D <= 8 || (D <= 12 && p.cpi_sys >= 2048))
-    return D <= 8 ? launch_df<4, 2, 16, MODE>(p, s) : launch_df<4, 3, 16, MODE>(p, s);
-  if (D <= 16) return launch_df<8, 2, 32, MODE>(p, s);
+  if (D <= 8) return wide ? launch_df<4, 2, 128, MODE>(p, s) : launch_df<4, 2, 16, MODE>(p, s);
+  if (D <= 12 && p.cpi_sys >= 2048) return launch_df<4, 3, 16, MODE>(p, s);
+  if (D <= 16) return wide ? launch_df<8, 2, 128, MODE>(p, s) : launch_df<8, 2, 32, MODE>(p, s);
   if (D <= 24) return launch_df<8, 3, 64, MODE>(p, s);
   return launch_df<16, 2, 128, MODE>(p, s);
 }

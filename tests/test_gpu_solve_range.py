@@ -216,6 +216,20 @@ def test_runs_and_steps_agree(C, T, S, K, NB, refine):
     assert torch.equal(out, steps)
 
 
+@pytest.mark.parametrize("solver", [stap.STAP_SOLVE_FP64, stap.STAP_SOLVE_MIXED_IR], ids=["default", "mixed_ir"])
+@pytest.mark.parametrize("n", [8, 512, 520, 1024, 1032, 2040, 2048])
+@pytest.mark.parametrize("C,T,S", [(3, 2, 5), (4, 2, 33), (5, 2, 16), (5, 3, 4), (4, 4, 17), (12, 2, 9)])
+def test_every_split_of_small_systems(C, T, S, n, solver):
+    """Teams of half a warp, a warp and 128 threads, by the systems' count and
+    the right-hand sides' (at most 4, 16, more)."""
+    R = _covariances(n, C * T, seed=S)
+    v = _default_steering(C, T, S)
+    for steer in (None, v * np.exp(1j * np.arange(C * T))):
+        w, status = _solve(R, C, T, S, steer, solver=solver, refine_steps=2)
+        assert status == (stap.STAP_OK, 0)
+        _check(w, _reference(R, v if steer is None else steer, 1e-3))
+
+
 def test_the_tuning_cache_tells_loads_apart(tmp_path):
     """A weak load is solved in FP64, with launch choices of its own; a plan
     with the default load, tuned into the same cache, does not take them."""
