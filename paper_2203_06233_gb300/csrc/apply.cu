@@ -337,6 +337,10 @@ cudaError_t launch_apply(const float2* dop, const float2* wts, float* out, int C
   // least, and where a tile is one or two chunks deep, i.e. nothing hides its
   // loads but other CTAs, the smaller tiles of which more fit an SM
   // (D = 15, K128 R3000 B100 S11: 38.7 us with 64-cell tiles, 41.9 with 128)
+  // Up to 8 steering vectors are one warp per CTA: 32-cell tiles, whose 11 KB let 21
+  // of them share an SM (D = 36, K64 R8192 B256 S4: 57 us, with 128-cell tiles
+  // 74; D = 128 B256 S8: 0.7 of the time)
+  if (S <= 8) return launch_apply_tile<1>(dop, wts, out, C, K, R, ldr, T, B, S, s);
   auto padded = [&](int cells) { return (B + 32 * cells - 1) / (32 * cells) * cells; };
   if (D > 2 * DC && padded(4) <= padded(2) && padded(4) <= padded(1))
     return launch_apply_tile<4>(dop, wts, out, C, K, R, ldr, T, B, S, s);
