@@ -168,6 +168,13 @@ struct CovPairsParams {
 // row pitch in cells: at least cb, and an odd number of 16-byte units
 __host__ __device__ constexpr int pair_ld(int cb) { return (cb + 1) / 4 * 4 + 2; }
 
+// SHORT: blocks of up to kShort cells, where an entry's few cells do not hide its
+// latency and the matrices' stores are most of the work: 32 registers, i.e. 64
+// warps per SM instead of 51, without the unrolling.  (D = 15 K64 R8192 B4: 494
+// -> 385 us; B 32: 3% better, B 50: 2% worse)
+constexpr int kShort = 32;
+
+template <bool SHORT>
 __device__ __forceinline__ void covariance_pairs_body(const CovPairsParams& prm, int bx, int by) {
   const float2* __restrict__ dop = prm.dop;
   double2* __restrict__ cov = prm.cov;
@@ -272,7 +279,7 @@ __device__ __forceinline__ void covariance_pairs_body(const CovPairsParams& prm,
       const float na = m[ra], nb = m[rb];
       const float s0 = 1.5f * pow2_ceil(fabsf(2.01f * na * nb));
       float sr = s0, si = s0, lr = 0.f, li = 0.f;
-#pragma unroll 4
+#pragma unroll (SHORT ? 1 : 4)
       for (int p = 0; p < ce / 2; ++p) {
         const float4 a = xa[p], bb = xb[p];
         grid_add(sr, lr, a.x, bb.x);
@@ -338,17 +345,29 @@ __device__ __forceinline__ void covariance_pairs_body(const CovPairsParams& prm,
   }
 }
 
-__global__ void __launch_bounds__(kPairMaxThreads)
+template <bool SHORT>
+__global__ void __launch_bounds__(kPairMaxThreads, SHORT ? 2 : 0)   // (0: no say)
 covariance_pairs_kernel(CovPairsParams p) {
-  covariance_pairs_body(p, blockIdx.x, blockIdx.y);
+  covariance_pairs_body<SHORT>(p, blockIdx.x, blockIdx.y);
 }
 
 // the same covariances as a persistent launch over the CPIs of a batch
-__global__ void __launch_bounds__(kPairMaxThreads)
+template <bool SHORT>
+__global__ void __launch_bounds__(kPairMaxThreads, SHORT ? 2 : 0)
 covariance_pairs_batched(BatchCtl ctl) {
   batched_loop<CovPairsParams>(ctl, [&](const CovPairsParams& p, int bx, int by, int) {
-    covariance_pairs_body(p, bx, by);
+    covariance_pairs_body<SHORT>(p, bx, by);
   });
+}
+
+template <bool SHORT>
+cudaError_t launch_pairs(const CovPairsParams& p, dim3 grid, int threads, size_t smem, cudaStream_t s) {
+  static int set_bytes[64] = {0}, set_bytes_b[64] = {0};
+  cudaError_t e = ensure_smem(covariance_pairs_kernel<SHORT>, smem, set_bytes);
+  if (e == cudaSuccess) e = ensure_smem(covariance_pairs_batched<SHORT>, smem, set_bytes_b);
+  if (e != cudaSuccess) return e;
+  return launch_params(reinterpret_cast<const void*>(covariance_pairs_kernel<SHORT>),
+                       reinterpret_cast<const void*>(covariance_pairs_batched<SHORT>), grid, threads, smem, s, p);
 }
 
 // Entries of KT bins, and the threads that take them: whole warps, at most
@@ -394,7 +413,7 @@ cudaError_t launch_covariance_fp32(const float2* dop, double2* cov, int C, int K
       const int slots = (items + threads - 1) / threads * threads;   // whole rounds of the CTA
       const double ctas = (double)NB * (K / kt), warps = threads / 32;
       double per = (double)((228 * 1024) / (sm + 1024));             // CTAs per SM: shared memory,
-      per = std::min({per, std::floor(51.0 / warps), std::ceil(ctas / 152.0)});   // 40 registers, the grid
+      per = std::min({per, std::floor((B <= kShort ? 64.0 : 51.0) / warps), std::ceil(ctas / 152.0)});   // registers, the grid
       if (per < 1.0) per = 1.0;
       const double w = per * warps;
       const double t = std::max(ctas / (152.0 * per), 1.0) * per * slots * (w + 12.0) / w;
@@ -409,15 +428,10 @@ cudaError_t launch_covariance_fp32(const float2* dop, double2* cov, int C, int K
     while (CB > 32 && pair_smem(KT, CB) > kPairBudget) CB = (CB + 1) / 2;
     if (pair_smem(KT, CB) <= kPairBudget) {
       const size_t smem = pair_smem(KT, CB);
-      static int set_bytes[64] = {0}, set_bytes_b[64] = {0};
-      cudaError_t e = ensure_smem(covariance_pairs_kernel, smem, set_bytes);
-      if (e == cudaSuccess) e = ensure_smem(covariance_pairs_batched, smem, set_bytes_b);
-      if (e != cudaSuccess) return e;
       dim3 grid(NB, K / KT);
       const CovPairsParams p{dop, cov, C, K, ldr, T, B, NB, KT, CB, lower_only ? 1 : 0, 1.0 / (double)B, (int)grid.x};
-      return launch_params(reinterpret_cast<const void*>(covariance_pairs_kernel),
-                           reinterpret_cast<const void*>(covariance_pairs_batched), grid,
-                           pair_threads(pair_items(C, T, KT)), smem, s, p);
+      const int threads = pair_threads(pair_items(C, T, KT));
+      return B <= kShort ? launch_pairs<true>(p, grid, threads, smem, s) : launch_pairs<false>(p, grid, threads, smem, s);
     }
   }
   // general form: one tile per system, cells in chunks
