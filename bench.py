@@ -11,7 +11,9 @@ timed on the same cube beside it.  The D = 64 CPI, the standard D = 12 CPI and
 the 512-CPI batch are keys of the same line, each with its mixed and plain
 legs; every single-CPI workload also runs the mixed-precision refinement
 solve, and the standard CPI runs the training and snapshot options.  Errors
-against the FP64 oracle on seeded range blocks accompany every leg.
+against the FP64 oracle on seeded range blocks accompany every leg.  The line
+has the headline in full and of every other leg its cells/s; ``--detail FILE``
+writes all the legs' particulars.
 
 Timing: inputs resident in HBM, L2 flushed (256 MiB write) between timed steps,
 each step bracketed by CUDA events on the launching stream; barrier and
@@ -244,6 +246,46 @@ MIR_TEXT = ("mixed-precision refinement solve: FP64 diagonal load, FP32 LDL^H an
 def log(msg):
     """Progress on stderr (the JSON line alone goes to stdout)."""
     print(f"[bench {time.strftime('%H:%M:%S')}] {msg}", file=sys.stderr, flush=True)
+
+
+def rounded(x):
+    """Every float of a nested result to six digits."""
+    if isinstance(x, dict):
+        return {k: rounded(v) for k, v in x.items()}
+    if isinstance(x, list):
+        return [rounded(v) for v in x]
+    return float(f"{x:.6g}") if isinstance(x, float) else x
+
+
+def summary(line):
+    """The result line without its legs' particulars: of each leg its cells/s,
+    of the headline leg also its kernels' times, of the roofline the figures.
+    Short enough (below 4 KB) for a reader that keeps the end of the output only."""
+    out = {k: v for k, v in line.items() if k not in ("mixed", "fp32", "mixed_ir", "workloads")}
+    if "basis" in (out.get("roofline") or {}):
+        out["roofline"] = {k: v for k, v in out["roofline"].items() if k != "basis"}
+    legs = {k: line[k]["value"] for k in ("mixed", "fp32", "mixed_ir") if k in line}
+    if legs:
+        out["legs"] = rounded(legs)
+        out["kernels_ms"] = rounded(line["mixed"]["kernels_ms"])
+    if "workloads" in line:
+        out["workloads"] = rounded({
+            name: {k: v["value"] if isinstance(v, dict) else v
+                   for k, v in dict(w, **w.get("options", {})).items()
+                   if (isinstance(v, dict) and "value" in v and k != "cpu_baseline") or k == "error"}
+            for name, w in line["workloads"].items()})
+    for k in ("errors_vs_oracle", "cpu_baseline", "roofline"):
+        if k in out:
+            out[k] = rounded(out[k])
+    return out
+
+
+def emit(line, args):
+    """One JSON line on stdout; everything that was measured to --detail."""
+    if args.detail:
+        with open(args.detail, "w") as f:
+            json.dump(line, f, indent=1)
+    print(json.dumps(summary(line)), flush=True)
 
 
 def sample_blocks(spec, n):
@@ -606,7 +648,7 @@ def run_gpu(args):
     if world > 1:
         dist.destroy_process_group()
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        emit(line, args)
 
 
 def workload_keys(args, name, rank, dev, stream, flush, pk):
@@ -898,7 +940,7 @@ def run_batch(args):
     if world > 1:
         dist.destroy_process_group()
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        emit(line, args)
 
 
 def run_paper_cube(args):
@@ -1016,7 +1058,7 @@ def run_paper_cube(args):
     if world > 1:
         dist.destroy_process_group()
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        emit(line, args)
 
 
 def plan_chunk(plan):
@@ -1119,6 +1161,8 @@ def main():
     ap.add_argument("--warmup", type=int, default=5)
     ap.add_argument("--impl", choices=["ours", "reference"], default="ours")
     ap.add_argument("--no-cpu-baseline", action="store_true")
+    ap.add_argument("--detail", default=None, metavar="FILE",
+                    help="write every leg's particulars (the other workloads' too) to FILE as JSON")
     ap.add_argument("--only-headline", action="store_true",
                     help="measure the headline workload only (no other workloads as keys)")
     ap.add_argument("--workload", choices=["large", "mixed", "mixed_small", "standard", "batch",
