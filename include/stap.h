@@ -96,7 +96,12 @@ typedef enum {
                              values, compensated sums, about 2^-44) on the FP32
                              pipe: for a covariance (positive semidefinite) the
                              weights are the same up to their complex64
-                             rounding.  Weaker loads are solved in FP64 */
+                             rounding, also for beams along interference.
+                             Weaker loads (refine_steps = 0 and D > 32: from 2^17
+                             on) and D <= 2 are solved in FP64, and so is what
+                             stap_solve_weights is given that is no covariance.
+                             A tuning whose solve kernel is 1 to 3 keeps a plan
+                             on the FP64 kernels (stap_plan_set_tuning) */
   STAP_SOLVE_MIXED_IR = 1 /* mixed-precision iterative refinement (not in the
                              paper; a faster option): Rl's FP32 part factored
                              and solved in FP32, and each of the refine_steps
@@ -105,7 +110,9 @@ typedef enum {
                              correction in FP32 and adds it to the double-float
                              solution.  Each step shrinks the error by about
                              cond(Rl) 2^-24; 2 steps reach FP32 weight accuracy
-                             for cond(Rl) up to about 1e5 */
+                             for cond(Rl) up to about 1e5, but for beams along
+                             strong interference with the default steering,
+                             which lose up to cond(Rl) 2^-39 */
 } stap_solver;
 
 /* Which range cells train the covariance that block b's weights use. */
@@ -218,7 +225,8 @@ stap_status stap_plan_set_wait_limit(stap_plan plan, int32_t max_polls);
 /* Change the stream later calls are issued on. */
 stap_status stap_plan_set_stream(stap_plan plan, void* cuda_stream);
 
-/* Replace the steering table of CPI `cpi` with host_c128[S][D] (copied).
+/* Replace the steering table of CPI `cpi` with host_c128[S][D] (copied; any
+ * finite vectors of any magnitude, the weights do not depend on it).
  * Needs the workspace to be set (the table is uploaded on the plan's stream). */
 stap_status stap_plan_set_steering(stap_plan plan, int32_t cpi, const double* host_c128);
 
@@ -267,7 +275,10 @@ stap_status stap_train_window(stap_plan plan, const void* cov_c128, void* cov_tr
  *   steps u_s += Rl^{-1} (v_s - Rl u_s),  w_s = u_s / sqrt(Re v_s^H u_s).
  * Only the lower triangle and the real part of the diagonal of each cov are
  * read.  A system whose pivot is not positive and finite gets zero weights
- * and is counted (stap_get_status).  cov: c128 [K][NB][D][D];
+ * and is counted (stap_get_status).  cov need not be a covariance: with the
+ * default solver any Hermitian matrix whose Rl is positive definite is solved to
+ * 64-bit accuracy (a second launch solves in FP64 what the double-float kernels
+ * mark; covariances are not marked).  cov: c128 [K][NB][D][D];
  * wts: c64 [K][NB][S][D]. */
 stap_status stap_solve_weights(stap_plan plan, const void* cov_c128, void* wts_c64);
 
@@ -424,18 +435,19 @@ stap_status stap_run_cpi_noalloc(const stap_dims* dims, const stap_options* opt,
  * step in turn it times candidate tile shapes and schedules on the device, on
  * the caller's cubes and output buffers, `reps` runs each (reps < 1 means 3),
  * and keeps the fastest.  Candidates: range cells per Doppler CTA (8/16/32);
- * Doppler bins per covariance CTA (plain precision); lanes per system and
- * warps per CTA of the D <= 32 solve, lanes per right-hand side of the larger
- * solve, and for D = 8, 12 or 16 the register-resident or the shared-memory
- * solve kernel; register-resident or general FP32 apply; for a one-CPI plan, 1, 2, 3,
- * 4, 6 or 8 pipelined range slabs of the whole run; for the mixed precisions
+ * Doppler bins per covariance CTA (plain precision); of solves in FP64 (loads
+ * too weak for the double-float kernels, which have no choices; see
+ * stap_solver) lanes per system and warps per CTA for D <= 32, lanes per
+ * right-hand side above, and for D = 8, 12 or 16 the register-resident or the
+ * shared-memory kernel; register-resident or tiled FP32 apply; for a one-CPI
+ * plan, 1, 2, 4 or 8 pipelined range slabs of the whole run; for the mixed precisions
  * (STAP_PREC_BF16X3, STAP_PREC_TF32X3, STAP_PREC_FP16_SCALED), the tensor-core
  * or the FP32 covariance and apply (the FP32 kernels are the more accurate,
  * and at small D the faster); for a batch, the persistent or the stream
  * schedule (stap_plan_set_batch_schedule).  Every candidate computes
- * the same result except that the apply kernels sum in different orders and
- * that a mixed-precision plan's FP32 choices are more accurate than its
- * tensor-core ones.  Needs the run workspace; synchronises the plan's stream; overwrites
+ * the same result up to the rounding of FP64 solves, except that a
+ * mixed-precision plan's FP32 choices are more accurate than its tensor-core
+ * ones.  Needs the run workspace; synchronises the plan's stream; overwrites
  * outs; clears the device status; drops a captured batch graph. */
 stap_status stap_plan_autotune(stap_plan plan, const void* const* cubes, float* const* outs,
                                int32_t reps);
@@ -443,10 +455,11 @@ stap_status stap_plan_autotune(stap_plan plan, const void* const* cubes, float* 
 /* The launch choices of CPI `cpi` as STAP_TUNING_LEN integers (0 = built-in
  * heuristic): Doppler cells per CTA, covariance bins per CTA, solve lanes per
  * system, solve warps per CTA, large-solve lanes per right-hand side, apply
- * kernel (1 register-resident, 2 general), range slabs of a one-CPI
- * stap_run_cpi (at most 8 and NB are used), solve kernel for D <= 32
+ * kernel (1 register-resident, 2 tiled), range slabs of a one-CPI
+ * stap_run_cpi (at most 8 and NB are used), FP64 solve kernel for D <= 32
  * (1 register-resident for D = 8, 12, 16, 2 shared-memory teams, 3 one
- * system per CTA), covariance of a mixed-precision
+ * system per CTA; above, any of them is one system per CTA; 0: double-float or
+ * FP64 by the load, see stap_solver), covariance of a mixed-precision
  * plan (1 FP32, 2 tensor cores; apply choice 3 = tensor cores).  set_tuning installs saved choices
  * (values 0..64; a choice that does not fit a launch falls back to the
  * heuristic). */

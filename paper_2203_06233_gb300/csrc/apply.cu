@@ -208,7 +208,7 @@ cudaError_t launch_apply_tile(const float2* dop, const float2* wts, float* out, 
 // memory as [block][s][d].  For each steering vector the thread reads its
 // weights as D/2 broadcast 16-byte loads and does 8 D FMAs: FMA-bound.
 // 128-thread CTAs: in a one-CPI run the apply of one range slab shares the
-// SMs with the FP64 solves of others, and a smaller CTA takes fewer of a
+// SMs with the solves of others, and a smaller CTA takes fewer of a
 // solve's warp slots (registers, shared memory) wherever it lands.
 constexpr int kRegThreads = 128;
 constexpr int kRegCells = 2 * kRegThreads;  // range cells per CTA

@@ -6,16 +6,16 @@
 // Precision: the solve downstream sees covariances whose condition number is
 // bounded only by the diagonal load (about 1e3 * D), so rounding R to FP32
 // would dominate the weight error.  Each entry is therefore accumulated
-// error-free in FP32 pairs: every product a*b is split exactly into p + e by
-// one FMA (TwoProduct), p is added to the running sum with Knuth's TwoSum, and
-// all rounding errors are collected in a second FP32 accumulator.  The result
-// sum + errors is accurate to about n^2 u^2 times the sum of |terms|
-// (Ogita, Rump & Oishi, "Accurate sum and dot product", SISC 2005, Dot2),
-// far below FP32 rounding, and is written as FP64.  All of this runs on the
-// FP32 pipe (about 10 FP32 ops per real product); only the final conversion
-// touches FP64.
+// error-free in FP32 pairs on the FP32 pipe and written as FP64; only the final
+// conversion touches FP64.  The bin-pair form below, which serves nearly every
+// shape, sums on a fixed grid (four FP32 instructions per real product, see
+// there).  The general form splits every product a*b exactly into p + e by one
+// FMA (TwoProduct), adds p to the running sum with Knuth's TwoSum and collects
+// all rounding errors in a second FP32 accumulator (about 10 instructions): the
+// result is accurate to about n^2 u^2 times the sum of |terms| (Ogita, Rump &
+// Oishi, "Accurate sum and dot product", SISC 2005, Dot2).
 //
-// Mapping: a CTA owns NS consecutive blocks of one Doppler bin, stages their
+// Mapping of the general form: a CTA owns NS consecutive blocks of one Doppler bin, stages their
 // D x B snapshot tiles in shared memory (chunks of BC cells if B is large) and
 // gives each thread whole entries (i >= l) of the lower triangle; the upper
 // triangle is written as the conjugate mirror.

@@ -38,10 +38,12 @@ __host__ __device__ constexpr int bitrev(int x, int bits) {
   return r;
 }
 
-// a b, with the FMAs as the compiler contracts the plain product in the
-// 32-point transform: the split second pass then gives its bits (the
-// tensor-core covariance of the mixed precisions amplifies any other rounding
-// of the transform far above it)
+// a b, with its roundings written out: the definition of the products of the
+// split second pass (K = 512).  They are those that the plain product had in the
+// 32-point transform in registers that it replaced, contracted by the compiler;
+// other roundings would be as good, but the tensor-core covariance of the mixed
+// precisions amplifies any change of them far above the transform's own error.
+// The other lengths keep the plain product and the compiler's contraction.
 struct SplitMul {
   __device__ __forceinline__ float2 operator()(float2 a, float2 b) const {
     return make_float2(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x)));

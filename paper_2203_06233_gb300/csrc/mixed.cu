@@ -665,11 +665,11 @@ apply_tcx_kernel(const float2* __restrict__ dop, const float2* __restrict__ wts,
     // one 8-row group: lane l takes weight vector 4 rg + (l / 4) % 4 and word
     // l & 3 of both its rows, [wr, wi] (even) and [-wi, wr] (odd), from one
     // load and one split (pieces of -x are minus those of x).  Warp w takes
-    // units w, w + 8, ... (at most 128 / NW); the next chunk's loads are issued
+    // units w, w + NW, ... (at most 128 / NW); the next chunk's loads are issued
     // before this chunk's barrier and MMAs.
-    // With NCM = 4 the 64 A units are units 0-63: warp w's unit uu < 8 is
-    // row group (w >> 2) + 2 uu, core matrix w & 3.  Its B unit vb (unit
-    // 64 + w + 8 vb) is row group (w >> 1) + 4 vb, core matrices 2 (w & 1) + h.
+    // With NCM = 4 the 64 A units are units 0-63: warp w's unit uu < 64 / NW is
+    // row group (w >> 2) + NW / 4 uu, core matrix w & 3.  Its B unit vb (unit
+    // 64 + w + NW vb) is row group (w >> 1) + NW / 2 vb, core matrices 2 (w & 1) + h.
     // Row offsets, weight-vector offsets and scales are fixed per tile; the
     // snapshot entry and the weight element per chunk.
     static_assert(NCM == 4 && NW % 4 == 0, "unit layout");

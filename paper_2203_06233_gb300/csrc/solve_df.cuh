@@ -1,4 +1,4 @@
-// The double-float weight solve (solve_df.cu): parameters and launcher.
+// The double-float weight solve (solve_df_kernel.cuh): parameters and launchers.
 #pragma once
 
 #include <type_traits>

@@ -27,13 +27,17 @@
 // 3.6e-6 off instead of 2.9e-8), though it would be a third faster.
 //
 // Where it may stand in for FP64.  The weights are stored as complex64
-// (2^-25), and the solution's relative error is at most kappa(Rl) times the
-// arithmetic's.  For a covariance (R positive semidefinite) the load bounds
-// kappa <= D / lf + 1, so launch_solve takes these kernels when that bound is
-// at most kDfMaxKappa = 2^19 (the default load 1e-3 gives 1.28e5 at D = 128)
-// and the FP64 kernels for weaker loads, where nothing bounds kappa.  With
-// the refinement step the measured weights are as far from the 64-bit ones as
-// the FP64 kernels' (both are the complex64 rounding).
+// (2^-25), and the error of a right-hand side's solution is at most kappa(Rl)
+// times the arithmetic's.  For a covariance (R positive semidefinite) the load
+// bounds kappa <= D / lf + 1, so launch_solve takes these kernels when that bound
+// is at most kDfMaxKappa = 2^19 (the default load 1e-3 gives 1.28e5 at D = 128;
+// see solve_df_eligible for plans without refinement) and the FP64 kernels for
+// weaker loads, where nothing bounds kappa.  Two things are outside of that
+// argument and are looked at per system: a combination of basis solutions that
+// cancels (combine) and, in stap_solve_weights, a matrix that is no covariance
+// (kAnyMatrix).  The measured weights are then as far from the 64-bit ones as
+// their complex64 rounding, 2.5e-8 normwise, at the default and at the weakest
+// accepted load, for 0 to 80 dB of interference, along beams or not.
 //
 // Range.  Floats span 2^+-126 only, so each system is scaled by the even
 // power of two 2^-e that brings Rl's trace into [1, 4): the conversion from
@@ -139,9 +143,14 @@ __device__ __forceinline__ void cms(Cdf& x, float4 l, float4 y) {
 
 // A sum whose partial sums a bound M is known for runs from sig = 3 P, P the
 // power of two above M, instead of from zero: it stays in (2 P, 4 P), where
-// floats have one spacing, so that t - s and the rest a b - (t - s) are exact
-// and need no TwoSum: 6 instructions instead of 12 per real product.  The error
-// is about 2^-46 of M where it was about 2^-47 of the running sums.
+// floats have one spacing, 2^-22 P, so that t - s is exact and no TwoSum is
+// needed: 6 instructions instead of 12 per real product.  What rounds: the rest
+// a b - (t - s), at most half a spacing, to 24 bits of itself (2^-47 P), the two
+// cross terms on top of it likewise, and the sum e of the rests, which after n
+// terms may have grown to n half spacings.  That is below n (3 + n / 2) 2^-47 P,
+// and as the roundings are independent about 2^-46 M for the n in question --
+// of the bound M, where the TwoSum form is about 2^-47 of the running sums:
+// the grid is for sums whose bound is close.
 __device__ __forceinline__ void gmac(float& s, float& e, float ah, float al, float bh, float bl) {
   const float t = __fmaf_rn(ah, bh, s);
   float q = __fmaf_rn(ah, bh, __fsub_rn(s, t));
@@ -1124,7 +1133,9 @@ __device__ __forceinline__ void solve_df_body(const SolveDfParams& prm, long lon
 }
 
 constexpr int cta_threads(int team) { return team > 32 ? team : 128; }
-// CTAs per SM that the registers must allow (shared memory allows about as many)
+// CTAs per SM that the registers must allow (shared memory allows about as many;
+// five of 128 threads for teams within a warp: 96 registers instead of 80, 1 to 4%
+// for D <= 16)
 constexpr int min_ctas(int team, int mode) {
   return team == 512 ? 1 : (team == 256 ? 3 : (team == 128 ? 6 : (team == 64 ? 12 : (f32f(mode) ? 6 : 5))));
 }

@@ -32,7 +32,7 @@ struct Tune {
   int solve_ts = 0;    // D <= 32 solve: lanes per system (power of two, >= one per RHS)
   int solve_nw = 0;    // D <= 32 solve: warps per CTA, 1..4; D > 64 FP64 solve: 16 for 512-thread CTAs
   int solve_lr = 0;    // D > 32 solve: lanes per right-hand side, 8 (D <= 64), 16 or 32
-  int apply_kind = 0;  // apply: 1 FP32 register-resident, 2 FP32 general, 3 tensor cores
+  int apply_kind = 0;  // apply: 1 FP32 register-resident, 2 FP32 tiled, 3 tensor cores
   int slabs = 0;       // single-CPI run: range slabs pipelined on prioritised streams, 1..8
   int solve_kind = 0;  // D <= 32 solve: 1 register-resident (D = 8, 12, 16), 2 shared-memory
                        // teams, 3 one system per CTA (all FP64; 0: by the load, solve_df.cuh)
