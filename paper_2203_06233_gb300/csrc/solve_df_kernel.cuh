@@ -63,13 +63,15 @@
 // faster split at D > 96 (2048 systems of 128 rows: half a warp 10230 us, a warp
 // 9470; without grids 10820, 10890), half a warp below (96 rows: 4958, 5540).
 //
-// Measured (GB300; the FP64 kernels, double-float without grids, as it is), us:
-//   D = 128, 16384 systems, C 32 S 64    266533, 82470, 71420
-//   D =  64, 8192 systems,  C 16 S 32     15859,  5403,  5234
-//   D =  15, 3840 systems,  C 5  S 11       258,   117 (no grids)
-//   D =  12, 16384 systems, C 4  S 16       324,   160 (no grids)
-//   D =  12, 256 systems,   C 4  S 4      103.5,    21 (no grids)
-// What bounds it at D = 128: issue, 74% of the slots in use by four warps per
+// Measured (GB300; the FP64 kernels, double-float without grids, with them, as it
+// is: with the look at combinations that cancel and, being the step, the check
+// of any matrix and its second launch of 3.5 us), us:
+//   D = 128, 16384 systems, C 32 S 64    266533, 82470, 71420, 75020
+//   D =  64, 8192 systems,  C 16 S 32     15859,  5403,  5234,  5400
+//   D =  15, 3840 systems,  C 5  S 11       258,   117 (no grids), 126
+//   D =  12, 16384 systems, C 4  S 16       324,   160 (no grids), 163
+//   D =  12, 256 systems,   C 4  S 4      103.5,    21 (no grids),  23
+// What bounds it at D = 128: issue, 72% of the slots in use by four warps per
 // scheduler (shared memory holds one system per SM), the sums' own
 // instructions a third of all slots; masked lanes of the diagonal blocks,
 // renormalisations, the shuffles that broadcast a column's entry and the loads
