@@ -49,7 +49,7 @@ L2_FLUSH_BYTES = 256 << 20
 # CPI's entry is an eighth of it (8192 of its 65536 systems, same kernel and
 # launch shape) scaled by 8, the traffic being per system (its lower triangle
 # read, its weights written).
-SOLVE_TRAFFIC = {("efc685a29c93665b", "large"): 8 * (1148994560 + 519895040)}
+SOLVE_TRAFFIC = {("ac093e2ce0f594b2", "large"): 8 * (1147861760 + 516840192)}
 SOLVE_KERNEL = "solve_df_kernel (double-float LDL^H, solves, refinement on the FP32 pipe)"
 
 

@@ -66,10 +66,10 @@
 // Measured (GB300; the FP64 kernels, double-float without grids, with them, as it
 // is: with the look at combinations that cancel and, being the step, the check
 // of any matrix and its second launch of 3.5 us), us:
-//   D = 128, 16384 systems, C 32 S 64    266533, 82470, 71420, 75020
-//   D =  64, 8192 systems,  C 16 S 32     15859,  5403,  5234,  5400
-//   D =  15, 3840 systems,  C 5  S 11       258,   117 (no grids), 126
-//   D =  12, 16384 systems, C 4  S 16       324,   160 (no grids), 163
+//   D = 128, 16384 systems, C 32 S 64    266533, 82470, 71420, 74020
+//   D =  64, 8192 systems,  C 16 S 32     15859,  5403,  5234,  5410
+//   D =  15, 3840 systems,  C 5  S 11       258,   117 (no grids), 124
+//   D =  12, 16384 systems, C 4  S 16       324,   160 (no grids), 164
 //   D =  12, 256 systems,   C 4  S 4      103.5,    21 (no grids),  23
 // What bounds it at D = 128: issue, 72% of the slots in use by four warps per
 // scheduler (shared memory holds one system per SM), the sums' own
@@ -443,7 +443,7 @@ __device__ __forceinline__ void ldl_solve_f32(Cdf (&x)[RPL], const float2* L, co
 // [2][D] (in the chunk's place: the factorisation is over before the first
 // residual), the factor
 // [Dp] (column-major packed), the pivot reciprocals [D], the pivot flag and
-// whether a steering vector's combination cancels.
+// three words of bits for passes with a vector whose combination cancels.
 template <int LR, int RPL>
 __host__ __device__ constexpr bool square() { return LR * RPL <= 12; }
 
@@ -573,7 +573,7 @@ __device__ __forceinline__ void factor(const System y, int D) {
       while (l > i) l -= ++i;
     }
   }
-  if (tt == 0) okf[0] = 1, okf[1] = 0;
+  if (tt < 4) okf[tt] = tt == 0;
   team_sync<TEAM>();
 
   for (int j = 0; j < D; j += 2) {
@@ -946,15 +946,46 @@ __device__ __noinline__ void emit(const SolveDfParams& prm, int off, long long s
 // 6e-15 / lf of sum max |U_c| (spatial factors of magnitude 1) for D = 12 to 128, loads 1e-3 to 2.3e-5 and
 // one or two steps.  (Rank one along v_s, 60 dB and more: errors of 2.5e-7 at D =
 // 12 to 1.8e-5 at D = 128 for load 1e-3, up to 5e-4 for the weakest loads; a solve
-// of v_s itself is below the complex64 rounding.)  A system with a vector whose
-// ratio is 2^21 lf or more (SolveDfParams::cancel), i.e. half a complex64
-// rounding, is marked, and its vectors are solved by themselves.  A clutter
-// ridge does not get there (D = 12 to 128, 40 to 60 dB, load 1e-3: median 3 to 30,
-// largest 300).  (The refinement option keeps the combination.)
+// of v_s itself is below the complex64 rounding.)  A vector whose ratio is 2^21
+// lf or more (SolveDfParams::cancel), i.e. half a complex64 rounding, is solved
+// by itself, with the others of its pass.  A clutter ridge seldom gets there
+// (whole CPIs, 40 dB, load 1e-3: median ratio 3 to 30; 77 of 16384 systems of
+// 128 rows have such a vector, none of up to 64 rows).  (The refinement option
+// keeps the combination.)
 // Most vectors need no look at the sums: |U_c| <= |g| / delta and Re v^H u <= max
 // |u| sum |v|, so that a q of cancel_q / delta or more rules the ratio out (or, once
 // the sum over the basis is there, of steer_sum times that; a caller's matrix need
 // not keep the first bound).
+// The sum over the basis of max |U_c|.  (A call: inlined it costs the combination
+// its registers, for a look that few vectors need.)
+template <int LR>
+__device__ __noinline__ float sum_of_largest(const float4* U, int C, int D) {
+  const int li = (threadIdx.x & 31) % LR;
+  float sum = 0.f;
+  for (int c = 0; c < C; ++c) {
+    float m = 0.f;
+    for (int i = li; i < D; i += LR)
+      m = fmaxf(m, fmaxf(fabsf(U[(size_t)c * D + i].x), fabsf(U[(size_t)c * D + i].y)));
+    sum += lanes_max<LR>(m);
+  }
+  return sum;
+}
+
+// Which passes solve steering vectors by themselves, PASS or (the rows of U) C of
+// them at a time: all, or of 512 threads, whose passes are long, those with a
+// marked vector -- a bit each beside the pivot flag, the last one for all from
+// the 96th on (D = 120, 191 of 4096 systems marked: 10% of the solve's time, with
+// the bits 5%; for smaller systems the bits cost 1 to 2% and save little).
+template <int TEAM>
+__host__ __device__ constexpr bool pass_bits() { return TEAM == 512; }
+template <int LR, int TEAM>
+__device__ __forceinline__ int direct_step(int C) { return min(TEAM / LR, C); }
+template <int LR, int TEAM>
+__device__ __forceinline__ void mark(int* bits, int s, int C) {
+  const int b = pass_bits<TEAM>() ? min(s / direct_step<LR, TEAM>(C), 95) : 0;
+  atomicOr(bits + b / 32, 1 << (b & 31));
+}
+
 template <int LR, int RPL, int TEAM, int MODE>
 __device__ __noinline__ void combine(const SolveDfParams& prm, int off, long long sys, bool valid, bool ok, int e,
                                      float delta) {
@@ -1037,17 +1068,14 @@ __device__ __noinline__ void combine(const SolveDfParams& prm, int off, long lon
       m1 = lanes_max<LR>(m1);
       m2 = lanes_max<LR>(m2);
       if (least < 0.f) {                           // the system's sum of max |U_c|, once
-        least = 0.f;
-        for (int c = 0; c < C; ++c) {
-          float m = 0.f;
-          for (int i = li; i < D; i += LR)
-            m = fmaxf(m, fmaxf(fabsf(U[(size_t)c * D + i].x), fabsf(U[(size_t)c * D + i].y)));
-          least += lanes_max<LR>(m);
-        }
+        least = sum_of_largest<LR>(U, C, D);
         least *= prm.cancel;
         least_q = fminf(least_q, least * prm.steer_sum);
       }
-      if (ok && li == 0 && p0 + g < n1 && (!(m1 >= least) || (sym && !(m2 >= least)))) *cancels = 1;
+      if (ok && li == 0 && p0 + g < n1) {
+        if (!(m1 >= least)) mark<LR, TEAM>(cancels, s1, C);
+        if (sym && !(m2 >= least)) mark<LR, TEAM>(cancels, s2, C);
+      }
     }
     const bool good1 = ok && usable(d1), good2 = ok && usable(d2);
     const Gain f1 = gain(d1, -e / 2), f2 = gain(d2, -e / 2);
@@ -1100,13 +1128,17 @@ __device__ __forceinline__ void solve_df_body(const SolveDfParams& prm, long lon
     y.sbase = 896 + e;
     factor<TEAM, MODE, square<LR, RPL>()>(y, D);
     const bool ok = *okf != 0;
-    // the basis and its combinations, and all the vectors where one cancelled;
-    // or all the vectors
+    // the basis and its combinations, and the passes with a vector whose
+    // combination cancelled; or all the vectors
     bool direct = !sep;
     for (;;) {
       const int nrhs = direct ? prm.S : prm.C;
-      const int step = direct && sep ? min(PASS, prm.C) : PASS;   // the rows of U
+      const int step = direct && sep ? direct_step<LR, TEAM>(prm.C) : PASS;   // the rows of U
       for (int r0 = 0; r0 < nrhs; r0 += step) {
+        if constexpr (pass_bits<TEAM>() && !f32f(MODE)) {
+          const int b = min(r0 / step, 95);
+          if (direct && sep && (okf[1 + b / 32] >> (b & 31) & 1) == 0) continue;
+        }
         const int g = tt / LR, w0 = (tt >> 5) * (32 / LR);        // group in team, its warp's first
         Rhs z;
         z.direct = direct;
@@ -1116,13 +1148,15 @@ __device__ __forceinline__ void solve_df_body(const SolveDfParams& prm, long lon
         z.row = direct ? min(g, step - 1) : z.rhs;
         solve_rhs<LR, RPL, TEAM, MODE>(prm, y, z);
         if (direct)
-          emit<LR, RPL, TEAM>(prm, y.off, sys, valid && z.live && (!sep || okf[1] != 0), ok, e, z.rhs, z.row);
+          emit<LR, RPL, TEAM>(prm, y.off, sys, valid && z.live && (pass_bits<TEAM>() || !sep || okf[1] != 0), ok, e, z.rhs,
+                              z.row);
         team_sync<TEAM>();   // the next pass reuses U's rows, the combination reads them all
       }
       if (direct) break;
       combine<LR, RPL, TEAM, MODE>(prm, y.off, sys, valid, ok, e, split(y.delta, y.sbase).hi);
       team_sync<TEAM>();
-      if (f32f(MODE) || (TEAM > 32 ? okf[1] == 0 : !__any_sync(0xffffffffu, okf[1] != 0))) break;   // alike in a warp
+      if (f32f(MODE)) break;
+      if (!pass_bits<TEAM>() && (TEAM > 32 ? okf[1] == 0 : !__any_sync(0xffffffffu, okf[1] != 0))) break;   // alike in a warp
       direct = true;
     }
     if constexpr (MODE == kAnyMatrix) {            // (the pass and the combination ended with a barrier)
